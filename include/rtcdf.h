@@ -20,6 +20,7 @@
  *  - `in` and `out` must be 4-byte aligned; any further alignment is handled.
  *    `in == out` (in-place) is allowed because output generation never reads
  *    the input; any other overlap is rejected with RTCDF_ERR_INVALID_ARG.
+ *    A sort may use `out` as scratch before it writes the result.
  *  - Calls are asynchronous and ordered on `stream` (0 = legacy default
  *    stream).  Errors detectable on the host return immediately and enqueue
  *    nothing.  Errors found by the device (a key outside [minVal, maxVal), a

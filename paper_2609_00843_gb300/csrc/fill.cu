@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(WIN) fill_kernel(FillArgs a) {
     // Programmatic dependent of the scan: wait for its results.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     for (uint32_t i = c * WIN + tid; i < a.scan_chunks; i += a.fill_ctas * WIN) a.scan_state[i] = 0;
-    if (c == 0 && tid == 0) a.ctl->scan_ticket = 0;
+    if (c == 0 && tid == 0) a.ctl->scan_ticket = a.ctl->part_ticket = 0;
 
     // A wait that ran out (or a stray scan ticket) leaves the run table and the
     // start runs incomplete: write nothing (the output is unspecified then and

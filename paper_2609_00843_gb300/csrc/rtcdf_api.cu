@@ -59,6 +59,8 @@ struct Plan {
     int hist_threads;
     size_t hist_smem;
     bool streaming;
+    bool shape_given;   // the histogram's shape comes from the caller or the tuning table
+    int sms;
     uint32_t head;
     uint64_t nvec;
     int fill_threads;
@@ -87,6 +89,8 @@ rtcdf_status make_plan_with(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t
     if (p) q = *p;
 
     pl->R = R;
+    pl->sms = dev.sms;
+    pl->shape_given = q.tile_width > 0 || q.hist_ctas_per_tile > 0 || q.hist_threads > 0;
     pl->hist_threads = q.hist_threads ? q.hist_threads : 1024;
     if (pl->hist_threads != 256 && pl->hist_threads != 512 && pl->hist_threads != 1024)
         return RTCDF_ERR_INVALID_ARG;
@@ -238,6 +242,14 @@ rtcdf_status finish_phase(int32_t *out, uint64_t n, int64_t minVal, uint32_t R, 
     return RTCDF_OK;
 }
 
+// Histogram by partition (part.cu) or by range tiles (hist.cu).  Partition
+// takes about 9 us more (two launches) and reads the input once where the
+// tiles read it m times, so it needs several tiles and enough keys.
+bool use_part(const int32_t *in, const int32_t *out, uint64_t n, const Plan &pl, PartPlan *pp) {
+    if (in == out || pl.shape_given || pl.m <= 5 || n * (pl.m - 5) < 40000000u) return false;
+    return part_plan(n, pl.R, pl.head, pl.nvec, (uintptr_t)out, pl.sms, pp);
+}
+
 rtcdf_status run_pipeline(const int32_t *in, int32_t *out, uint64_t n, int64_t minVal,
                           uint32_t R, const Plan &pl, void *ws, size_t ws_bytes,
                           const rtcdf_debug *dbg, cudaStream_t s) {
@@ -247,7 +259,14 @@ rtcdf_status run_pipeline(const int32_t *in, int32_t *out, uint64_t n, int64_t m
     if (dbg)
         for (int i = 0; i < 4; i++) ev[i] = (cudaEvent_t)dbg->stage_events[i];
     if (ev[0] && cudaEventRecord(ev[0], s) != cudaSuccess) return RTCDF_ERR_CUDA;
-    rtcdf_status st = hist_phase(in, n, minVal, R, pl, L, base, s);
+    PartPlan pp;
+    rtcdf_status st;
+    if (use_part(in, out, n, pl, &pp)) {
+        st = launch_part(pp, in, n, pl.head, pl.nvec, (uint32_t)(int32_t)minVal, R, (uint32_t *)(base + L.hist),
+                         (Ctl *)(base + L.ctl), pl.sms, s) == cudaSuccess ? RTCDF_OK : RTCDF_ERR_CUDA;
+    } else {
+        st = hist_phase(in, n, minVal, R, pl, L, base, s);
+    }
     if (st) return st;
     if (ev[1] && cudaEventRecord(ev[1], s) != cudaSuccess) return RTCDF_ERR_CUDA;
     return finish_phase(out, n, minVal, R, pl, L, base, dbg, ev[2], ev[3], s, 0, n);

@@ -41,7 +41,8 @@ struct Ctl {
     uint32_t status;       // RTCDF_DEV_* bits, sticky until read
     uint32_t scan_ticket;  // dynamic chunk index of the lookback scan
     uint32_t num_runs;     // number of values with c_v > 0 (written by the scan)
-    uint32_t pad[61];
+    uint32_t part_ticket;  // items of bucket_kernel taken so far (zero between sorts)
+    uint32_t pad[60];
 };
 static_assert(sizeof(Ctl) == 256, "control block is 256 bytes");
 
@@ -105,6 +106,36 @@ struct HistArgs {
 cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool streaming,
                         cudaStream_t s);
 cudaError_t hist_max_ctas_per_sm(int threads, size_t smem, bool streaming, int *ctas);
+
+// ---------------------------------------------------------------- histogram by partition
+constexpr uint32_t kPartMaxBuckets = 512;
+
+struct PartArgs {
+    const int32_t *in;
+    uint64_t n, nvec;      // keys; 16-byte vectors after the unaligned head
+    uint32_t head, min_u, R;
+    uint32_t buckets;      // ranges of 2^15 values
+    uint32_t slabs, slab_keys;
+    uint32_t slab_units;   // 16-byte units between the slabs in `payload`
+    uint32_t part_ctas;    // CTAs of part_kernel
+    uint32_t tile_cost;    // of an item, in 16 keys, beside its keys
+    uint32_t target_items; // items bucket_kernel aims at
+    int4 *payload;         // per slab: its buckets' keys, 16 bits each
+    uint16_t *starts;      // per slab: buckets + 1 starts (units)
+    uint32_t *rows;        // per CTA of part_kernel: its keys of each bucket
+    uint32_t *H;           // global histogram, R entries (zero on entry)
+    Ctl *ctl;
+};
+struct PartPlan {
+    uint32_t buckets, slabs, slab_keys, slab_units, ctas;
+    size_t smem;
+    uintptr_t payload, starts, rows;  // in the scratch
+};
+// The plan for n keys over R values with the n words at out_addr as scratch;
+// false when they cannot hold it.
+bool part_plan(uint64_t n, uint32_t R, uint32_t head, uint64_t nvec, uintptr_t out_addr, int sms, PartPlan *p);
+cudaError_t launch_part(const PartPlan &p, const int32_t *in, uint64_t n, uint32_t head, uint64_t nvec, uint32_t min_u,
+                        uint32_t R, uint32_t *H, Ctl *ctl, int sms, cudaStream_t s);
 
 // ---------------------------------------------------------------- scan
 struct ScanArgs {

@@ -1,0 +1,86 @@
+"""Sorts of ranges wider than one shared-memory tile, at the sizes where the
+histogram's kernels change form: against the CPU oracle, element by element."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import assert_matches_oracle, dev_keys, gpu_sort, stream_handle
+from paper_2609_00843_gb300 import gen, rtcdf
+
+pytestmark = pytest.mark.gpu
+
+
+# Buckets of 2^15 values: one more than the widest of each counter layout (64,
+# 128 buckets), a last bucket of one value, the widest range; lengths with and
+# without keys before and after the whole vectors, and a last slab of few keys.
+@pytest.mark.parametrize("R,n,offset", [
+    (1 << 19, 8_000_001, 1), ((1 << 20) + 1, 3_100_000, 0), (64 << 15, 2_000_003, 3), ((64 << 15) + 1, 1_400_006, 2),
+    (128 << 15, 1_000_000, 0), ((128 << 15) + 5, 900_001, 1), ((1 << 24) - 1, 500_000, 2), (1 << 24, 16384 * 700 + 9, 0),
+])
+@pytest.mark.parametrize("dist", [gen.UNIFORM, gen.NORMAL, gen.ALL_EQUAL])
+def test_partitioned_histogram(R, n, offset, dist):
+    mn = -(1 << 31) if dist == gen.UNIFORM else 5 - R
+    x = torch.empty(n + offset, dtype=torch.int32, device="cuda")[offset:]
+    gen.keys_device(x.data_ptr(), n, mn, R, dist, gen.derive_seed(31, R, n), stream=stream_handle())
+    out = torch.full((n + 3,), 77, dtype=torch.int32, device="cuda")[3 - offset:3 - offset + n]
+    gpu_sort(x, mn, mn + R, out)
+    assert_matches_oracle(x, out, mn, mn + R)
+
+
+def test_partitioned_histogram_of_sorted_and_two_valued_keys():
+    n, R = 6_000_000, 1 << 20
+    x = dev_keys(n, 0, R, gen.UNIFORM, 5).sort().values
+    assert_matches_oracle(x, gpu_sort(x, 0, R), 0, R)
+    x = torch.where(torch.arange(n, device="cuda") % 3 == 0, R - 1, 0).int()
+    assert_matches_oracle(x, gpu_sort(x, 0, R), 0, R)
+
+
+def test_partitioned_histogram_in_place_and_in_a_graph():
+    n, R, mn = 5_000_000, 1 << 20, -9
+    x = dev_keys(n, mn, R, gen.NORMAL, 6)
+    want = gpu_sort(x, mn, mn + R)
+    assert_matches_oracle(x, want, mn, mn + R)
+    y = x.clone()
+    gpu_sort(y, mn, mn + R, y)  # no scratch: the range-tile histogram
+    assert torch.equal(y, want)
+    s = torch.cuda.Stream()
+    assert rtcdf.rtcdf_reserve(R, s.cuda_stream) == rtcdf.OK
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        assert rtcdf.rtcdf_sort(x.data_ptr(), y.data_ptr(), n, mn, mn + R, s.cuda_stream) == rtcdf.OK
+    for seed in (7, 8):
+        gen.keys_device(x.data_ptr(), n, mn, R, gen.UNIFORM, seed, stream=stream_handle())
+        g.replay()
+        torch.cuda.synchronize()
+        assert_matches_oracle(x, y, mn, mn + R)
+
+
+@pytest.mark.parametrize("key", [-1, 1_000_000, 1_000_000 + (1 << 15), np.iinfo(np.int32).max, np.iinfo(np.int32).min])
+def test_partitioned_histogram_reports_a_key_out_of_range(key):
+    n, R = 4_000_000, 1_000_000
+    x = dev_keys(n, 0, R, gen.UNIFORM, 9)
+    x[n // 2 + 1] = int(key)
+    out = torch.empty_like(x)
+    assert rtcdf.rtcdf_sort(x.data_ptr(), out.data_ptr(), n, 0, R, stream_handle()) == rtcdf.OK
+    rc, bits = rtcdf.rtcdf_status_get(stream_handle())
+    assert rc == rtcdf.ERR_KEY_OUT_OF_RANGE and bits == rtcdf.DEV_KEY_OUT_OF_RANGE
+    x[n // 2 + 1] = 3
+    gpu_sort(x, 0, R, out)
+    assert_matches_oracle(x, out, 0, R)
+
+
+def test_nothing_is_written_while_a_timeout_is_unread():
+    n, R = 4_000_000, 1 << 20
+    x = dev_keys(n, 0, R, gen.UNIFORM, 10)
+    out = torch.full_like(x, -7)
+    wsb = rtcdf.rtcdf_workspace_size(R)
+    ws = torch.zeros(wsb // 4, dtype=torch.int32, device="cuda")
+    ws[0] = rtcdf.DEV_TIMEOUT                    # control block word 0: the status
+    s = stream_handle()
+    assert rtcdf.rtcdf_sort_ws(x.data_ptr(), out.data_ptr(), n, 0, R, ws.data_ptr(), wsb, s) == rtcdf.OK
+    assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s)[0] == rtcdf.ERR_TIMEOUT
+    assert bool((out == -7).all())
+    assert rtcdf.rtcdf_sort_ws(x.data_ptr(), out.data_ptr(), n, 0, R, ws.data_ptr(), wsb, s) == rtcdf.OK
+    assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
+    assert_matches_oracle(x, out, 0, R)
