@@ -228,7 +228,7 @@ rtcdf_status finish_phase(int32_t *out, uint64_t n, int64_t minVal, uint32_t R, 
     sc.dbg_hist = dbg ? dbg->tile_hist : nullptr;
     sc.dbg_cdf = dbg ? dbg->cdf : nullptr;
     sc.dbg_offset = dbg ? dbg->tile_offset : nullptr;
-    if (launch_scan(sc, s) != cudaSuccess) return RTCDF_ERR_CUDA;
+    if (launch_scan(sc, pl.sms, s) != cudaSuccess) return RTCDF_ERR_CUDA;
     if (ev_scan && cudaEventRecord(ev_scan, s) != cudaSuccess) return RTCDF_ERR_CUDA;
 
     FillArgs f;

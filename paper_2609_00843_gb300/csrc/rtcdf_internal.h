@@ -152,10 +152,11 @@ struct ScanArgs {
     uint32_t pos_base;     // the output CTAs cover positions [pos_base, pos_end) of
     uint32_t pos_end;      // the sorted array (0 and n for a whole sort)
     uint32_t R, T, chunks;
+    uint32_t ctas;         // scan CTAs (set by launch_scan)
     int32_t minVal;
     uint32_t *dbg_hist, *dbg_cdf, *dbg_offset;  // optional exports
 };
-cudaError_t launch_scan(const ScanArgs &a, cudaStream_t s);
+cudaError_t launch_scan(const ScanArgs &a, int sms, cudaStream_t s);
 
 // ---------------------------------------------------------------- output
 struct FillArgs {

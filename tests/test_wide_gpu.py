@@ -70,6 +70,25 @@ def test_partitioned_histogram_reports_a_key_out_of_range(key):
     assert_matches_oracle(x, out, 0, R)
 
 
+# One scan CTA per 4096 values up to two per SM (304 on GB300), several chunks
+# each beyond: both sides of the step, a last chunk of one value.
+@pytest.mark.parametrize("R", [304 * 4096, 304 * 4096 + 1, 305 * 4096, 3 * 304 * 4096 + 17])
+@pytest.mark.parametrize("dist", [gen.UNIFORM, gen.ALL_EQUAL])
+def test_windows_over_a_wide_range(R, dist):
+    n, mn, s = 700_001, -3, stream_handle()
+    x = dev_keys(n, mn, R, dist, gen.derive_seed(33, R))
+    counts = torch.zeros(R, dtype=torch.int32, device="cuda")
+    assert rtcdf.rtcdf_hist_accumulate(x.data_ptr(), n, mn, mn + R, counts.data_ptr(), s) == rtcdf.OK
+    wsb = rtcdf.rtcdf_workspace_size(R)
+    ws = torch.zeros(wsb // 4, dtype=torch.int32, device="cuda")
+    out = torch.empty_like(x)
+    for lo, hi in ((0, 1), (1, 300_002), (300_002, n)):
+        assert rtcdf.rtcdf_fill_from_counts(counts.data_ptr(), n, mn, mn + R, lo, hi, out.data_ptr() + 4 * lo,
+                                            ws.data_ptr(), wsb, s) == rtcdf.OK
+    assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
+    assert_matches_oracle(x, out, mn, mn + R)
+
+
 def test_nothing_is_written_while_a_timeout_is_unread():
     n, R = 4_000_000, 1 << 20
     x = dev_keys(n, 0, R, gen.UNIFORM, 10)
