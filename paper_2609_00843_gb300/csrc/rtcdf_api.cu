@@ -191,18 +191,41 @@ rtcdf_status check_args(const int32_t *in, int32_t *out, uint64_t n) {
     return RTCDF_OK;
 }
 
-// Algorithm 5 (all tiles) into the workspace's H.  H accumulates, so several
-// calls over slices of one array add up to the array's histogram.
-rtcdf_status hist_phase(const int32_t *in, uint64_t n, int64_t minVal, uint32_t R, const Plan &pl,
-                        const WsLayout &L, char *base, cudaStream_t s) {
+// Histogram by packed counters (pack.cu) or by range tiles (hist.cu): one pass
+// over the input against one per tile, and about 10 us more (the sample and a
+// second launch; without scratch, the counters added to H by every CTA).
+bool use_pack(uint64_t n, const Plan &pl, uintptr_t scratch, PackPlan *pp) {
+    if (pl.shape_given || pl.R <= 49152 || n * pl.m < (scratch ? 70000000u : 120000000u)) return false;
+    return pack_plan(n, pl.R, pl.nvec, scratch, pl.sms, pp);
+}
+
+// Histogram by partition (part.cu) or by range tiles (hist.cu).  Partition
+// takes about 9 us more (two launches) and reads the input once where the
+// tiles read it m times, so it needs several tiles and enough keys.
+bool use_part(uint64_t n, const Plan &pl, uintptr_t scratch, PartPlan *pp) {
+    if (!scratch || pl.shape_given || pl.m <= 5 || n * (pl.m - 5) < 40000000u) return false;
+    return part_plan(n, pl.R, pl.head, pl.nvec, scratch, pl.sms, pp);
+}
+
+// Algorithm 5 (all tiles) into H (R counters).  H accumulates, so several calls
+// over slices of one array add up to the array's histogram.  ctl and scratch (n
+// words, 0 if there are none): of a whole sort.
+rtcdf_status hist_phase(const int32_t *in, uint64_t n, int64_t minVal, uint32_t R, const Plan &pl, uint32_t *H,
+                        Ctl *ctl, uintptr_t scratch, cudaStream_t s) {
     HistArgs h;
     h.in = in; h.n = n; h.nvec = pl.nvec; h.head = pl.head;
     h.min_u = (uint32_t)(int32_t)minVal; h.R = R; h.T = pl.T; h.m = pl.m; h.g = pl.g;
-    h.H = (uint32_t *)(base + L.hist);
-    h.ctl = (Ctl *)(base + L.ctl);
-    if (launch_hist(h, pl.hist_threads, pl.hist_smem, pl.streaming, s) != cudaSuccess)
-        return RTCDF_ERR_CUDA;
-    return RTCDF_OK;
+    h.H = H;
+    PackPlan pack;
+    PartPlan part;
+    cudaError_t e;
+    if (use_pack(n, pl, scratch, &pack))
+        e = launch_pack(pack, h, ctl && pack.dump ? &ctl->pack_copies : nullptr, s);
+    else if (ctl && use_part(n, pl, scratch, &part))
+        e = launch_part(part, in, n, pl.head, pl.nvec, h.min_u, R, H, ctl, pl.sms, s);
+    else
+        e = launch_hist(h, pl.hist_threads, pl.hist_smem, pl.streaming, s);
+    return e == cudaSuccess ? RTCDF_OK : RTCDF_ERR_CUDA;
 }
 
 // Local CDFs + offsets (Algorithm 6) and output generation (Algorithm 7)
@@ -242,14 +265,6 @@ rtcdf_status finish_phase(int32_t *out, uint64_t n, int64_t minVal, uint32_t R, 
     return RTCDF_OK;
 }
 
-// Histogram by partition (part.cu) or by range tiles (hist.cu).  Partition
-// takes about 9 us more (two launches) and reads the input once where the
-// tiles read it m times, so it needs several tiles and enough keys.
-bool use_part(const int32_t *in, const int32_t *out, uint64_t n, const Plan &pl, PartPlan *pp) {
-    if (in == out || pl.shape_given || pl.m <= 5 || n * (pl.m - 5) < 40000000u) return false;
-    return part_plan(n, pl.R, pl.head, pl.nvec, (uintptr_t)out, pl.sms, pp);
-}
-
 rtcdf_status run_pipeline(const int32_t *in, int32_t *out, uint64_t n, int64_t minVal,
                           uint32_t R, const Plan &pl, void *ws, size_t ws_bytes,
                           const rtcdf_debug *dbg, cudaStream_t s) {
@@ -259,14 +274,9 @@ rtcdf_status run_pipeline(const int32_t *in, int32_t *out, uint64_t n, int64_t m
     if (dbg)
         for (int i = 0; i < 4; i++) ev[i] = (cudaEvent_t)dbg->stage_events[i];
     if (ev[0] && cudaEventRecord(ev[0], s) != cudaSuccess) return RTCDF_ERR_CUDA;
-    PartPlan pp;
-    rtcdf_status st;
-    if (use_part(in, out, n, pl, &pp)) {
-        st = launch_part(pp, in, n, pl.head, pl.nvec, (uint32_t)(int32_t)minVal, R, (uint32_t *)(base + L.hist),
-                         (Ctl *)(base + L.ctl), pl.sms, s) == cudaSuccess ? RTCDF_OK : RTCDF_ERR_CUDA;
-    } else {
-        st = hist_phase(in, n, minVal, R, pl, L, base, s);
-    }
+    // (a sort in place has no scratch)
+    rtcdf_status st = hist_phase(in, n, minVal, R, pl, (uint32_t *)(base + L.hist), (Ctl *)(base + L.ctl),
+                                 in == out ? 0 : (uintptr_t)out, s);
     if (st) return st;
     if (ev[1] && cudaEventRecord(ev[1], s) != cudaSuccess) return RTCDF_ERR_CUDA;
     return finish_phase(out, n, minVal, R, pl, L, base, dbg, ev[2], ev[3], s, 0, n);
@@ -362,7 +372,7 @@ rtcdf_status host_pipeline_hist(const int32_t *in, uint64_t n, int64_t minVal, u
     Plan pl;
     rtcdf_status st = make_plan(n, R, (uintptr_t)in, 0, nullptr, &pl);
     if (st) return st;
-    return hist_phase(in, n, minVal, R, pl, ws_layout(R, ws_bytes), (char *)ws, s);
+    return hist_phase(in, n, minVal, R, pl, (uint32_t *)((char *)ws + ws_layout(R, ws_bytes).hist), nullptr, 0, s);
 }
 
 rtcdf_status host_pipeline_finish(int32_t *out, uint64_t n, int64_t minVal, uint32_t R, void *ws,
@@ -481,14 +491,7 @@ rtcdf_status rtcdf_hist_accumulate(const int32_t *in, uint64_t n, int64_t minVal
     st = make_plan(n, R, (uintptr_t)in, 0, nullptr, &pl);
     if (st) return st;
     // Algorithm 5 for every tile, added straight into the caller's counts.
-    HistArgs h;
-    h.in = in; h.n = n; h.nvec = pl.nvec; h.head = pl.head;
-    h.min_u = (uint32_t)(int32_t)minVal; h.R = R; h.T = pl.T; h.m = pl.m; h.g = pl.g;
-    h.H = counts;
-    h.ctl = nullptr;
-    if (launch_hist(h, pl.hist_threads, pl.hist_smem, pl.streaming, (cudaStream_t)stream) != cudaSuccess)
-        return RTCDF_ERR_CUDA;
-    return RTCDF_OK;
+    return hist_phase(in, n, minVal, R, pl, counts, nullptr, 0, (cudaStream_t)stream);
 }
 
 rtcdf_status rtcdf_fill_from_counts(const uint32_t *counts, uint64_t total_n, int64_t minVal,

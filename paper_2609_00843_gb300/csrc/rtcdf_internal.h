@@ -42,7 +42,8 @@ struct Ctl {
     uint32_t scan_ticket;  // dynamic chunk index of the lookback scan
     uint32_t num_runs;     // number of values with c_v > 0 (written by the scan)
     uint32_t part_ticket;  // items of bucket_kernel taken so far (zero between sorts)
-    uint32_t pad[60];
+    uint32_t pack_copies;  // written-out counters of pack_kernel (written before it is read)
+    uint32_t pad[59];
 };
 static_assert(sizeof(Ctl) == 256, "control block is 256 bytes");
 
@@ -100,12 +101,33 @@ struct HistArgs {
     uint32_t head;         // elements before the first 16-byte aligned address
     uint32_t min_u;        // (uint32_t)minVal
     uint32_t R, T, m, g;   // range size, tile width, tiles, CTAs per tile
-    uint32_t *H;           // global histogram, R entries (zero on entry)
-    Ctl *ctl;
+    uint32_t *H;           // global histogram, R entries (added to)
 };
 cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool streaming,
                         cudaStream_t s);
 cudaError_t hist_max_ctas_per_sm(int threads, size_t smem, bool streaming, int *ctas);
+
+// ---------------------------------------------------------------- packed histogram
+struct PackArgs {
+    HistArgs h;            // (T, m, g: the range tiles of inputs that packed counters cannot hold)
+    uint32_t words, fields, magic;
+    uint32_t coarse_shift; // the sample's stretches of the range
+    float limit;           // expected keys of the fullest field in a round
+    uint32_t max_rounds;
+    uint32_t *dump;        // written-out counters, or null: added to H by each CTA
+    uint32_t *copies;
+};
+struct PackPlan {
+    uint32_t words, fields, magic, max_rounds, ctas, tile, m, g;
+    float limit;
+    size_t smem;
+    uintptr_t dump;
+};
+// The plan for n keys over R values; scratch: n words, or 0.  False when the
+// range does not fit.
+bool pack_plan(uint64_t n, uint32_t R, uint64_t nvec, uintptr_t scratch, int sms, PackPlan *p);
+// copies: a word of the workspace, or null for no scratch.
+cudaError_t launch_pack(const PackPlan &p, const HistArgs &hist, uint32_t *copies, cudaStream_t s);
 
 // ---------------------------------------------------------------- histogram by partition
 constexpr uint32_t kPartMaxBuckets = 512;
