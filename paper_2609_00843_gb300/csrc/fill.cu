@@ -45,12 +45,63 @@ __device__ __forceinline__ int next_run_after(const uint32_t *s_end, int lo, int
     return first_run_after(s_end, lo, probe, p);
 }
 
-// Runs per shared-memory window: four per thread, so that a CTA whose
+// Short runs: a warp's vectors [wb, we) (positions from `frame` on, four a
+// vector), `kBlock` positions at a time.  The warp writes the key of every run
+// that begins in the block to its first position in `m` (kBlock words of shared
+// memory, `none` elsewhere: no key of the array), reads it back as vectors and
+// carries the last key before it into every position without one: a ballot
+// finds the lane that holds it.  The same rule as the searches (Algorithm 7),
+// at a cost that does not depend on the runs' lengths.
+constexpr int kBlock = 512;
+
+template <class Store>
+__device__ __forceinline__ void fill_short_runs(uint32_t *m, const uint32_t *s_end, const int32_t *s_val, int nw,
+                                                uint32_t frame, uint32_t wb, uint32_t we, int32_t none, Store store) {
+    const int lane = threadIdx.x & 31;
+    if (wb >= we) return;
+    int4 *m4 = reinterpret_cast<int4 *>(m);
+    int j = first_run_after(s_end, 0, nw - 1, frame + 4 * wb);  // the run of the block's first position
+    for (uint32_t w = wb; w < we; w += kBlock / 4) {
+        const uint32_t q0 = frame + 4 * w, q1 = min(q0 + kBlock, frame + 4 * we);
+#pragma unroll
+        for (int k = 0; k < kBlock / 128; k++) m4[lane + 32 * k] = make_int4(none, none, none, none);
+        int32_t carry = s_val[j];
+        __syncwarp();
+        for (int r = j + 1 + lane;; r += 32) {
+            const uint32_t start = r < nw ? s_end[r - 1] : 0xffffffffu;
+            const bool begins = start < q1;
+            if (begins) m[start - q0] = (uint32_t)s_val[r];
+            const unsigned b = __ballot_sync(0xffffffffu, begins);
+            j += __popc(b);
+            if (b != 0xffffffffu) break;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < kBlock / 128; k++) {
+            int4 x = m4[lane + 32 * k];
+            const int32_t last = x.w != none ? x.w : x.z != none ? x.z : x.y != none ? x.y : x.x;
+            const unsigned has = __ballot_sync(0xffffffffu, last != none);
+            const unsigned before = has & ((1u << lane) - 1u);
+            const int32_t from = __shfl_sync(0xffffffffu, last, before ? 31 - __clz(before) : 0);
+            const int32_t next = __shfl_sync(0xffffffffu, last, has ? 31 - __clz(has) : 0);
+            if (x.x == none) x.x = before ? from : carry;
+            if (x.y == none) x.y = x.x;
+            if (x.z == none) x.z = x.y;
+            if (x.w == none) x.w = x.z;
+            if (has) carry = next;
+            const uint32_t v = w + lane + 32 * k;
+            if (v < we) store(v, x);
+        }
+        __syncwarp();  // the block has been read
+    }
+}
+
+// Runs per shared-memory window: four per thread (eight for short runs), so that a CTA whose
 // positions cross thousands of short runs (the tails of a peaked distribution
 // over a wide range) needs few window rounds -- each round costs a global
 // round trip and two barriers.
-template <int WIN>
-constexpr int kRunWindow = 4 * WIN;
+template <int WIN, bool SHORT>
+constexpr int kRunWindow = SHORT && WIN < 1024 ? 8 * WIN : 4 * WIN;
 
 // CTAs issued first that take the LAST output chunks.  With a peaked shape
 // the chunks at both ends of the output cross by far the most runs (the
@@ -58,11 +109,18 @@ constexpr int kRunWindow = 4 * WIN;
 // first anyway, and the last ones, issued last, would end the launch.
 constexpr uint32_t kTailChunksFirst = 32;
 
-template <int WIN>
+// SHORT (arrays of few keys per value): windows whose runs average less than
+// kShortRun positions are filled from the runs' first positions.
+constexpr uint32_t kShortRun = 256;
+
+template <int WIN, bool SHORT>
 __global__ void __launch_bounds__(WIN) fill_kernel(FillArgs a) {
-    constexpr int RW = kRunWindow<WIN>;
-    __shared__ uint32_t s_end[RW];
-    __shared__ int32_t s_val[RW];
+    constexpr int RW = kRunWindow<WIN, SHORT>;
+    extern __shared__ __align__(16) uint32_t s_fill[];  // SHORT: run ends, run keys, a block per warp
+    __shared__ uint32_t s_end_static[SHORT ? 1 : RW];
+    __shared__ int32_t s_val_static[SHORT ? 1 : RW];
+    uint32_t *s_end = SHORT ? s_fill : s_end_static;
+    int32_t *s_val = SHORT ? reinterpret_cast<int32_t *>(s_fill + RW) : s_val_static;
     const int tid = threadIdx.x;
     const uint32_t K = min(kTailChunksFirst, a.fill_ctas);
     const uint32_t c = blockIdx.x < K ? a.fill_ctas - K + blockIdx.x : blockIdx.x - K;  // output chunk
@@ -120,6 +178,12 @@ __global__ void __launch_bounds__(WIN) fill_kernel(FillArgs a) {
                 __stcs(vout + w + 3 * WIN, vv);
             }
             for (; w < w_hi; w += WIN) __stcs(vout + w, vv);
+        } else if (SHORT && (hi - pos) / (uint32_t)nw < kShortRun) {
+            const uint32_t warp = tid >> 5, nvec = w_hi > w_lo ? w_hi - w_lo : 0u;
+            const uint32_t per_warp = ((nvec + (WIN / 32) - 1) / (WIN / 32) + 31) & ~31u;
+            const uint32_t wb = w_lo + warp * per_warp;
+            fill_short_runs(s_fill + 2 * RW + warp * kBlock, s_end, s_val, nw, hb, wb, min(w_hi, wb + per_warp), a.none,
+                            [&](uint32_t v, int4 x) { __stcs(vout + v, x); });
         } else {
             // Each warp takes a contiguous share of the vectors and its lanes
             // interleave inside it: every store instruction still covers 512
@@ -184,26 +248,32 @@ __global__ void __launch_bounds__(WIN) fill_kernel(FillArgs a) {
     }
 }
 
-template <int WIN>
+template <int WIN, bool SHORT>
 cudaError_t launch_fill_t(const FillArgs &a, cudaStream_t s) {
+    constexpr size_t smem = SHORT ? 4 * (size_t)(2 * kRunWindow<WIN, true> + WIN / 32 * kBlock) : 0;
+    if (smem > 48 * 1024) {
+        cudaError_t e =
+            cudaFuncSetAttribute(fill_kernel<WIN, SHORT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.fill_ctas);
     cfg.blockDim = dim3(WIN);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, fill_kernel<WIN>, a);
+    return cudaLaunchKernelEx(&cfg, fill_kernel<WIN, SHORT>, a);
 }
 
-cudaError_t launch_fill(const FillArgs &a, int threads, cudaStream_t s) {
+cudaError_t launch_fill(const FillArgs &a, int threads, bool short_runs, cudaStream_t s) {
     switch (threads) {
-        case 256: return launch_fill_t<256>(a, s);
-        case 512: return launch_fill_t<512>(a, s);
-        case 1024: return launch_fill_t<1024>(a, s);
+        case 256: return short_runs ? launch_fill_t<256, true>(a, s) : launch_fill_t<256, false>(a, s);
+        case 512: return short_runs ? launch_fill_t<512, true>(a, s) : launch_fill_t<512, false>(a, s);
+        case 1024: return short_runs ? launch_fill_t<1024, true>(a, s) : launch_fill_t<1024, false>(a, s);
         default: return cudaErrorInvalidValue;
     }
 }

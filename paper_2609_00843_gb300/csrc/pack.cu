@@ -358,7 +358,7 @@ bool pack_plan(uint64_t n, uint32_t R, uint64_t nvec, uintptr_t scratch, int sms
     p->words = W;
     // Expected keys of the fullest field that overflow with a chance below 1e-7
     // (Poisson tails).
-    p->limit = fields == 2 ? 30000.f : fields == 4 ? 140.f : fields == 5 ? 24.f : fields == 6 ? 9.5f : 2.5f;
+    p->limit = fields == 2 ? 30000.f : fields == 4 ? 140.f : fields == 5 ? 24.f : fields == 6 ? 10.f : 2.5f;
     p->ctas = (uint32_t)std::min<uint64_t>(sms, std::max<uint64_t>(1, nvec / (4 * kPackThreads)));
     // Range tiles: as few as 45056 values allow, and the trash word.
     p->m = (R + 45055) / 45056;

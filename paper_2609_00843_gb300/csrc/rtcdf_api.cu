@@ -77,6 +77,10 @@ rtcdf_status check_range(int64_t minVal, int64_t maxVal, uint32_t *R) {
     return RTCDF_OK;
 }
 
+// Few keys per value: the output kernel's form for short runs.  (R = 2^19, n =
+// 1e8, 190 keys per value: 65.5 against 71.7 us; 381 keys: 73.7 against 63.5.)
+bool short_runs(uint64_t n, uint32_t R) { return n < 256ull * R; }
+
 // Choose the launch shape (Section 3.3): tile width T from shared memory, CTAs
 // per tile from occupancy, output CTAs from n.
 rtcdf_status make_plan_with(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t out_addr,
@@ -138,12 +142,18 @@ rtcdf_status make_plan_with(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t
     // Not clamped to n: positions below head_out are written one by one, and
     // the vector frame must stay 16-byte aligned.
     const uint32_t head_out = (uint32_t)(((16 - (out_addr & 15)) & 15) / 4);
-    pl->fill_threads = q.fill_threads ? q.fill_threads : 512;
+    const bool short_fill = short_runs(n, R) && !q.fill_threads && !q.fill_ctas && !q.fill_chunk;
+    pl->fill_threads = q.fill_threads ? q.fill_threads : short_fill && n >= 2000000 ? 256 : 512;
     if (pl->fill_threads != 256 && pl->fill_threads != 512 && pl->fill_threads != 1024)
         return RTCDF_ERR_INVALID_ARG;
     // Many more CTAs than fit at once (about 32K positions each, at least four
     // waves' worth): the block scheduler then balances CTAs whose positions
-    // cross many short runs against CTAs inside one long run.
+    // cross many short runs against CTAs inside one long run.  Where all runs
+    // are short (few keys per value) small CTAs with 4096 positions, or as few
+    // as kMaxFillCtas allows, are best (R = 2^20 normal, output kernel, us, for
+    // 256 threads with 4K / 8K / 16K / 32K positions and 512 threads with 4K /
+    // 16K: n = 1e7 16 / 23 / 35 / 55 and 27 / 23; 3e6 14 / 21 / 35 / 55 and 12 / 21;
+    // 1e6 12 / 21 / 35 / 57 and 10 / 23).
     uint64_t body = n > head_out ? n - head_out : 0;
     uint64_t chunk;
     if (q.fill_chunk < 0 || q.fill_ctas < 0) return RTCDF_ERR_INVALID_ARG;
@@ -151,6 +161,8 @@ rtcdf_status make_plan_with(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t
         chunk = std::max<uint64_t>((uint64_t)q.fill_chunk,
                                    (body + kMaxFillCtas - 1) / kMaxFillCtas);
         chunk = std::max<uint64_t>(chunk, 4 * (uint64_t)pl->fill_threads);
+    } else if (short_fill) {
+        chunk = std::max<uint64_t>(4096, (body + kMaxFillCtas - 1) / kMaxFillCtas);
     } else {
         uint64_t want = q.fill_ctas > 0 ? (uint64_t)q.fill_ctas
                                         : std::max<uint64_t>((uint64_t)dev.sms * 4, body / 32768);
@@ -172,7 +184,11 @@ rtcdf_status make_plan(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t out_
                        const rtcdf_params *p, Plan *pl) {
     if (p) return make_plan_with(n, R, in_addr, out_addr, p, pl);
     rtcdf_params t;
-    if (tune_lookup(n, R, &t) && make_plan_with(n, R, in_addr, out_addr, &t, pl) == RTCDF_OK)
+    bool builtin = false;
+    const bool found = tune_lookup(n, R, &t, &builtin);
+    // (the compiled-in table's output shapes are those of the kernel's form for long runs)
+    if (found && builtin && short_runs(n, R)) t.fill_ctas = t.fill_threads = t.fill_chunk = 0;
+    if (found && make_plan_with(n, R, in_addr, out_addr, &t, pl) == RTCDF_OK)
         return RTCDF_OK;
     return make_plan_with(n, R, in_addr, out_addr, nullptr, pl);
 }
@@ -259,8 +275,8 @@ rtcdf_status finish_phase(int32_t *out, uint64_t n, int64_t minVal, uint32_t R, 
     f.head = head_out;
     f.fill_ctas = pl.fill_ctas; f.run_end = run_end; f.run_val = run_val;
     f.start_run = start_run; f.ctl = ctl; f.scan_state = state; f.scan_chunks = L.scan_chunks;
-    f.R = R;
-    if (launch_fill(f, pl.fill_threads, s) != cudaSuccess) return RTCDF_ERR_CUDA;
+    f.R = R; f.none = (int32_t)((uint32_t)minVal - 1u);
+    if (launch_fill(f, pl.fill_threads, short_runs(n, R), s) != cudaSuccess) return RTCDF_ERR_CUDA;
     if (ev_fill && cudaEventRecord(ev_fill, s) != cudaSuccess) return RTCDF_ERR_CUDA;
     return RTCDF_OK;
 }

@@ -11,8 +11,8 @@
 namespace rtcdf {
 
 // Launch parameters of the tuning table for (n, R), if it has an entry
-// (tune.cu).
-bool tune_lookup(uint64_t n, uint32_t R, rtcdf_params *out);
+// (tune.cu); whether the table is the compiled-in one.
+bool tune_lookup(uint64_t n, uint32_t R, rtcdf_params *out, bool *builtin);
 
 // Device status bits (mirror RTCDF_DEV_* in rtcdf.h).
 constexpr uint32_t kDevKeyOutOfRange = 0x1;
@@ -195,7 +195,8 @@ struct FillArgs {
     uint64_t *scan_state;  // reset here for the next call
     uint32_t scan_chunks;
     uint32_t R;            // entries of run_end / run_val
+    int32_t none;          // a value no key of the array has (minVal - 1)
 };
-cudaError_t launch_fill(const FillArgs &a, int threads, cudaStream_t s);
+cudaError_t launch_fill(const FillArgs &a, int threads, bool short_runs, cudaStream_t s);
 
 }  // namespace rtcdf

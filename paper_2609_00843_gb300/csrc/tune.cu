@@ -22,12 +22,13 @@ const rtcdf_tune_entry kBuiltin[] = {
 std::mutex g_tune_mu;
 std::vector<rtcdf_tune_entry> g_table;
 bool g_loaded = false;
+bool g_builtin = false;  // the table is the compiled-in one
 
 void load_builtin_locked() {
     g_table.clear();
     for (const rtcdf_tune_entry &e : kBuiltin)
         if (e.log2_R >= 0) g_table.push_back(e);
-    g_loaded = true;
+    g_loaded = g_builtin = true;
 }
 
 int32_t log2_ceil(uint32_t R) {
@@ -40,7 +41,7 @@ int32_t log2_ceil(uint32_t R) {
 
 namespace rtcdf {
 
-bool tune_lookup(uint64_t n, uint32_t R, rtcdf_params *out) {
+bool tune_lookup(uint64_t n, uint32_t R, rtcdf_params *out, bool *builtin) {
     const int32_t lr = log2_ceil(R), nc = rtcdf_tune_n_class(n);
     std::lock_guard<std::mutex> lk(g_tune_mu);
     if (!g_loaded) {
@@ -55,6 +56,7 @@ bool tune_lookup(uint64_t n, uint32_t R, rtcdf_params *out) {
     for (auto it = g_table.rbegin(); it != g_table.rend(); ++it) {
         if (it->log2_R == lr && it->n_class == nc) {
             *out = it->params;
+            *builtin = g_builtin;
             return true;
         }
     }
@@ -84,6 +86,7 @@ rtcdf_status rtcdf_tune_set(const rtcdf_tune_entry *entries, int32_t count) try 
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_table.assign(entries, entries + count);
     g_loaded = true;
+    g_builtin = false;
     return RTCDF_OK;
 } catch (...) {  // an allocation failed (std::bad_alloc and the like)
     return RTCDF_ERR_NO_MEMORY;

@@ -103,3 +103,18 @@ def test_nothing_is_written_while_a_timeout_is_unread():
     assert rtcdf.rtcdf_sort_ws(x.data_ptr(), out.data_ptr(), n, 0, R, ws.data_ptr(), wsb, s) == rtcdf.OK
     assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
     assert_matches_oracle(x, out, 0, R)
+
+
+# Output of short runs: few keys per value, up to the step at 256, values present
+# now and then, and outputs at every alignment.
+@pytest.mark.parametrize("R,n", [(4096, 4096 * 256 - 1), (4096, 4096 * 256), (5000, 20_011), (50_000, 3), (300_000, 1_000_003),
+                                 (1 << 22, 100_000), (1 << 22, 6_000_001)])
+@pytest.mark.parametrize("dist", [gen.UNIFORM, gen.NORMAL])
+@pytest.mark.parametrize("offset", [0, 1, 2, 3])
+def test_short_runs(R, n, dist, offset):
+    mn = -(1 << 31)                # the value that marks no run wraps around
+    x = dev_keys(n, mn, R, dist, gen.derive_seed(35, R, n))
+    out = torch.full((n + 8,), 5, dtype=torch.int32, device="cuda")
+    gpu_sort(x, mn, mn + R, out[offset:offset + n])
+    assert_matches_oracle(x, out[offset:offset + n], mn, mn + R)
+    assert bool((out[:offset] == 5).all()) and bool((out[offset + n:] == 5).all())
