@@ -254,6 +254,17 @@ __host__ __device__ inline uint32_t devplan_hist_class(uint64_t keys, uint64_t h
     return keys >= hist_chunk / 2 ? 0u : keys >= hist_chunk / 4 ? 1u : 2u;
 }
 
+// Whether an in-CTA sort of the scan launch (256 threads: about 5 us + 1.05 ns
+// per key + 1.9 ns per value) would outlast the rest of that launch, which the
+// output launch waits for: the segment is split into work items instead.  The
+// device planner knows only the number of segments when it classifies one; the
+// launch takes about 42 ns for each (six CTAs per SM, measured on the benchmark's
+// shapes), and 20 us at least.
+__host__ __device__ inline bool devplan_outlasts(uint32_t n, uint32_t R, uint32_t S) {
+    const uint64_t launch_ns = 42ull * S > 20000 ? 42ull * S : 20000;
+    return 5000 + 21ull * n / 20 + 19ull * R / 10 > launch_ns;
+}
+
 // Segment s from its metadata: its descriptor (workspace offsets left to the
 // caller) and its items per list, as build_host_plan classifies it; false
 // when it breaks the bounds or the limits of a segmented sort.
@@ -270,7 +281,8 @@ __host__ __device__ inline bool devplan_segment(int64_t o0, int64_t o1, int64_t 
     g->R = (uint32_t)(mx - mn);
     g->minVal = (int32_t)mn;
     if (n == 0) return true;
-    if (g->n <= t.small_max_n && g->R <= kBatchSmallMaxR) {
+    if (g->n <= t.small_max_n && g->R <= kBatchSmallMaxR &&
+        !(t.small_by_time && g->R <= t.small_scan_max_R && devplan_outlasts(g->n, g->R, b.S))) {
         if (g->R <= t.small_scan_max_R) c->v[kListSmall2] = 1;
         else c->v[kListSmall1] = 1;
         return true;
