@@ -17,8 +17,9 @@
 //                  segment's H: local CDF + offsets (Algorithm 6) by a
 //                  decoupled lookback chained within the segment, the run
 //                  table and the first run of each output item;
-//   output launch  one CTA per output item: positions from the run table
-//                  (Algorithm 7's rule), as in the single-array output kernel.
+//   output launch  two or more CTAs per output item: positions from the run
+//                  table (Algorithm 7's rule), as in the single-array output
+//                  kernels.
 //
 // The second and third launches are programmatic dependents of the one before
 // (their launch latency overlaps its tail).  Every phase runs at full
@@ -29,6 +30,7 @@
 // reads it, so a plan can be replayed (e.g. from a CUDA graph) with no host
 // work.
 #include "batched.h"
+#include "fill_runs.cuh"
 
 namespace rtcdf {
 
@@ -350,35 +352,13 @@ __device__ void do_hist(const BatchArgs &a, const BatchSeg &g, const BatchItem &
 }
 
 __device__ __forceinline__ void prof_item(const BatchArgs &a, uint32_t kind, unsigned long long t0,
-                                          unsigned long long wait) {
+                                          unsigned long long wait, bool counts = true) {
     const unsigned long long t1 = global_ns();
     atomicAdd(a.prof + kind, t1 - t0);
-    atomicAdd(a.prof + 4 + kind, 1ull);
+    if (counts) atomicAdd(a.prof + 4 + kind, 1ull);
     atomicMin(a.prof + 8 + kind, t0);
     atomicMax(a.prof + 12 + kind, t1);
     if (wait) atomicAdd(a.prof + 16 + kind, wait);
-}
-
-// Smallest j in [lo, hi] with e[j] > p, given e[hi] > p.
-__device__ __forceinline__ uint32_t first_after(const uint32_t *e, uint32_t lo, uint32_t hi, uint32_t p) {
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (e[mid] > p) hi = mid; else lo = mid + 1;
-    }
-    return lo;
-}
-
-// The same when the answer is expected close to lo: probes lo, lo + 1,
-// lo + 3, lo + 7, ... until e exceeds p, then a binary search inside the last
-// step -- O(log(j - lo)) reads.
-__device__ __forceinline__ uint32_t next_after(const uint32_t *e, uint32_t lo, uint32_t hi, uint32_t p) {
-    uint32_t probe = lo, step = 1;
-    while (e[probe] <= p) {  // e[hi] > p ends it
-        lo = probe + 1;
-        probe = min(hi, probe + step);
-        step <<= 1;
-    }
-    return first_after(e, lo, probe, p);
 }
 
 }  // namespace
@@ -683,16 +663,40 @@ __global__ void __launch_bounds__(kScanCtaThreads, 6) seg_scan_kernel(BatchArgs 
     scan_chunk(a, it, g, s_warp, s_prefix, s_total, s_wait, s_buf, t0);
 }
 
-// Output CTAs of 512 threads: four resident per SM, so that one CTA's
-// descriptor loads and window round trip overlap the others' stores.
-constexpr int kFillCtaThreads = 512;
+// Output CTAs of 256 threads, six resident per SM (42 registers a thread), so
+// that one CTA's descriptor loads and window round trip overlap the others'
+// stores.
+constexpr int kFillCtaThreads = 256;
+constexpr uint32_t kFillWarps = kFillCtaThreads / 32;
 
-// One output item: positions [it.a, it.b) of its segment from the run table
-// (Algorithm 7's rule).
-__device__ __forceinline__ void fill_item(const BatchArgs &a, const BatchItem &it, const BatchSeg &g, uint32_t *s_end,
-                                          int32_t *s_val, unsigned long long t0) {
-    const uint32_t tid = threadIdx.x, nt = blockDim.x;
-    if (it.aux == 0 && g.scan_chunks > 1) {
+// Windows whose runs average fewer positions are filled from the runs' starts.
+// 4096 segments 904 us against 942 with the searches alone, 1024 243 against 259
+// (260 with 512-thread CTAs, one an item); 64 segments (115 items) 62 against 105
+// us, from the items' parts.
+constexpr uint32_t kSegShortRun = 256;
+
+// First run of [lo, hi] whose end exceeds p (run_end[hi] does), 32 probes at a
+// time; every warp for itself.
+__device__ __forceinline__ uint32_t first_run_global(const uint32_t *run_end, uint32_t lo, uint32_t hi, uint32_t p) {
+    const uint32_t lane = threadIdx.x & 31;
+    while (lo < hi) {
+        const uint32_t step = (hi - lo) / 32 + 1, at = min(hi, lo + step * (lane + 1) - 1);
+        const unsigned above = __ballot_sync(0xffffffffu, run_end[at] > p);  // lane 31 probes hi or beyond
+        const uint32_t f = above ? (uint32_t)__ffs(above) - 1 : 31u;
+        hi = min(hi, lo + step * (f + 1) - 1);
+        lo = min(hi, lo + step * f);
+    }
+    return lo;
+}
+
+// Part `part` of `parts` of one output item: the item's positions [it.a, it.b) of
+// its segment from the run table (Algorithm 7's rule).  s_m: a block of words per
+// warp.
+__device__ __forceinline__ void fill_item(const BatchArgs &a, const BatchItem &it, const BatchSeg &g, uint32_t part,
+                                          uint32_t parts, uint32_t *s_end, int32_t *s_val, uint32_t *s_m,
+                                          unsigned long long t0) {
+    const uint32_t tid = threadIdx.x, nt = kFillCtaThreads;
+    if (part == 0 && it.aux == 0 && g.scan_chunks > 1) {
         // The segment's first output item leaves its lookback state zeroed.
         uint64_t *state = reinterpret_cast<uint64_t *>(a.ws_u32 + g.state_off);
         for (uint32_t i = tid; i < g.scan_chunks; i += nt) state[i] = 0;
@@ -707,17 +711,22 @@ __device__ __forceinline__ void fill_item(const BatchArgs &a, const BatchItem &i
     const uint32_t *run_end = a.ws_u32 + g.run_end_off;
     const int32_t *run_val = reinterpret_cast<const int32_t *>(a.ws_u32 + g.run_val_off);
     const uint32_t *start_run = a.ws_u32 + g.start_run_off;
+    const uint32_t len = (uint32_t)(it.b - it.a), per = ((len + parts - 1) / parts + 127) & ~127u;
+    if (part * per >= len) return;
+    uint32_t pos = (uint32_t)it.a + part * per;
+    const uint32_t P1 = min((uint32_t)it.b, pos + per);
     uint32_t k_cur = min(start_run[it.aux], D - 1);
     // Last run this item can need: the one holding the next item's first position.
     const uint32_t k_last = (it.aux + 1 < g.fill_items) ? min(start_run[it.aux + 1], D - 1) : D - 1;
+    if (part) k_cur = first_run_global(run_end, k_cur, max(k_cur, k_last), pos);
     int32_t *out = a.out + g.out_off;
     // Positions relative to the segment; vectors aligned to the global `out`.
     const uint32_t head = (uint32_t)(((16 - ((uintptr_t)out & 15)) & 15) / 4);
     int4 *vout = reinterpret_cast<int4 *>(out + head);
-    uint32_t pos = (uint32_t)it.a;
-    const uint32_t P1 = (uint32_t)it.b;
+    const uint32_t lane = tid & 31, warp = tid >> 5;
     while (pos < P1 && k_cur < D) {
-        const uint32_t nw = min((uint32_t)kSegFillRuns, (k_last >= k_cur ? k_last - k_cur : 0u) + 1u);
+        // (every run holds at least one position)
+        const uint32_t nw = min(min(kSegFillRuns, P1 - pos), (k_last >= k_cur ? k_last - k_cur : 0u) + 1u);
         __syncthreads();
         for (uint32_t i = tid; i < nw; i += nt) {
             s_end[i] = run_end[k_cur + i];
@@ -727,26 +736,28 @@ __device__ __forceinline__ void fill_item(const BatchArgs &a, const BatchItem &i
         const uint32_t hi = min(P1, s_end[nw - 1]);
         const uint32_t w_lo = pos >= head ? (pos - head + 3) >> 2 : 0u;
         const uint32_t w_hi = hi >= head ? (hi - head) >> 2 : 0u;
+        const uint32_t nvec = w_hi > w_lo ? w_hi - w_lo : 0u;
+        const uint32_t per_warp = ((nvec + kFillWarps - 1) / kFillWarps + 31) & ~31u;
+        const uint32_t wb = w_lo + warp * per_warp;
+        const uint32_t we = min(w_hi, wb + per_warp);
         if (s_end[0] >= hi) {
             // One run covers the whole round: constant stores.
             const int32_t v = s_val[0];
             const int4 vv = make_int4(v, v, v, v);
             for (uint32_t w = w_lo + tid; w < w_hi; w += nt) __stcs(vout + w, vv);
+        } else if ((hi - pos) / nw < kSegShortRun) {
+            fill_short_runs(s_m + warp * kBlock, s_end, s_val, (int)nw, head, wb, we,
+                            (int32_t)((uint32_t)g.minVal - 1u), [&](uint32_t v, int4 x) { __stcs(vout + v, x); });
         } else {
-            const uint32_t lane = tid & 31, warp = tid >> 5, nwarps = nt >> 5;
-            const uint32_t nvec = w_hi > w_lo ? w_hi - w_lo : 0u;
-            const uint32_t per_warp = ((nvec + nwarps - 1) / nwarps + 31) & ~31u;
-            const uint32_t wb = w_lo + warp * per_warp;
-            const uint32_t we = min(w_hi, wb + per_warp);
             // The run of this lane's last vector, its end and value in
             // registers (no shared-memory read inside the same run).
-            uint32_t j = 0;
+            int j = 0;
             uint32_t ej = s_end[0];
             int32_t vj = s_val[0];
             for (uint32_t w = wb + lane; w < we; w += 32) {
                 const uint32_t q = head + 4 * w;
                 if (ej <= q) {
-                    j = next_after(s_end, j + 1, nw - 1, q);
+                    j = next_run_after(s_end, j + 1, (int)nw - 1, q);
                     ej = s_end[j];
                     vj = s_val[j];
                 }
@@ -757,7 +768,8 @@ __device__ __forceinline__ void fill_item(const BatchArgs &a, const BatchItem &i
                     // plus the number of runs among j, j+1, j+2 that end at or
                     // before it (ends read independently, clamped to the
                     // window's last run, whose end exceeds every position).
-                    const uint32_t e1 = s_end[min(j + 1, nw - 1)], e2 = s_end[min(j + 2, nw - 1)];
+                    const int last = (int)nw - 1;
+                    const uint32_t e1 = s_end[min(j + 1, last)], e2 = s_end[min(j + 2, last)];
                     int32_t r[4];
                     r[0] = vj;  // q < ej
 #pragma unroll
@@ -779,23 +791,25 @@ __device__ __forceinline__ void fill_item(const BatchArgs &a, const BatchItem &i
                 p = tid < n_front ? pos + tid : q_hi + (tid - n_front);
             }
             if (p >= pos && p < hi && (w_lo >= w_hi || p < q_lo || p >= q_hi))
-                out[p] = s_val[first_after(s_end, 0, nw - 1, p)];
+                out[p] = s_val[first_run_after(s_end, 0, (int)nw - 1, p)];
         }
         pos = hi;
         k_cur += nw;
     }
     if (a.prof) {
         __syncthreads();
-        if (tid == 0) prof_item(a, kItemFill, t0, 0);
+        if (tid == 0) prof_item(a, kItemFill, t0, 0, part == 0);
     }
 }
 
 
 template <bool DEV>
-__global__ void __launch_bounds__(kFillCtaThreads) seg_fill_kernel(BatchArgs a) {
+__global__ void __launch_bounds__(kFillCtaThreads, 6) seg_fill_kernel(BatchArgs a) {
     __shared__ uint32_t s_end[kSegFillRuns];
     __shared__ int32_t s_val[kSegFillRuns];
+    __shared__ __align__(16) uint32_t s_m[kFillWarps * kBlock];
     const uint32_t tid = threadIdx.x;
+    const uint32_t item = blockIdx.x / a.fill_parts, part = blockIdx.x - item * a.fill_parts;
     if (DEV && blockIdx.x == 0) {
         // The first CTA leaves the device planner's ticket and lookback
         // records zeroed for the next run (the planner finished before this
@@ -803,7 +817,7 @@ __global__ void __launch_bounds__(kFillCtaThreads) seg_fill_kernel(BatchArgs a) 
         for (uint32_t i = tid; i < a.plan_look_words; i += blockDim.x) a.plan_look[i] = 0;
         if (tid == 0) a.ctl->plan_ticket = 0;
     }
-    if (DEV && blockIdx.x >= a.dev_counts[3]) {
+    if (DEV && item >= a.dev_counts[3]) {
         // Past the device-built list (the grid is sized by its bound); the
         // first CTA still resets the scan ticket, even for an empty list.
         if (blockIdx.x == 0) {
@@ -815,13 +829,21 @@ __global__ void __launch_bounds__(kFillCtaThreads) seg_fill_kernel(BatchArgs a) 
     // The item and its segment are plan data: fetched before waiting for the
     // scan launch.  A host plan's output items sit after its other lists;
     // device-built ones in two lists by cost, the expensive one first.
-    const BatchItem it = a.items[DEV ? devplan_chain_pos(dev_lb(a), kListFill0, a.dev_counts + 11, 2, blockIdx.x)
-                                     : a.n_first + a.n_scan + a.n_small2 + blockIdx.x];
+    const BatchItem it = a.items[DEV ? devplan_chain_pos(dev_lb(a), kListFill0, a.dev_counts + 11, 2, item)
+                                     : a.n_first + a.n_scan + a.n_small2 + item];
     const BatchSeg g = a.segs[it.seg];
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const unsigned long long t0 = (a.prof && tid == 0) ? global_ns() : 0ull;
     if (blockIdx.x == 0 && tid == 0) a.ctl->scan_ticket = 0;
-    fill_item(a, it, g, s_end, s_val, t0);
+    fill_item(a, it, g, part, a.fill_parts, s_end, s_val, s_m, t0);
+}
+
+// CTAs per output item: two at least (they have 256 threads), and enough for
+// about four waves of six CTAs per SM when the items are few.
+uint32_t fill_parts(uint64_t items) {
+    uint32_t parts = items <= 0x3fffffffu ? 2 : 1;  // (a grid has fewer than 2^31 CTAs)
+    while (parts < 16 && items * parts < 3648) parts *= 2;
+    return parts;
 }
 
 namespace {
@@ -844,7 +866,9 @@ cudaError_t launch_dep(const void *fn, uint32_t grid, int threads, const BatchAr
 
 }  // namespace
 
-cudaError_t launch_batched(const BatchArgs &a, cudaStream_t s) {
+cudaError_t launch_batched(const BatchArgs &args, cudaStream_t s) {
+    BatchArgs a = args;
+    a.fill_parts = fill_parts(a.n_fill);
     cudaError_t e = cudaFuncSetAttribute(seg_first_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kSegSmemBytes);
     if (e != cudaSuccess) return e;
@@ -863,13 +887,15 @@ cudaError_t launch_batched(const BatchArgs &a, cudaStream_t s) {
         chained = true;
     }
     if (a.n_fill &&
-        (e = launch_dep((const void *)seg_fill_kernel<false>, a.n_fill, kFillCtaThreads, a, chained, s)) != cudaSuccess)
+        (e = launch_dep((const void *)seg_fill_kernel<false>, a.n_fill * a.fill_parts, kFillCtaThreads, a, chained, s)) != cudaSuccess)
         return e;
     return cudaSuccess;
 }
 
-cudaError_t launch_batched_dev(const BatchArgs &a, uint32_t first_ctas, uint32_t scan_ctas, uint32_t fill_ctas,
+cudaError_t launch_batched_dev(const BatchArgs &args, uint32_t first_ctas, uint32_t scan_ctas, uint32_t fill_items,
                                cudaStream_t s) {
+    BatchArgs a = args;
+    a.fill_parts = fill_parts(fill_items);
     cudaError_t e = cudaFuncSetAttribute(seg_first_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kSegSmemBytes);
     if (e != cudaSuccess) return e;
@@ -879,7 +905,7 @@ cudaError_t launch_batched_dev(const BatchArgs &a, uint32_t first_ctas, uint32_t
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     e = launch_dep((const void *)seg_scan_kernel<true>, scan_ctas, kScanCtaThreads, a, true, s);
     if (e != cudaSuccess) return e;
-    return launch_dep((const void *)seg_fill_kernel<true>, fill_ctas, kFillCtaThreads, a, true, s);
+    return launch_dep((const void *)seg_fill_kernel<true>, fill_items * a.fill_parts, kFillCtaThreads, a, true, s);
 }
 
 }  // namespace rtcdf

@@ -16,14 +16,14 @@ namespace rtcdf {
 //      plus the in-CTA sorts of the small segments with R <= kSmallInScanMaxR
 //      (these do not wait for the first launch, so they overlap its tail and
 //      the latency-bound scan chunks);
-//   3. output items of the large segments (512-thread CTAs).
+//   3. output items of the large segments (256-thread CTAs, several an item).
 constexpr int kSegThreads = 1024;
 constexpr size_t kSegSmemBytes = 112 * 1024;          // first launch, per CTA
 constexpr uint32_t kBatchSmallMaxN = 65535;           // 16-bit counters are exact below 2^16
 constexpr uint32_t kBatchSmallMaxR = 55296;           // 16-bit counters in 108 KB
 constexpr uint32_t kBatchTileMax = 28672;             // 32-bit tile histogram in 112 KB
 constexpr uint32_t kBatchScanChunk = 4096;            // bins per scan CTA (4 per thread)
-constexpr uint32_t kSegFillRuns = 4096;               // run window of an output CTA
+constexpr uint32_t kSegFillRuns = 2048;               // run window of an output CTA
 constexpr uint32_t kSmallInScanMaxR = 16000;          // default: in-CTA segments run by scan-launch CTAs
 // Shared memory of a scan-launch CTA (words): the chunk's staged runs (end and
 // value, one padding word per 32), reused for an in-CTA segment's counters and
@@ -94,11 +94,12 @@ struct BatchArgs {
     // The device planner's lookback records, zeroed by the output launch.
     uint32_t *plan_look = nullptr;
     uint32_t plan_look_words = 0;
+    uint32_t fill_parts = 1;  // CTAs of an output item (set by launch_batched*)
 };
 
 cudaError_t launch_batched(const BatchArgs &a, cudaStream_t s);
 // The three launches over device-built lists with fixed grids.
-cudaError_t launch_batched_dev(const BatchArgs &a, uint32_t first_ctas, uint32_t scan_ctas, uint32_t fill_ctas,
+cudaError_t launch_batched_dev(const BatchArgs &a, uint32_t first_ctas, uint32_t scan_ctas, uint32_t fill_items,
                                cudaStream_t s);
 
 // Host planner shared by the plan API and the server: segment s reads

@@ -18,83 +18,9 @@
 // All positions are below n < 2^32, so the index arithmetic is 32-bit.  The
 // CTA also clears the scan's lookback state so the workspace is ready for the
 // next sort.
-#include "rtcdf_internal.h"
+#include "fill_runs.cuh"
 
 namespace rtcdf {
-
-// Smallest j in [lo, hi] with s_end[j] > p, given s_end[hi] > p.
-__device__ __forceinline__ int first_run_after(const uint32_t *s_end, int lo, int hi, uint32_t p) {
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (s_end[mid] > p) hi = mid; else lo = mid + 1;
-    }
-    return lo;
-}
-
-// The same when the answer is expected close to lo: probes lo, lo + 1,
-// lo + 3, lo + 7, ... until s_end exceeds p, then a binary search inside the
-// last step -- O(log(j - lo)) reads, so a lane that crosses a few short runs
-// between its vectors does not pay a search over the whole window.
-__device__ __forceinline__ int next_run_after(const uint32_t *s_end, int lo, int hi, uint32_t p) {
-    int probe = lo, step = 1;
-    while (s_end[probe] <= p) {  // s_end[hi] > p ends it
-        lo = probe + 1;
-        probe = min(hi, probe + step);
-        step <<= 1;
-    }
-    return first_run_after(s_end, lo, probe, p);
-}
-
-// Short runs: a warp's vectors [wb, we) (positions from `frame` on, four a
-// vector), `kBlock` positions at a time.  The warp writes the key of every run
-// that begins in the block to its first position in `m` (kBlock words of shared
-// memory, `none` elsewhere: no key of the array), reads it back as vectors and
-// carries the last key before it into every position without one: a ballot
-// finds the lane that holds it.  The same rule as the searches (Algorithm 7),
-// at a cost that does not depend on the runs' lengths.
-constexpr int kBlock = 512;
-
-template <class Store>
-__device__ __forceinline__ void fill_short_runs(uint32_t *m, const uint32_t *s_end, const int32_t *s_val, int nw,
-                                                uint32_t frame, uint32_t wb, uint32_t we, int32_t none, Store store) {
-    const int lane = threadIdx.x & 31;
-    if (wb >= we) return;
-    int4 *m4 = reinterpret_cast<int4 *>(m);
-    int j = first_run_after(s_end, 0, nw - 1, frame + 4 * wb);  // the run of the block's first position
-    for (uint32_t w = wb; w < we; w += kBlock / 4) {
-        const uint32_t q0 = frame + 4 * w, q1 = min(q0 + kBlock, frame + 4 * we);
-#pragma unroll
-        for (int k = 0; k < kBlock / 128; k++) m4[lane + 32 * k] = make_int4(none, none, none, none);
-        int32_t carry = s_val[j];
-        __syncwarp();
-        for (int r = j + 1 + lane;; r += 32) {
-            const uint32_t start = r < nw ? s_end[r - 1] : 0xffffffffu;
-            const bool begins = start < q1;
-            if (begins) m[start - q0] = (uint32_t)s_val[r];
-            const unsigned b = __ballot_sync(0xffffffffu, begins);
-            j += __popc(b);
-            if (b != 0xffffffffu) break;
-        }
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < kBlock / 128; k++) {
-            int4 x = m4[lane + 32 * k];
-            const int32_t last = x.w != none ? x.w : x.z != none ? x.z : x.y != none ? x.y : x.x;
-            const unsigned has = __ballot_sync(0xffffffffu, last != none);
-            const unsigned before = has & ((1u << lane) - 1u);
-            const int32_t from = __shfl_sync(0xffffffffu, last, before ? 31 - __clz(before) : 0);
-            const int32_t next = __shfl_sync(0xffffffffu, last, has ? 31 - __clz(has) : 0);
-            if (x.x == none) x.x = before ? from : carry;
-            if (x.y == none) x.y = x.x;
-            if (x.z == none) x.z = x.y;
-            if (x.w == none) x.w = x.z;
-            if (has) carry = next;
-            const uint32_t v = w + lane + 32 * k;
-            if (v < we) store(v, x);
-        }
-        __syncwarp();  // the block has been read
-    }
-}
 
 // Runs per shared-memory window: four per thread (eight for short runs), so that a CTA whose
 // positions cross thousands of short runs (the tails of a peaked distribution

@@ -283,3 +283,24 @@ def test_in_cta_counter_layouts_at_their_capacity(scan_max_R):
     assert plan.info()["small_segments"] == len(lengths)
     check_segments(x, out, offs, mn, mx)
     plan.close()
+
+
+@pytest.mark.parametrize("lengths,Rs", [
+    ([65536], [65536]), ([70_001, 200_000, 131_073], [1 << 16, 3, 1 << 17]),        # several CTAs an output item
+    ([1_000_000] * 6, [1 << 20, 1 << 18, 1 << 16, 5000, 4000, 1]),                 # both forms of the output
+])
+@pytest.mark.parametrize("lead", [0, 1])
+def test_output_items_in_parts(lengths, Rs, lead):
+    L = np.array([lead] + lengths, np.int64)                # an odd first segment shifts every later one
+    R = np.array([1] + Rs, np.int64)
+    mn = np.array([-(1 << 31)] * len(L), np.int64)
+    x, offs, mins, maxs = make_segments(L, R, mn, np.arange(len(L)) % 2, np.arange(len(L)) + 90)
+    out = torch.full((x.numel() + 4,), -3, dtype=torch.int32, device="cuda")
+    plan = rtcdf.BatchPlan(offs, mins, maxs)
+    wsb = plan.workspace_size()
+    ws = torch.zeros(wsb // 4 + 64, dtype=torch.int32, device="cuda")
+    for _ in range(2):
+        assert plan.run(x.data_ptr(), out.data_ptr(), ws.data_ptr(), wsb, stream_handle()) == rtcdf.OK
+    assert rtcdf.rtcdf_batch_status_get(ws.data_ptr(), stream_handle()) == (rtcdf.OK, 0)
+    assert bool((out[x.numel():] == -3).all())
+    check_segments(x, out[:x.numel()], offs, mins, maxs)
