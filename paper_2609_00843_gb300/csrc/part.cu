@@ -2,7 +2,7 @@
 // partition: every key is read from HBM once and counted once, where the
 // range-tile kernel (hist.cu) reads and examines every key once per tile.
 //
-//   part_kernel   cuts the input into slabs (16384 keys), partitions each slab
+//   part_kernel   cuts the input into slabs (32768 keys), partitions each slab
 //                 in shared memory by bucket (value >> 15, at most 512 buckets)
 //                 and writes the 15-bit positions inside the buckets to scratch,
 //                 two bytes a key: the slab's buckets one after another, each
@@ -18,10 +18,10 @@
 // output kernel fills it (2 bytes a key plus padding, of its 4); a sort in
 // place has none and keeps the range-tile kernel.
 //
-// Measured (n = 1e8, uniform / normal / one value, histogram of a sort, us; the
-// range tiles before that): R = 2^19 219 / 242 / 176 (459 / 424 / 400), 2^20
-// 230 / 251 / 179 (771 / 777 / 717), 2^22 277 / 297 / 208 (2394 / 2699 / 2718),
-// 2^24 398 / 380 / 271 (8144 / 8353 / 9810).
+// Measured (n = 1e8, uniform / normal / one value, both kernels, us; the range
+// tiles before that): R = 2^19 214 / 225 / 167 (459 / 424 / 400), 2^20 220 / 237 / 172
+// (771 / 777 / 717), 2^22 287 / 273 / 198 (2394 / 2699 / 2718), 2^24 335 / 329 / 246
+// (8144 / 8353 / 9810).
 #include <algorithm>
 
 #include "rtcdf_internal.h"
@@ -32,16 +32,16 @@ namespace {
 
 constexpr uint32_t kPartShift = 15;
 constexpr uint32_t kPartWidth = 1u << kPartShift;  // values per bucket
-constexpr int kPartThreads = 512;
-constexpr uint32_t kPartSlabMax = 16384;           // keys per slab
+constexpr int kPartThreads = 1024;
+constexpr uint32_t kPartSlabMax = 32768;           // keys per slab: 32 a thread, in registers
 constexpr uint32_t kPartSlabMin = 4096;
 static_assert(kPartSlabMax % (4 * kPartThreads) == 0, "slabs are whole vectors of the CTA");
+static_assert(kPartMaxBuckets <= kPartThreads, "one thread per bucket");
 constexpr int kBucketThreads = 1024;
 constexpr uint32_t kPartList = 4096;               // slabs listed at once
 // A bucket's tile (zeroed, and its counts added to H) costs about as much as
 // counting this many keys, and looking up the bucket in a slab as counting 2.
 constexpr uint32_t kPartTileKeys = 32768;
-static_assert(kPartMaxBuckets <= kPartThreads, "one thread per bucket");
 static_assert(RTCDF_MAX_R >> kPartShift == kPartMaxBuckets, "buckets of the widest range");
 
 // Counters per bucket, log2: lane l of a warp counts in copy l mod copies.
@@ -81,14 +81,16 @@ __device__ __forceinline__ uint32_t pad_of(uint32_t bucket) { return bucket & 1 
 
 }  // namespace
 
-// Two CTAs per SM with a slab each in registers (32 keys a thread, so the input
-// is read once), whose next slab's loads are in flight while the staged one is
-// written out.  What bounds it (n = 1e8, R = 2^20, 149 us; the 4 + 2 bytes a key
-// take 88): about 18 instructions a key and the shared-memory pipe, 7 wavefronts
-// for 32 keys, of which the two-byte stores' bank conflicts are four.  Reading
-// the keys a second time from L2 instead, at four CTAs per SM, took 157 us.
+// One CTA per SM with a slab in registers (32 keys a thread, so the input is read
+// once), whose next slab's loads are in flight while the staged one is written
+// out.  What bounds it (n = 1e8, R = 2^20, 149 us; the 4 + 2 bytes a key take 88):
+// about 18 instructions a key, the shared-memory pipe, 7 wavefronts for 32 keys,
+// of which the two-byte stores' bank conflicts are four, and seven barriers a
+// slab.  Two CTAs per SM with half the slab each take the same time, but shorter
+// runs slow bucket_kernel down (R = 2^24: 139 us against 202; 2^20: 71 against 80);
+// the keys read a second time from L2 instead, at four CTAs per SM, took 157 us.
 template <int LOGC>
-__global__ void __launch_bounds__(kPartThreads, 2) part_kernel(PartArgs a) {
+__global__ void __launch_bounds__(kPartThreads, 1) part_kernel(PartArgs a) {
     extern __shared__ __align__(128) uint32_t sm[];
     constexpr uint32_t C = 1u << LOGC;
     constexpr int V = kPartSlabMax / 4 / kPartThreads;  // vectors of a slab per thread
@@ -177,7 +179,6 @@ __global__ void __launch_bounds__(kPartThreads, 2) part_kernel(PartArgs a) {
         if (lane >= tid >> 5) w = 0;
         const uint32_t off = __reduce_add_sync(0xffffffffu, w) + inc - room;
         if (tid <= B) s_off[tid] = off;
-        if (B == kPartThreads && tid + 1 == B) s_off[B] = off + room;
         row += t;
         for (uint32_t p = off + t; p < off + room; p++) sts_u16(stage_slot(stage + 2 * p), pad_of(tid));
         __syncthreads();
@@ -224,7 +225,7 @@ __global__ void __launch_bounds__(kPartThreads, 2) part_kernel(PartArgs a) {
 // item's slabs, 4096 at a time, are listed in shared memory as pieces of up to
 // 128 units and the warps take the pieces in turn.  Either way each thread has
 // the next four units in flight while it counts four, and the runs' ends are
-// looked up one step earlier still.  n = 1e8, R = 2^20: 80 us uniform, 99 normal
+// looked up one step earlier still.  n = 1e8, R = 2^20: 71 us uniform, 89 normal
 // (30 for the reads alone): bound by its shared-memory reductions and, for
 // buckets of a few keys a slab, by the latency of their many short runs (one run
 // at a time instead of the groups of lanes: 206 us for the normal keys).
@@ -444,10 +445,9 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(PartArgs a) {
 bool part_plan(uint64_t n, uint32_t R, uint32_t head, uint64_t nvec, uintptr_t out_addr, int sms, PartPlan *p) {
     p->buckets = (R + kPartWidth - 1) >> kPartShift;
     const uint32_t B = p->buckets;
-    // Slabs of up to 16384 keys, fewer when the input has less than that for
-    // each of two CTAs per SM.
-    const uint64_t slots = 2ull * sms;
-    const uint64_t want = (n + slots - 1) / slots;
+    // Slabs of up to 32768 keys, fewer when the input has less than that for
+    // each SM.
+    const uint64_t want = (n + sms - 1) / sms;
     // (in whole vectors of the CTA: its threads' vectors past a slab's end are
     // staged too, as keys outside the range)
     const uint64_t step = 4 * kPartThreads;
@@ -457,7 +457,7 @@ bool part_plan(uint64_t n, uint32_t R, uint32_t head, uint64_t nvec, uintptr_t o
     p->slabs = (uint32_t)slabs;
     // A slab's keys (and up to six outside whole vectors), each bucket padded to 8.
     p->slab_units = (p->slab_keys + 8 + 8 * B) / 8;
-    p->ctas = (uint32_t)std::min<uint64_t>(slabs, slots);
+    p->ctas = (uint32_t)std::min<uint64_t>(slabs, sms);
     p->smem = 4 * (size_t)part_head_words(B) + align_up(16 * (size_t)p->slab_units, 128);
     const uintptr_t base = (out_addr + 15) & ~(uintptr_t)15;
     const uint64_t payload = slabs * p->slab_units * 16;
