@@ -445,13 +445,14 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(PartArgs a) {
 bool part_plan(uint64_t n, uint32_t R, uint32_t head, uint64_t nvec, uintptr_t out_addr, int sms, PartPlan *p) {
     p->buckets = (R + kPartWidth - 1) >> kPartShift;
     const uint32_t B = p->buckets;
-    // Slabs of up to 32768 keys, fewer when the input has less than that for
-    // each SM.
+    // Slabs of up to 32768 keys, as even over the SMs as whole vectors of the
+    // CTA allow.
     const uint64_t want = (n + sms - 1) / sms;
     // (in whole vectors of the CTA: its threads' vectors past a slab's end are
     // staged too, as keys outside the range)
     const uint64_t step = 4 * kPartThreads;
-    const uint64_t keys = std::max<uint64_t>({kPartSlabMin, 16ull * B, want});
+    const uint64_t rounds = (want + kPartSlabMax - 1) / kPartSlabMax;
+    const uint64_t keys = std::max<uint64_t>({kPartSlabMin, 16ull * B, (want + rounds - 1) / rounds});
     p->slab_keys = (uint32_t)std::min<uint64_t>(kPartSlabMax, (keys + step - 1) / step * step);
     const uint64_t slabs = std::max<uint64_t>(1, (nvec + p->slab_keys / 4 - 1) / (p->slab_keys / 4));
     p->slabs = (uint32_t)slabs;
