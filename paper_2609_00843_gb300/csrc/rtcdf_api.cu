@@ -298,6 +298,22 @@ rtcdf_status run_pipeline(const int32_t *in, int32_t *out, uint64_t n, int64_t m
     return finish_phase(out, n, minVal, R, pl, L, base, dbg, ev[2], ev[3], s, 0, n);
 }
 
+// One sort with checked arguments in a workspace of at least ws_required(R) bytes.
+rtcdf_status sort_checked(const int32_t *in, int32_t *out, uint64_t n, int64_t minVal, uint32_t R,
+                          const rtcdf_params *params, void *ws, size_t ws_bytes, const rtcdf_debug *dbg,
+                          cudaStream_t s) {
+    // Small arrays in one launch (small.cu), unless the caller asks for launch
+    // parameters, intermediates or stage events.
+    if (n <= kSmallMaxN && R <= kSmallMaxR && !params && !dbg && tune_is_builtin())
+        return launch_small(in, out, (uint32_t)n, (uint32_t)(int32_t)minVal, R, (Ctl *)ws, s) == cudaSuccess
+                   ? RTCDF_OK
+                   : RTCDF_ERR_CUDA;
+    Plan pl;
+    const rtcdf_status st = make_plan(n, R, (uintptr_t)in, (uintptr_t)out, params, &pl);
+    if (st) return st;
+    return run_pipeline(in, out, n, minVal, R, pl, ws, ws_bytes, dbg, s);
+}
+
 // ---------------------------------------------------------------- workspace cache
 struct CachedWs {
     void *ptr = nullptr;
@@ -374,10 +390,7 @@ rtcdf_status sort_with_workspace(const int32_t *in, int32_t *out, uint64_t n, in
     if (!ws || ws_bytes < ws_required(R)) return RTCDF_ERR_NO_MEMORY;
     const WsLayout L = ws_layout(R, ws_bytes);
     if (cudaMemsetAsync(ws, 0, L.zero_bytes, s) != cudaSuccess) return RTCDF_ERR_CUDA;
-    Plan pl;
-    st = make_plan(n, R, (uintptr_t)in, (uintptr_t)out, nullptr, &pl);
-    if (st) return st;
-    return run_pipeline(in, out, n, minVal, R, pl, ws, ws_bytes, nullptr, s);
+    return sort_checked(in, out, n, minVal, R, nullptr, ws, ws_bytes, nullptr, s);
 }
 
 // The two halves of a sort, for rtcdf_sort_host: histogram of a slice (may be
@@ -453,11 +466,7 @@ rtcdf_status rtcdf_sort_ex(const int32_t *in, int32_t *out, uint64_t n, int64_t 
     if (st) return st;
     if (!workspace || ((uintptr_t)workspace & 255)) return RTCDF_ERR_INVALID_ARG;
     if (ws_bytes < ws_required(R)) return RTCDF_ERR_NO_MEMORY;
-    Plan pl;
-    st = make_plan(n, R, (uintptr_t)in, (uintptr_t)out, params, &pl);
-    if (st) return st;
-    return run_pipeline(in, out, n, minVal, R, pl, workspace, ws_bytes, debug,
-                        (cudaStream_t)stream);
+    return sort_checked(in, out, n, minVal, R, params, workspace, ws_bytes, debug, (cudaStream_t)stream);
 }
 
 rtcdf_status rtcdf_sort_ws(const int32_t *in, int32_t *out, uint64_t n, int64_t minVal,
@@ -485,10 +494,7 @@ rtcdf_status rtcdf_sort(const int32_t *in, int32_t *out, uint64_t n, int64_t min
     size_t ws_bytes = 0;
     st = cached_workspace((cudaStream_t)stream, ws_required(R), &ws, &ws_bytes);
     if (st) return st;
-    Plan pl;
-    st = make_plan(n, R, (uintptr_t)in, (uintptr_t)out, nullptr, &pl);
-    if (st) return st;
-    return run_pipeline(in, out, n, minVal, R, pl, ws, ws_bytes, nullptr, (cudaStream_t)stream);
+    return sort_checked(in, out, n, minVal, R, nullptr, ws, ws_bytes, nullptr, (cudaStream_t)stream);
 }
 
 rtcdf_status rtcdf_hist_accumulate(const int32_t *in, uint64_t n, int64_t minVal, int64_t maxVal,

@@ -13,6 +13,8 @@ namespace rtcdf {
 // Launch parameters of the tuning table for (n, R), if it has an entry
 // (tune.cu); whether the table is the compiled-in one.
 bool tune_lookup(uint64_t n, uint32_t R, rtcdf_params *out, bool *builtin);
+// Whether the tuning table is the compiled-in one.
+bool tune_is_builtin();
 
 // Device status bits (mirror RTCDF_DEV_* in rtcdf.h).
 constexpr uint32_t kDevKeyOutOfRange = 0x1;
@@ -106,6 +108,19 @@ struct HistArgs {
 cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool streaming,
                         cudaStream_t s);
 cudaError_t hist_max_ctas_per_sm(int threads, size_t smem, bool streaming, int *ctas);
+
+// ---------------------------------------------------------------- small arrays
+constexpr uint32_t kSmallMaxN = 32768, kSmallMaxR = 16384;
+struct SmallArgs {
+    const int32_t *in;
+    int32_t *out;
+    uint32_t n, R, min_u;
+    uint32_t words, max_runs;  // shared memory: counters (and the output's blocks), runs
+    Ctl *ctl;
+};
+// The whole sort of n <= kSmallMaxN keys over R <= kSmallMaxR values in one CTA.
+cudaError_t launch_small(const int32_t *in, int32_t *out, uint32_t n, uint32_t min_u, uint32_t R, Ctl *ctl,
+                         cudaStream_t s);
 
 // ---------------------------------------------------------------- packed histogram
 struct PackArgs {

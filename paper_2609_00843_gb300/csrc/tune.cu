@@ -3,6 +3,7 @@
 // mean of their normalised times (Section 4.1's selection of the tile width,
 // applied to every launch parameter).
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <mutex>
 #include <vector>
@@ -22,13 +23,14 @@ const rtcdf_tune_entry kBuiltin[] = {
 std::mutex g_tune_mu;
 std::vector<rtcdf_tune_entry> g_table;
 bool g_loaded = false;
-bool g_builtin = false;  // the table is the compiled-in one
+std::atomic<bool> g_builtin{true};  // the table is the compiled-in one (also before it is loaded)
 
 void load_builtin_locked() {
     g_table.clear();
     for (const rtcdf_tune_entry &e : kBuiltin)
         if (e.log2_R >= 0) g_table.push_back(e);
-    g_loaded = g_builtin = true;
+    g_loaded = true;
+    g_builtin = true;
 }
 
 int32_t log2_ceil(uint32_t R) {
@@ -40,6 +42,8 @@ int32_t log2_ceil(uint32_t R) {
 }  // namespace
 
 namespace rtcdf {
+
+bool tune_is_builtin() { return g_builtin.load(std::memory_order_relaxed); }
 
 bool tune_lookup(uint64_t n, uint32_t R, rtcdf_params *out, bool *builtin) {
     const int32_t lr = log2_ceil(R), nc = rtcdf_tune_n_class(n);

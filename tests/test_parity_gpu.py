@@ -374,3 +374,24 @@ def test_bounded_wait_runs_out_and_reports_timeout():
     assert rc == rtcdf.OK
     assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
     assert_matches_oracle(x, out, 0, R)
+
+
+# One launch for the whole sort: its largest size and range and one more of each,
+# the smallest, keys and outputs at every alignment, a key out of range, in place.
+@pytest.mark.parametrize("n", [1, 3, 5, 4095, 10_007, 32768, 32769])
+@pytest.mark.parametrize("R", [1, 2, 1024, 1025, 16384, 16385])
+def test_small_arrays(n, R):
+    for k in range(4):
+        mn = (-(1 << 31), (1 << 31) - R, -5, 0)[k]
+        x = torch.empty(n + 3, dtype=torch.int32, device="cuda")[k:k + n]
+        gen.keys_device(x.data_ptr(), n, mn, R, k % 3, gen.derive_seed(81, n, R), stream=stream_handle())
+        out = torch.full((n + 8,), 9, dtype=torch.int32, device="cuda")
+        gpu_sort(x, mn, mn + R, out[3 - k:3 - k + n])
+        assert_matches_oracle(x, out[3 - k:3 - k + n], mn, mn + R)
+        assert bool((out[:3 - k] == 9).all()) and bool((out[3 - k + n:] == 9).all())
+        y = x.clone()
+        gpu_sort(y, mn, mn + R, y)
+        assert torch.equal(y, out[3 - k:3 - k + n])
+    x[n // 2] = mn + R
+    assert rtcdf.rtcdf_sort(x.data_ptr(), y.data_ptr(), n, mn, mn + R, stream_handle()) == rtcdf.OK
+    assert rtcdf.rtcdf_status_get(stream_handle()) == (rtcdf.ERR_KEY_OUT_OF_RANGE, rtcdf.DEV_KEY_OUT_OF_RANGE)
