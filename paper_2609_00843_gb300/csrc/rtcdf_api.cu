@@ -60,6 +60,7 @@ struct Plan {
     size_t hist_smem;
     bool streaming;
     bool shape_given;   // the histogram's shape comes from the caller or the tuning table
+    bool fill_given;    // the output's shape comes from the caller
     int sms;
     uint32_t head;
     uint64_t nvec;
@@ -142,8 +143,9 @@ rtcdf_status make_plan_with(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t
     // Not clamped to n: positions below head_out are written one by one, and
     // the vector frame must stay 16-byte aligned.
     const uint32_t head_out = (uint32_t)(((16 - (out_addr & 15)) & 15) / 4);
+    pl->fill_given = p != nullptr;
     const bool short_fill = short_runs(n, R) && !q.fill_threads && !q.fill_ctas && !q.fill_chunk;
-    pl->fill_threads = q.fill_threads ? q.fill_threads : short_fill && n >= 2000000 ? 256 : 512;
+    pl->fill_threads = q.fill_threads ? q.fill_threads : short_fill ? 256 : 512;
     if (pl->fill_threads != 256 && pl->fill_threads != 512 && pl->fill_threads != 1024)
         return RTCDF_ERR_INVALID_ARG;
     // Many more CTAs than fit at once (about 32K positions each, at least four
@@ -152,8 +154,7 @@ rtcdf_status make_plan_with(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t
     // are short (few keys per value) small CTAs with 4096 positions, or as few
     // as kMaxFillCtas allows, are best (R = 2^20 normal, output kernel, us, for
     // 256 threads with 4K / 8K / 16K / 32K positions and 512 threads with 4K /
-    // 16K: n = 1e7 16 / 23 / 35 / 55 and 27 / 23; 3e6 14 / 21 / 35 / 55 and 12 / 21;
-    // 1e6 12 / 21 / 35 / 57 and 10 / 23).
+    // 16K: n = 1e7 16 / 23 / 35 / 55 and 27 / 23; 3e6 14 / 21 / 35 / 55 and 12 / 21).
     uint64_t body = n > head_out ? n - head_out : 0;
     uint64_t chunk;
     if (q.fill_chunk < 0 || q.fill_ctas < 0) return RTCDF_ERR_INVALID_ARG;
@@ -162,7 +163,9 @@ rtcdf_status make_plan_with(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t
                                    (body + kMaxFillCtas - 1) / kMaxFillCtas);
         chunk = std::max<uint64_t>(chunk, 4 * (uint64_t)pl->fill_threads);
     } else if (short_fill) {
-        chunk = std::max<uint64_t>(4096, (body + kMaxFillCtas - 1) / kMaxFillCtas);
+        // (fewer than 4096 when that makes less than four CTAs per SM)
+        chunk = std::min<uint64_t>(4096, std::max<uint64_t>(1024, body / (4 * (uint64_t)dev.sms)));
+        chunk = std::max<uint64_t>(chunk, (body + kMaxFillCtas - 1) / kMaxFillCtas);
     } else {
         uint64_t want = q.fill_ctas > 0 ? (uint64_t)q.fill_ctas
                                         : std::max<uint64_t>((uint64_t)dev.sms * 4, body / 32768);
@@ -188,9 +191,12 @@ rtcdf_status make_plan(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t out_
     const bool found = tune_lookup(n, R, &t, &builtin);
     // (the compiled-in table's output shapes are those of the kernel's form for long runs)
     if (found && builtin && short_runs(n, R)) t.fill_ctas = t.fill_threads = t.fill_chunk = 0;
-    if (found && make_plan_with(n, R, in_addr, out_addr, &t, pl) == RTCDF_OK)
-        return RTCDF_OK;
-    return make_plan_with(n, R, in_addr, out_addr, nullptr, pl);
+    if (!(found && make_plan_with(n, R, in_addr, out_addr, &t, pl) == RTCDF_OK)) {
+        const rtcdf_status st = make_plan_with(n, R, in_addr, out_addr, nullptr, pl);
+        if (st) return st;
+    }
+    pl->fill_given = !tune_is_builtin();
+    return RTCDF_OK;
 }
 
 bool overlaps(const void *a, const void *b, uint64_t n) {
@@ -244,6 +250,13 @@ rtcdf_status hist_phase(const int32_t *in, uint64_t n, int64_t minVal, uint32_t 
     return e == cudaSuccess ? RTCDF_OK : RTCDF_ERR_CUDA;
 }
 
+// Most positions that scan and output in one launch serve (small.cu).  Whole
+// sorts replayed from a graph, us, one launch / two, uniform keys over R = 128 and
+// 16384: n = 1e6 6.4 / 7.9 and 11.9 / 15.3, 1e7 17.5 / 17.9 and 24.5 / 25.9, 3e7
+// 45.1 / 46.3 and 50.8 / 53.4, 6e7 85.1 / 84.8 and 89.2 / 91.0, 1e8 140 / 137 and
+// 143 / 140: one CTA per SM stores a little slower than the output kernel's many.
+constexpr uint64_t kFinishMaxN = 40000000;
+
 // Local CDFs + offsets (Algorithm 6) and output generation (Algorithm 7)
 // for an n-key array whose histogram is in H: positions [pos_base, pos_end)
 // of the sorted array are written, position p to out[p - pos_base] (the
@@ -258,6 +271,13 @@ rtcdf_status finish_phase(int32_t *out, uint64_t n, int64_t minVal, uint32_t R, 
     int32_t *run_val = (int32_t *)(base + L.run_val);
     uint32_t *start_run = (uint32_t *)(base + L.start_run);
     const uint32_t head_out = (uint32_t)(((16 - ((uintptr_t)out & 15)) & 15) / 4);
+    if (!dbg && !pl.fill_given && R <= kSmallMaxR && pos_end - pos_base <= kFinishMaxN) {
+        FinishArgs f;
+        f.H = (uint32_t *)(base + L.hist); f.out = out; f.n = (uint32_t)n;
+        f.pos_base = (uint32_t)pos_base; f.pos_end = (uint32_t)pos_end;
+        f.R = R; f.min_u = (uint32_t)(int32_t)minVal; f.ctl = ctl;
+        return launch_finish(f, pl.sms, s) == cudaSuccess ? RTCDF_OK : RTCDF_ERR_CUDA;
+    }
     ScanArgs sc;
     sc.H = (uint32_t *)(base + L.hist); sc.state = state; sc.ctl = ctl; sc.run_end = run_end;
     sc.run_val = run_val; sc.start_run = start_run; sc.n = n; sc.fill_chunk = pl.fill_chunk;

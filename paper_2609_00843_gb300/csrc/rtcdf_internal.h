@@ -45,7 +45,8 @@ struct Ctl {
     uint32_t num_runs;     // number of values with c_v > 0 (written by the scan)
     uint32_t part_ticket;  // items of bucket_kernel taken so far (zero between sorts)
     uint32_t pack_copies;  // written-out counters of pack_kernel (written before it is read)
-    uint32_t pad[59];
+    uint32_t finished;     // CTAs of finish_kernel that have read H (zero between sorts)
+    uint32_t pad[58];
 };
 static_assert(sizeof(Ctl) == 256, "control block is 256 bytes");
 
@@ -121,6 +122,16 @@ struct SmallArgs {
 // The whole sort of n <= kSmallMaxN keys over R <= kSmallMaxR values in one CTA.
 cudaError_t launch_small(const int32_t *in, int32_t *out, uint32_t n, uint32_t min_u, uint32_t R, Ctl *ctl,
                          cudaStream_t s);
+
+// Scan and output of counts H over R <= kSmallMaxR values in one launch.
+struct FinishArgs {
+    uint32_t *H;           // R counts, zeroed
+    int32_t *out;          // out[0] holds position pos_base
+    uint32_t n, pos_base, pos_end, R, min_u;
+    uint32_t words, max_runs;  // (set by launch_finish)
+    Ctl *ctl;
+};
+cudaError_t launch_finish(const FinishArgs &a, int sms, cudaStream_t s);
 
 // ---------------------------------------------------------------- packed histogram
 struct PackArgs {

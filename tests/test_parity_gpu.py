@@ -395,3 +395,31 @@ def test_small_arrays(n, R):
     x[n // 2] = mn + R
     assert rtcdf.rtcdf_sort(x.data_ptr(), y.data_ptr(), n, mn, mn + R, stream_handle()) == rtcdf.OK
     assert rtcdf.rtcdf_status_get(stream_handle()) == (rtcdf.ERR_KEY_OUT_OF_RANGE, rtcdf.DEV_KEY_OUT_OF_RANGE)
+
+
+# Scan and output in one launch: the sizes around it, windows of a sharded sort,
+# and counts that do not add up.
+@pytest.mark.parametrize("n,R", [(32769, 1), (40_001, 16384), (100_003, 3), (1_000_001, 16383), (39_999_999, 1000),
+                                 (40_000_001, 16384)])
+@pytest.mark.parametrize("dist", [gen.UNIFORM, gen.NORMAL])
+def test_scan_and_output_in_one_launch(n, R, dist):
+    mn, s = -(1 << 31), stream_handle()
+    x = dev_keys(n, mn, R, dist, gen.derive_seed(82, n, R))
+    out = torch.full((n + 4,), 9, dtype=torch.int32, device="cuda")
+    gpu_sort(x, mn, mn + R, out[1:1 + n])
+    assert_matches_oracle(x, out[1:1 + n], mn, mn + R)
+    assert int(out[0]) == 9 and bool((out[1 + n:] == 9).all())
+    counts = torch.zeros(R, dtype=torch.int32, device="cuda")
+    assert rtcdf.rtcdf_hist_accumulate(x.data_ptr(), n, mn, mn + R, counts.data_ptr(), s) == rtcdf.OK
+    wsb = rtcdf.rtcdf_workspace_size(R)
+    ws = torch.zeros(wsb // 4, dtype=torch.int32, device="cuda")
+    win = torch.full((n + 4,), 9, dtype=torch.int32, device="cuda")
+    cuts = [0, 1, n // 3 + 1, n - 2, n]
+    for lo, hi in zip(cuts, cuts[1:]):
+        assert rtcdf.rtcdf_fill_from_counts(counts.data_ptr(), n, mn, mn + R, lo, hi, win[1:].data_ptr() + 4 * lo,
+                                            ws.data_ptr(), wsb, s) == rtcdf.OK
+    assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
+    assert torch.equal(win, out)
+    assert rtcdf.rtcdf_fill_from_counts(counts.data_ptr(), n - 1, mn, mn + R, 0, n - 1, win.data_ptr(), ws.data_ptr(),
+                                        wsb, s) == rtcdf.OK
+    assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s)[1] == rtcdf.DEV_KEY_OUT_OF_RANGE
