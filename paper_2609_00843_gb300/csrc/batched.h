@@ -36,7 +36,7 @@ constexpr uint64_t kBatchMaxR = 1ull << 20;
 enum : uint32_t { kItemHist = 0, kItemSmall = 1, kItemScan = 2, kItemFill = 3 };
 
 // One segment (all offsets in 32-bit words of the workspace).
-struct BatchSeg {
+struct alignas(16) BatchSeg {
     uint64_t off;          // first element of the segment in `in`
     uint64_t out_off;      // first element of the segment in `out`
     uint32_t n, R;
@@ -49,7 +49,7 @@ struct BatchSeg {
     uint64_t hist_off, run_end_off, run_val_off, start_run_off, state_off;
 };
 
-struct BatchItem {
+struct alignas(16) BatchItem {
     uint32_t kind, seg;
     uint64_t a, b;         // HIST: key range; SCAN: chunk index; FILL: position range
     uint32_t tile;         // HIST: range tile
@@ -290,21 +290,22 @@ __host__ __device__ inline bool devplan_segment(int64_t o0, int64_t o1, int64_t 
     }
     g->m = (g->R + kBatchTileMax - 1) / kBatchTileMax;
     g->T = (g->R + g->m - 1) / g->m;
-    const uint64_t chunks = (n + t.hist_chunk - 1) / t.hist_chunk;
-    g->hist_items = (uint32_t)(chunks * g->m);
+    // (32-bit divisions: n < 2^32, and so is the chunk)
+    const uint32_t hist_chunk = (uint32_t)t.hist_chunk;
+    const uint32_t whole = g->n / hist_chunk, rest = g->n - whole * hist_chunk, chunks = whole + (rest ? 1u : 0u);
+    const uint32_t fwhole = g->n / t.fill_chunk, frest = g->n - fwhole * t.fill_chunk;
+    g->hist_items = chunks * g->m;
     g->single_hist = chunks == 1 ? 1u : 0u;
     g->scan_chunks = (g->R + kBatchScanChunk - 1) / kBatchScanChunk;
     g->fill_chunk = t.fill_chunk;
-    g->fill_items = (uint32_t)((n + t.fill_chunk - 1) / t.fill_chunk);
+    g->fill_items = fwhole + (frest ? 1u : 0u);
     // Whole histogram chunks are class 0; the last chunk, when shorter, goes
     // by its keys.  Output items likewise: the whole ones share a class, the
     // last one goes by its length.
-    const uint64_t whole = n / t.hist_chunk, rest = n - whole * t.hist_chunk;
-    c->v[kListHist0] = (uint32_t)(whole * g->m);
+    c->v[kListHist0] = whole * g->m;
     if (rest) c->v[devplan_hist_class(rest, t.hist_chunk)] += g->m;
     c->v[g->scan_chunks >= kLongChain ? kListScan0 : kListScan1] = g->scan_chunks;
-    const uint64_t fwhole = n / t.fill_chunk, frest = n - fwhole * t.fill_chunk;
-    c->v[kListFill0 + devplan_fill_class(t.fill_chunk, *g)] = (uint32_t)fwhole;
+    c->v[kListFill0 + devplan_fill_class(t.fill_chunk, *g)] = fwhole;
     if (frest) c->v[kListFill0 + devplan_fill_class(frest, *g)] += 1;
     return true;
 }
@@ -319,8 +320,9 @@ __host__ __device__ inline BatchItem devplan_item(uint32_t list, uint32_t s, uin
     BatchItem it{};
     it.seg = s;
     if (list < kHistClasses) {
-        const uint32_t whole_items = list == kListHist0 ? (uint32_t)(g.n / t.hist_chunk) * g.m : 0u;
-        const uint32_t c = k < whole_items ? k / g.m : (uint32_t)(g.n / t.hist_chunk);
+        const uint32_t whole = g.n / (uint32_t)t.hist_chunk;
+        const uint32_t whole_items = list == kListHist0 ? whole * g.m : 0u;
+        const uint32_t c = k < whole_items ? k / g.m : whole;
         it.kind = kItemHist;
         it.a = (uint64_t)c * t.hist_chunk;
         it.b = ((uint64_t)c + 1) * t.hist_chunk < g.n ? ((uint64_t)c + 1) * t.hist_chunk : g.n;

@@ -6,11 +6,11 @@
 //
 // Each segment is still sorted by Algorithms 4-7 (Section 3); the plan is the
 // same three work lists as the host planner's (batch_api.cu), built by one
-// kernel: each CTA classifies 1024 segments (the rules of devplan_segment,
-// batched.h), scans their item counts per list, gets the counts of the
-// segments before its own from the CTAs before it (a decoupled lookback over
-// CTAs taken in start order, every wait bounded), and writes its segments'
-// descriptors and items.  The lists sit at fixed offsets (the bounds of the
+// kernel: eight CTAs each classify the same 1024 segments (the rules of
+// devplan_segment, batched.h), scan their item counts per list, get the counts
+// of the segments before from the CTAs before them (a decoupled lookback over
+// CTAs taken in start order, every wait bounded), and write an eighth of the
+// segments' descriptors and items each.  The lists sit at fixed offsets (the bounds of the
 // lists before them), so no CTA needs the totals to place its items; the
 // last CTA writes the lists' lengths.
 // The three launches then run over these lists (seg_*_kernel<true>); their
@@ -71,6 +71,13 @@ struct DevLook {
 static_assert(sizeof(DevLook) == 128, "lookback record is 32 words");
 constexpr uint32_t kLookWords = sizeof(DevLook) / 4;
 
+// CTAs of the planner per 1024 segments.  All of them classify the block's
+// segments; each writes a part of its descriptors and items (one SM's stores
+// would bound it: 1024 segments have about 100 KB of descriptors and 200 KB of
+// items: the planner takes 21 us for them with one CTA, 12 with four, 10 with
+// eight).
+constexpr uint32_t kPlanSplit = 8;
+
 __device__ __forceinline__ void st_release_u32(uint32_t *p, uint32_t v) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -84,7 +91,8 @@ __global__ void __launch_bounds__(1024) devplan_kernel(DevPlanArgs p) {
     __shared__ uint32_t s_ex[kNumLists][1024];  // exclusive prefix of each list's counts within the CTA
     __shared__ uint32_t s_warp[kNumLists][32];
     __shared__ uint32_t s_tot[kLookCounts], s_base[kLookCounts];
-    __shared__ uint32_t s_blk;
+    __shared__ uint32_t s_n[1024], s_R[1024];   // keys and range of the block's segments
+    __shared__ uint32_t s_ticket;
     __shared__ int s_bad;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     BatchCtl *ctl = reinterpret_cast<BatchCtl *>(p.ws + p.L.ctl);
@@ -93,18 +101,18 @@ __global__ void __launch_bounds__(1024) devplan_kernel(DevPlanArgs p) {
     DevLook *look = reinterpret_cast<DevLook *>(p.ws + p.L.look);
     // CTAs in start order, so a CTA only waits for CTAs already running.
     if (tid == 0) {
-        s_blk = atomicAdd(&ctl->plan_ticket, 1u);
+        s_ticket = atomicAdd(&ctl->plan_ticket, 1u);
         s_bad = 0;
     }
     __syncthreads();
-    const uint32_t blk = s_blk;
+    const uint32_t blk = s_ticket / kPlanSplit, sub = s_ticket % kPlanSplit;
     if (blk >= p.L.look_blocks) {
         // Only with a workspace whose ticket was not zero: the lists of this
         // run are incomplete, so the output launch must not trust them.
         if (tid == 0) atomicOr(&ctl->status, kDevTimeout);
         return;
     }
-    if (blk == 0 && tid == 0) {  // the previous run has finished (stream order)
+    if (blk == 0 && sub == 0 && tid == 0) {  // the previous run has finished (stream order)
         ctl->first_ticket = 0;
         ctl->scan_ticket = 0;
     }
@@ -145,8 +153,10 @@ __global__ void __launch_bounds__(1024) devplan_kernel(DevPlanArgs p) {
         // add the predecessors' until one has published its inclusive counts.
         uint32_t pre[kLookCounts] = {};
         if (blk > 0) {
-            for (int i = 0; i < kLookCounts; i++) look[blk].own[i] = s_tot[i];
-            st_release_u32(&look[blk].flag, 1u);
+            if (sub == 0) {
+                for (int i = 0; i < kLookCounts; i++) look[blk].own[i] = s_tot[i];
+                st_release_u32(&look[blk].flag, 1u);
+            }
             int64_t j = (int64_t)blk - 1;
             uint32_t spins = 0;
             while (j >= 0) {
@@ -169,12 +179,14 @@ __global__ void __launch_bounds__(1024) devplan_kernel(DevPlanArgs p) {
         }
         for (int i = 0; i < kLookCounts; i++) {
             s_base[i] = pre[i];
-            look[blk].incl[i] = pre[i] + s_tot[i];
+            if (sub == 0) look[blk].incl[i] = pre[i] + s_tot[i];
         }
-        st_release_u32(&look[blk].flag, 2u);
+        if (sub == 0) st_release_u32(&look[blk].flag, 2u);
     }
+    s_n[tid] = g.n;
+    s_R[tid] = g.R;
     __syncthreads();
-    if (s < S) {
+    if (s < S && tid / (1024 / kPlanSplit) == sub) {  // this CTA's part of the block's descriptors
         if (g.m > 0) {
             const size_t slot = p.L.slots + (size_t)s * p.L.slot_words;
             g.hist_off = slot;
@@ -187,23 +199,31 @@ __global__ void __launch_bounds__(1024) devplan_kernel(DevPlanArgs p) {
         }
         segs[s] = g;
     }
-    __syncthreads();  // the descriptors are read back below, by other threads of the CTA
-    // This CTA's items of every list, all threads together: the owner of the
-    // k-th is the last segment whose prefix is at most k.
+    // The block's items of every list, the threads of its CTAs together over all
+    // lists as one sequence: the owner of a list's k-th item is the last segment
+    // whose prefix is at most k.
     const uint32_t nseg = min(1024u, S - blk * 1024);
-    for (uint32_t f = 0; f < kNumLists; f++) {
-        for (uint32_t k = tid; k < s_tot[f]; k += 1024) {
-            uint32_t lo = 0, hi = nseg;
-            while (hi - lo > 1) {
-                const uint32_t mid = (lo + hi) >> 1;
-                if (s_ex[f][mid] <= k) lo = mid;
-                else hi = mid;
-            }
-            const uint32_t sg = blk * 1024 + lo;
-            items[devplan_pos(p.L.lb, f, (uint64_t)s_base[f] + k)] = devplan_item(f, sg, k - s_ex[f][lo], segs[sg], p.t);
+    uint32_t n_items = 0;
+#pragma unroll
+    for (uint32_t f = 0; f < kNumLists; f++) n_items += s_tot[f];
+    for (uint32_t i = sub * 1024 + tid; i < n_items; i += kPlanSplit * 1024) {
+        uint32_t f = 0, k = i;
+        while (k >= s_tot[f]) k -= s_tot[f++];
+        uint32_t lo = 0, hi = nseg;
+        while (hi - lo > 1) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (s_ex[f][mid] <= k) lo = mid;
+            else hi = mid;
         }
+        // What an item is made from, of the owner's descriptor.
+        BatchSeg o{};
+        o.n = s_n[lo];
+        o.R = s_R[lo];
+        o.m = (o.R + kBatchTileMax - 1) / kBatchTileMax;
+        o.fill_chunk = p.t.fill_chunk;
+        items[devplan_pos(p.L.lb, f, (uint64_t)s_base[f] + k)] = devplan_item(f, blk * 1024 + lo, k - s_ex[f][lo], o, p.t);
     }
-    if (blk == p.L.look_blocks - 1 && tid == 0) {
+    if (blk == p.L.look_blocks - 1 && sub == 0 && tid == 0) {
         uint32_t t[kLookCounts];
         for (int i = 0; i < kLookCounts; i++) t[i] = s_base[i] + s_tot[i];
         DevPlanHdr *h = reinterpret_cast<DevPlanHdr *>(p.ws + p.L.hdr);
@@ -421,7 +441,7 @@ rtcdf_status rtcdf_sort_batched_device_ws(const int32_t *in, int32_t *out, const
     p.t = tun;
     p.ws = ws;
     p.L = L;
-    devplan_kernel<<<L.look_blocks, 1024, 0, s>>>(p);
+    devplan_kernel<<<kPlanSplit * L.look_blocks, 1024, 0, s>>>(p);
     if (cudaGetLastError() != cudaSuccess) return RTCDF_ERR_CUDA;
     BatchArgs a;
     a.in = in;
