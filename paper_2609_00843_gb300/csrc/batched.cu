@@ -121,6 +121,13 @@ __device__ __forceinline__ void count_key_pred(uint32_t s_base, uint32_t y, uint
         ::"r"(y), "r"(w), "r"(s_base + 4u * y));
 }
 
+// What a CTA does beside an item: nothing, or (NextItem, below) fetching the next
+// one.  stage(0) comes once the item's counters are cleared, stage(1) once its
+// keys are counted.
+struct NoNext {
+    __device__ __forceinline__ void stage(int) {}
+};
+
 // ---------------------------------------------------------------- SMALL
 // One segment, n < 65536 keys, R <= kBatchSmallMaxR values, in one CTA.
 // WIDE: one 32-bit counter per value (R words).  Otherwise 16-bit counters,
@@ -128,13 +135,14 @@ __device__ __forceinline__ void count_key_pred(uint32_t s_base, uint32_t y, uint
 // v >= W in the high half of word v - W.
 // `sm` holds the counters, `s_tmp` the block scan's scratch (blockDim / 32 + 1
 // words).
-template <bool WIDE>
-__device__ void do_small_impl(const BatchArgs &a, const BatchSeg &g, uint32_t *sm, uint32_t *s_tmp) {
+template <bool WIDE, class Next>
+__device__ void do_small_impl(const BatchArgs &a, const BatchSeg &g, uint32_t *sm, uint32_t *s_tmp, Next &next) {
     const uint32_t R = g.R, n = g.n, nt = blockDim.x, tid = threadIdx.x;
     const uint32_t W = WIDE ? R : (R + 1) / 2;
     uint32_t *cnt = sm;
     for (uint32_t i = tid; i < W; i += nt) cnt[i] = 0;
     __syncthreads();
+    next.stage(0);
     const int32_t *in = a.in + g.off;
     const uint32_t min_u = (uint32_t)g.minVal;
     const uint32_t s_base = (uint32_t)__cvta_generic_to_shared(cnt);
@@ -167,6 +175,7 @@ __device__ void do_small_impl(const BatchArgs &a, const BatchSeg &g, uint32_t *s
     }
     if (tid < lead) count1(in[tid]);
     for (uint32_t i = lead + 4 * nv + tid; i < n; i += nt) count1(in[i]);
+    next.stage(1);
     __syncthreads();
     // In-place inclusive CDF over the counters (values <= n < 2^16).  Each
     // thread takes an odd number of consecutive values, so that the 32 lanes
@@ -260,10 +269,11 @@ __device__ void do_small_impl(const BatchArgs &a, const BatchSeg &g, uint32_t *s
 }
 
 // 32-bit counters when R of them fit in the `cap` words before s_tmp.
+template <class Next>
 __device__ __forceinline__ void do_small(const BatchArgs &a, const BatchSeg &g, uint32_t *sm, uint32_t cap,
-                                         uint32_t *s_tmp) {
-    if (g.R <= cap) do_small_impl<true>(a, g, sm, s_tmp);
-    else do_small_impl<false>(a, g, sm, s_tmp);
+                                         uint32_t *s_tmp, Next &next) {
+    if (g.R <= cap) do_small_impl<true>(a, g, sm, s_tmp, next);
+    else do_small_impl<false>(a, g, sm, s_tmp, next);
 }
 
 // ---------------------------------------------------------------- HIST
@@ -272,12 +282,14 @@ __device__ __forceinline__ void do_small(const BatchArgs &a, const BatchSeg &g, 
 // registers each).  Measured on the benchmark's segments: four vectors
 // loaded then counted 0.969 ms, eight 0.944 ms, sixteen spilled (1.09 ms),
 // pipelined four 0.939 ms, pipelined six 0.930 ms.
-__device__ void do_hist(const BatchArgs &a, const BatchSeg &g, const BatchItem &it, uint32_t *S) {
+template <class Next>
+__device__ void do_hist(const BatchArgs &a, const BatchSeg &g, const BatchItem &it, uint32_t *S, Next &next) {
     const uint32_t tid = threadIdx.x, nt = blockDim.x;
     const uint32_t b = it.tile * g.T;
     const uint32_t w = min(g.T, g.R - b);
     for (uint32_t i = tid; i < w; i += nt) S[i] = 0;
     __syncthreads();
+    next.stage(0);
     const uint32_t base = (uint32_t)g.minVal + b;
     const uint32_t s_base = (uint32_t)__cvta_generic_to_shared(S);
     const int32_t *in = a.in + g.off;
@@ -338,6 +350,7 @@ __device__ void do_hist(const BatchArgs &a, const BatchSeg &g, const BatchItem &
     if (tid < lead) count_key_pred(s_base, (uint32_t)in[k0 + tid] - base, w);
     for (uint64_t i = k0 + lead + 4 * nv + tid; i < k1; i += nt)
         count_key_pred(s_base, (uint32_t)in[i] - base, w);
+    next.stage(1);
     __syncthreads();
     uint32_t *H = a.ws_u32 + g.hist_off + b;
     if (g.single_hist) {
@@ -367,46 +380,115 @@ __device__ __forceinline__ DevListBounds dev_lb(const BatchArgs &a) {
     return DevListBounds{a.dev_bounds[0], a.dev_bounds[1], a.dev_bounds[2], a.dev_bounds[3], a.dev_bounds[4]};
 }
 
-__device__ __forceinline__ void first_item(const BatchArgs &a, uint32_t idx, uint32_t *sm) {
+template <class Next>
+__device__ __forceinline__ void first_item(const BatchArgs &a, const BatchItem &it, const BatchSeg &g, uint32_t *sm,
+                                           Next &next) {
     const unsigned long long t0 = (a.prof && threadIdx.x == 0) ? global_ns() : 0ull;
-    const BatchItem it = a.items[idx];
-    const BatchSeg g = a.segs[it.seg];
-    if (it.kind == kItemSmall) do_small(a, g, sm, kBatchSmallMaxR / 2, sm + kBatchSmallMaxR / 2);
-    else do_hist(a, g, it, sm);
+    const uint32_t kind = it.kind;
+    if (kind == kItemSmall) do_small(a, g, sm, kBatchSmallMaxR / 2, sm + kBatchSmallMaxR / 2, next);
+    else do_hist(a, g, it, sm, next);
     if (a.prof) {
         __syncthreads();
-        if (threadIdx.x == 0) prof_item(a, it.kind, t0, 0);
+        if (threadIdx.x == 0) prof_item(a, kind, t0, 0);
     }
 }
 
-// DEV: the lists were built on the device (their lengths are in
-// a.dev_counts) and the grid is a fixed number of CTAs that take items by
-// ticket; otherwise one CTA per item of the host-built plan.
+__device__ __forceinline__ void copy16_async(void *shared, const void *global) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(shared)),
+                 "l"(global)
+                 : "memory");
+}
+
+// The next item of a device-built first launch, fetched by thread 0 while the CTA
+// works on the current one: the ticket is drawn when that starts, the item copied
+// to shared memory once its counters are cleared, and its segment's descriptor
+// once its keys are counted -- three round trips that the CTA does not wait for
+// (4096 segments planned on the device 940 us against 960, 1024 288 against 291,
+// 700 the same).
+struct NextItem {
+    const BatchArgs &a;
+    const uint32_t *nc;  // lengths of the histogram lists
+    uint32_t n_small, total, ticket;
+    BatchItem *it;       // shared: the next item and its segment
+    BatchSeg *seg;
+
+    __device__ __forceinline__ void draw() {
+        if (threadIdx.x == 0) ticket = atomicAdd(&a.ctl->first_ticket, 1u);
+    }
+    __device__ __forceinline__ void stage(int s) {
+        if (threadIdx.x != 0 || ticket >= total) return;
+        if (s == 0) {
+            const BatchItem *src = a.items + devplan_first_pos(ticket, nc, n_small, dev_lb(a));
+            for (int i = 0; i < (int)sizeof(BatchItem) / 16; i++)
+                copy16_async(reinterpret_cast<uint4 *>(it) + i, reinterpret_cast<const uint4 *>(src) + i);
+        } else {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            const BatchSeg *src = a.segs + *reinterpret_cast<volatile uint32_t *>(&it->seg);
+            for (int i = 0; i < (int)sizeof(BatchSeg) / 16; i++)
+                copy16_async(reinterpret_cast<uint4 *>(seg) + i, reinterpret_cast<const uint4 *>(src) + i);
+        }
+    }
+};
+
+// kFirstHost: one CTA per item of the host-built plan.  Otherwise the lists were
+// built on the device (their lengths are in a.dev_counts) and the grid is a fixed
+// number of CTAs that take items by ticket: one at a time, or fetching the next
+// one ahead (with few items per CTA one drawn early waits behind a long one: 256
+// segments 139 us against 133).
 // One 1024-thread CTA per SM (the registers of a whole SM: 64 per thread):
 // with two per SM (32 registers per thread) the same items ran so much slower
 // that the segmented sort took 1.038 against 0.969 ms (host plan; the device-
 // planned form 1.12 against 1.035 ms), measured.  The shared memory stays at
 // kSegSmemBytes (a larger tile, 57344 bins in 224 KB, made it slower again).
-template <bool DEV>
+enum FirstMode { kFirstHost, kFirstTickets, kFirstAhead };
+template <int MODE>
 __global__ void __launch_bounds__(kSegThreads, 1) seg_first_kernel(BatchArgs a) {
     extern __shared__ uint32_t sm[];
     // The scan launch may be scheduled as soon as every CTA here has started;
     // it waits for this grid to finish before reading anything.
     asm volatile("griddepcontrol.launch_dependents;");
-    if (!DEV) {
-        first_item(a, blockIdx.x, sm);
+    if (MODE == kFirstHost) {
+        const BatchItem it = a.items[blockIdx.x];
+        const BatchSeg g = a.segs[it.seg];
+        NoNext none;
+        first_item(a, it, g, sm, none);
         return;
     }
-    __shared__ uint32_t s_idx;
-    const uint32_t n_hist = a.dev_counts[4], n_small1 = a.dev_counts[5];
+    const uint32_t n_small1 = a.dev_counts[5], total = a.dev_counts[4] + n_small1;
     const uint32_t nc[kHistClasses] = {a.dev_counts[6], a.dev_counts[7], a.dev_counts[8]};
-    for (;;) {
-        if (threadIdx.x == 0) s_idx = atomicAdd(&a.ctl->first_ticket, 1u);
-        __syncthreads();
-        const uint32_t k = s_idx;
-        __syncthreads();  // every thread has read s_idx (and the previous item's shared memory is free)
-        if (k >= n_hist + n_small1) break;
-        first_item(a, (uint32_t)devplan_first_pos(k, nc, n_small1, dev_lb(a)), sm);
+    if (MODE == kFirstTickets) {
+        __shared__ uint32_t s_idx;
+        for (;;) {
+            if (threadIdx.x == 0) s_idx = atomicAdd(&a.ctl->first_ticket, 1u);
+            __syncthreads();
+            const uint32_t k = s_idx;
+            __syncthreads();  // every thread has read s_idx (and the previous item's shared memory is free)
+            if (k >= total) break;
+            const BatchItem it = a.items[devplan_first_pos(k, nc, n_small1, dev_lb(a))];
+            const BatchSeg g = a.segs[it.seg];
+            NoNext none;
+            first_item(a, it, g, sm, none);
+        }
+        return;
+    }
+    __shared__ BatchItem s_it[2];
+    __shared__ BatchSeg s_seg[2];
+    __shared__ uint32_t s_more[2];
+    NextItem next{a, nc, n_small1, total, 0, &s_it[0], &s_seg[0]};
+    next.draw();
+    next.stage(0);
+    next.stage(1);
+    for (uint32_t cur = 0;; cur ^= 1) {
+        if (threadIdx.x == 0) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            s_more[cur] = next.ticket < total;
+        }
+        __syncthreads();  // the item is there (and the previous one's shared memory is free)
+        if (!s_more[cur]) break;
+        next.it = &s_it[cur ^ 1];
+        next.seg = &s_seg[cur ^ 1];
+        next.draw();
+        first_item(a, s_it[cur], s_seg[cur], sm, next);
     }
 }
 
@@ -582,7 +664,8 @@ __global__ void __launch_bounds__(kScanCtaThreads, 6) seg_scan_kernel(BatchArgs 
         const unsigned long long ts = (a.prof && tid == 0) ? global_ns() : 0ull;
         const BatchItem it = a.items[DEV ? devplan_pos(dev_lb(a), kListSmall2, i) : a.n_first + a.n_scan + i];
         const BatchSeg g = a.segs[it.seg];
-        do_small(a, g, s_buf, kScanSmemWords - 64, s_buf + kScanSmemWords - 64);
+        NoNext none;
+        do_small(a, g, s_buf, kScanSmemWords - 64, s_buf + kScanSmemWords - 64, none);
         if (a.prof) {
             __syncthreads();
             if (tid == 0) prof_item(a, kItemSmall, ts, 0);
@@ -869,7 +952,7 @@ cudaError_t launch_dep(const void *fn, uint32_t grid, int threads, const BatchAr
 cudaError_t launch_batched(const BatchArgs &args, cudaStream_t s) {
     BatchArgs a = args;
     a.fill_parts = fill_parts(a.n_fill);
-    cudaError_t e = cudaFuncSetAttribute(seg_first_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(seg_first_kernel<kFirstHost>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kSegSmemBytes);
     if (e != cudaSuccess) return e;
     // A launch is a programmatic dependent only of the plan's own launch
@@ -877,7 +960,7 @@ cudaError_t launch_batched(const BatchArgs &args, cudaStream_t s) {
     // the first launch issued waits for all earlier work in the stream.
     bool chained = false;
     if (a.n_first) {
-        seg_first_kernel<false><<<a.n_first, kSegThreads, kSegSmemBytes, s>>>(a);
+        seg_first_kernel<kFirstHost><<<a.n_first, kSegThreads, kSegSmemBytes, s>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         chained = true;
     }
@@ -896,13 +979,15 @@ cudaError_t launch_batched_dev(const BatchArgs &args, uint32_t first_ctas, uint3
                                cudaStream_t s) {
     BatchArgs a = args;
     a.fill_parts = fill_parts(fill_items);
-    cudaError_t e = cudaFuncSetAttribute(seg_first_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSegSmemBytes);
+    const void *first = a.num_segs < 700 ? (const void *)seg_first_kernel<kFirstTickets>
+                                         : (const void *)seg_first_kernel<kFirstAhead>;
+    cudaError_t e = cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSmemBytes);
     if (e != cudaSuccess) return e;
     // The first launch waits for the planner; every launch runs (the lists
     // may be empty), so that the tickets are consumed and reset in order.
-    seg_first_kernel<true><<<first_ctas, kSegThreads, kSegSmemBytes, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    void *first_args[] = {&a};
+    if ((e = cudaLaunchKernel(first, dim3(first_ctas), dim3(kSegThreads), first_args, kSegSmemBytes, s)) != cudaSuccess)
+        return e;
     e = launch_dep((const void *)seg_scan_kernel<true>, scan_ctas, kScanCtaThreads, a, true, s);
     if (e != cudaSuccess) return e;
     return launch_dep((const void *)seg_fill_kernel<true>, fill_items * a.fill_parts, kFillCtaThreads, a, true, s);
