@@ -23,8 +23,12 @@
 //
 // The fields leave the CTA as they are, 32 MB for R = 2^18, into the sort's
 // output buffer (which nothing reads before the output kernel fills it), and
-// pack_sum_kernel adds them up; without that scratch each CTA adds its fields
-// to H.
+// pack_sum_kernel adds them up.  Without that scratch the two CTAs of a cluster
+// add up their fields over distributed shared memory, half each, and the sums to
+// H: an SM passes on about 20 bytes of reductions a cycle, so its own counters,
+// 1 MB for R = 2^18, take it 28 us however many SMs there are, half of them 14
+// (n = 5e7, R = 2^18, histogram alone: 70 us against 78.5; clusters of four do not
+// fit all SMs: 119).
 //
 // Measured (n = 1e8, uniform / normal / one value, histogram of a sort, us; the
 // range tiles before that): R = 2^16 82 / 82 / 81 (92 / 92 / 85), 2^17 85 / 86 / 85
@@ -47,10 +51,25 @@ constexpr int kSampleVecs = 2;                      // vectors each thread sampl
 constexpr uint32_t kSampleKeys = kPackThreads * kSampleVecs * 4;
 constexpr uint32_t kHashBits = 14;                  // sample hash table, in the counters' shared memory
 constexpr uint32_t kCoarse = 256;                   // stretches of the range
+constexpr int kPackCluster = 2;                     // CTAs that add up their fields before H (without scratch)
 constexpr uint32_t kHotMin = 64;                    // sampled keys that make a key hot
 constexpr uint32_t kSingleNoise = 12;               // hash counts that uniform and normal keys reach
 
 __device__ __forceinline__ uint32_t sample_hash(uint32_t y) { return (y * 0x9E3779B1u) >> (32 - kHashBits); }
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
+// The word at `s_addr` of the cluster's CTA c.
+__device__ __forceinline__ uint32_t cluster_word(uint32_t s_addr, uint32_t c) {
+    uint32_t x;
+    asm volatile(
+        "{\n\t.reg .u32 r;\n\t"
+        "mapa.shared::cluster.u32 r, %1, %2;\n\t"
+        "ld.shared::cluster.u32 %0, [r];\n\t}"
+        : "=r"(x) : "r"(s_addr), "r"(c) : "memory");
+    return x;
+}
 
 }  // namespace
 
@@ -64,7 +83,6 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack_kernel(PackArgs a) {
     const int4 *vin = reinterpret_cast<const int4 *>(h.in + h.head);
     const uint64_t nvec = h.nvec;
     const uint32_t min_u = h.min_u, R = h.R;
-
 
     // ---- the sample
     for (uint32_t i = tid; i < (1u << kHashBits); i += kPackThreads) S[i] = 0;
@@ -245,19 +263,6 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack_kernel(PackArgs a) {
             __syncthreads();
             recount = s_diff != 0;
             if (!recount) hot_total += s_hot;
-            if (!recount && !dump) {
-                // Every CTA starts at another word, so that they do not meet.
-                const uint32_t rot = (uint32_t)((uint64_t)W * blockIdx.x / gridDim.x);
-                for (uint32_t i = tid; i < W; i += kPackThreads) {
-                    const uint32_t w = i + rot < W ? i + rot : i + rot - W;
-                    const uint32_t x = S[w];
-                    S[w] = 0;
-                    for (uint32_t f = 0, sh = 0; f < F; f++, sh += bits) {
-                        const uint32_t c = (x >> sh) & mask;
-                        if (c) atomicAdd(&h.H[f * W + w], c);
-                    }
-                }
-            }
             __syncthreads();
             if (tid == 0) s_diff = s_hot = 0;
         }
@@ -296,6 +301,38 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack_kernel(PackArgs a) {
             for (uint32_t i = tid; i < W / 4; i += kPackThreads) S4[i] = make_uint4(0, 0, 0, 0);
         }
         __syncthreads();
+        if (!dump) {
+            // The CTAs of a cluster add up their fields, each a share of the
+            // words, and every cluster starts at another word of the share, so
+            // that they do not meet.
+            constexpr uint32_t cs = kPackCluster;
+            const uint32_t rank = blockIdx.x % cs;
+            cluster_sync();
+            const uint32_t w0 = (uint32_t)((uint64_t)W * rank / cs), len = (uint32_t)((uint64_t)W * (rank + 1) / cs) - w0;
+            const uint32_t rot = (uint32_t)((uint64_t)len * blockIdx.x / gridDim.x);
+            constexpr int P = 4;
+            for (uint32_t i0 = tid; i0 < len; i0 += P * kPackThreads) {
+                uint32_t w[P], x[P][kPackCluster];
+#pragma unroll
+                for (int u = 0; u < P; u++) {
+                    const uint32_t i = i0 + u * kPackThreads;
+                    w[u] = w0 + (i + rot < len ? i + rot : i + rot - len);
+#pragma unroll
+                    for (int c = 0; c < kPackCluster; c++) x[u][c] = i < len ? cluster_word(s_base + 4 * w[u], c) : 0u;
+                }
+                for (uint32_t f = 0, sh = 0; f < F; f++, sh += bits)
+#pragma unroll
+                    for (int u = 0; u < P; u++) {
+                        uint32_t sum = 0;
+#pragma unroll
+                        for (int c = 0; c < kPackCluster; c++) sum += (x[u][c] >> sh) & mask;
+                        if (sum) atomicAdd(&h.H[f * W + w[u]], sum);
+                    }
+            }
+            cluster_sync();
+            for (uint32_t i = tid; i < W / 4; i += kPackThreads) S4[i] = make_uint4(0, 0, 0, 0);
+            __syncthreads();
+        }
     }
     asm volatile("griddepcontrol.launch_dependents;");
     if (has_hot && tid == 0 && hot_total) atomicAdd(&h.H[hot], hot_total);
@@ -359,7 +396,8 @@ bool pack_plan(uint64_t n, uint32_t R, uint64_t nvec, uintptr_t scratch, int sms
     // Expected keys of the fullest field that overflow with a chance below 1e-7
     // (Poisson tails).
     p->limit = fields == 2 ? 30000.f : fields == 4 ? 140.f : fields == 5 ? 24.f : fields == 6 ? 10.f : 2.5f;
-    p->ctas = (uint32_t)std::min<uint64_t>(sms, std::max<uint64_t>(1, nvec / (4 * kPackThreads)));
+    p->ctas = (uint32_t)std::min<uint64_t>(sms, nvec / (4 * kPackThreads)) / kPackCluster * kPackCluster;
+    if (p->ctas == 0) return false;
     // Range tiles: as few as 45056 values allow, and the trash word.
     p->m = (R + 45055) / 45056;
     p->tile = (R + p->m - 1) / p->m;
@@ -395,24 +433,29 @@ cudaError_t launch_pack(const PackPlan &p, const HistArgs &hist, uint32_t *copie
     void *args[] = {&a};
     cudaError_t e = cudaFuncSetAttribute(pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e != cudaSuccess) return e;
-    if ((e = cudaLaunchKernel((const void *)pack_kernel, dim3(p.ctas), dim3(kPackThreads), args, p.smem, s)) != cudaSuccess)
-        return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.blockDim = dim3(kPackThreads);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3(p.ctas);
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = a.dump ? 1 : kPackCluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    if ((e = cudaLaunchKernelExC(&cfg, (const void *)pack_kernel, args)) != cudaSuccess) return e;
     if (!a.dump) return cudaSuccess;
     const void *fn = p.fields == 2   ? (const void *)pack_sum_kernel<2>
                      : p.fields == 4 ? (const void *)pack_sum_kernel<4>
                      : p.fields == 5 ? (const void *)pack_sum_kernel<5>
                      : p.fields == 6 ? (const void *)pack_sum_kernel<6>
                                      : (const void *)pack_sum_kernel<8>;
-    cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((p.words / 4 + 15) / 16);
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 

@@ -215,9 +215,11 @@ rtcdf_status check_args(const int32_t *in, int32_t *out, uint64_t n) {
 
 // Histogram by packed counters (pack.cu) or by range tiles (hist.cu): one pass
 // over the input against one per tile, and about 10 us more (the sample and a
-// second launch; without scratch, the counters added to H by every CTA).
+// second launch; without scratch, the counters added to H by pairs of CTAs: packed
+// / tiles, us, n = 2e7, R = 200000, four tiles 46 / 48, 1.5e7 over 2^18, five, 46 /
+// 44, 4e7 over 100000, two, 50 / 58, 3.5e7 over 150000, three, 50 / 62).
 bool use_pack(uint64_t n, const Plan &pl, uintptr_t scratch, PackPlan *pp) {
-    if (pl.shape_given || pl.R <= 49152 || n * pl.m < (scratch ? 70000000u : 120000000u)) return false;
+    if (pl.shape_given || pl.R <= 49152 || n * pl.m < (scratch ? 70000000u : 80000000u)) return false;
     return pack_plan(n, pl.R, pl.nvec, scratch, pl.sms, pp);
 }
 

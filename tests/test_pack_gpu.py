@@ -85,3 +85,14 @@ def test_packed_histogram_reports_a_key_out_of_range(key):
     x[n - 5] = 3
     gpu_sort(x, 0, R, out)
     assert_matches_oracle(x, out, 0, R)
+
+
+# Pairs of CTAs add up their fields: every layout, and several rounds (normal keys).
+@pytest.mark.parametrize("R,n", [(49153, 45_000_001), (131071, 28_000_002), (163840, 21_000_003), (270336, 14_000_001),
+                                 (350_001, 60_000_000)])
+@pytest.mark.parametrize("dist", [gen.UNIFORM, gen.NORMAL])
+def test_packed_counts_of_every_layout_without_scratch(R, n, dist):
+    x = dev_keys(n, -5, R, dist, R)
+    counts = torch.zeros(R, dtype=torch.int32, device="cuda")
+    assert rtcdf.rtcdf_hist_accumulate(x.data_ptr(), n, -5, R - 5, counts.data_ptr(), stream_handle()) == rtcdf.OK
+    assert np.array_equal(counts.cpu().numpy(), np.bincount(x.cpu().numpy() + 5, minlength=R))
