@@ -30,7 +30,7 @@ __device__ __forceinline__ int next_run_after(const uint32_t *s_end, int lo, int
 }
 
 // Short runs: a warp's vectors [wb, we) (positions from `frame` on, four a
-// vector), `kBlock` positions at a time.  The warp writes the key of every run
+// vector), BLK positions at a time.  The warp writes the key of every run
 // that begins in the block to its first position in `m` (kBlock words of shared
 // memory, `none` elsewhere: no key of the array), reads it back as vectors and
 // carries the last key before it into every position without one: a ballot
@@ -42,30 +42,35 @@ __device__ __forceinline__ int next_run_after(const uint32_t *s_end, int lo, int
 // 107 / 94 (172 / 143; 134 MB of runs are read besides); n = 3e7, R = 1e6: 29 (57).
 constexpr int kBlock = 512;
 
-template <class Store>
+//
+// CDF: the table has an entry for every value (s_val unused, the first value's key
+// is none + 1); a value without keys, whose entry repeats the one before, begins
+// no run.
+template <bool CDF = false, int BLK = kBlock, class Store>
 __device__ __forceinline__ void fill_short_runs(uint32_t *m, const uint32_t *s_end, const int32_t *s_val, int nw,
                                                 uint32_t frame, uint32_t wb, uint32_t we, int32_t none, Store store) {
     const int lane = threadIdx.x & 31;
+    auto key = [&](int r) { return CDF ? (int32_t)((uint32_t)none + 1u + (uint32_t)r) : s_val[r]; };
     if (wb >= we) return;
     int4 *m4 = reinterpret_cast<int4 *>(m);
     int j = first_run_after(s_end, 0, nw - 1, frame + 4 * wb);  // the run of the block's first position
-    for (uint32_t w = wb; w < we; w += kBlock / 4) {
-        const uint32_t q0 = frame + 4 * w, q1 = min(q0 + kBlock, frame + 4 * we);
+    for (uint32_t w = wb; w < we; w += BLK / 4) {
+        const uint32_t q0 = frame + 4 * w, q1 = min(q0 + BLK, frame + 4 * we);
 #pragma unroll
-        for (int k = 0; k < kBlock / 128; k++) m4[lane + 32 * k] = make_int4(none, none, none, none);
-        int32_t carry = s_val[j];
+        for (int k = 0; k < BLK / 128; k++) m4[lane + 32 * k] = make_int4(none, none, none, none);
+        int32_t carry = key(j);
         __syncwarp();
         for (int r = j + 1 + lane;; r += 32) {
             const uint32_t start = r < nw ? s_end[r - 1] : 0xffffffffu;
             const bool begins = start < q1;
-            if (begins) m[start - q0] = (uint32_t)s_val[r];
+            if (begins && (!CDF || s_end[r] > start)) m[start - q0] = (uint32_t)key(r);
             const unsigned b = __ballot_sync(0xffffffffu, begins);
             j += __popc(b);
             if (b != 0xffffffffu) break;
         }
         __syncwarp();
 #pragma unroll
-        for (int k = 0; k < kBlock / 128; k++) {
+        for (int k = 0; k < BLK / 128; k++) {
             int4 x = m4[lane + 32 * k];
             const int32_t last = x.w != none ? x.w : x.z != none ? x.z : x.y != none ? x.y : x.x;
             const unsigned has = __ballot_sync(0xffffffffu, last != none);

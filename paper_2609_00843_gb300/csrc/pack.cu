@@ -308,7 +308,8 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack_kernel(PackArgs a) {
             constexpr uint32_t cs = kPackCluster;
             const uint32_t rank = blockIdx.x % cs;
             cluster_sync();
-            const uint32_t w0 = (uint32_t)((uint64_t)W * rank / cs), len = (uint32_t)((uint64_t)W * (rank + 1) / cs) - w0;
+            const uint32_t w0 = (uint32_t)((uint64_t)W * rank / cs);
+            const uint32_t len = (uint32_t)((uint64_t)W * (rank + 1) / cs) - w0;
             const uint32_t rot = (uint32_t)((uint64_t)len * blockIdx.x / gridDim.x);
             constexpr int P = 4;
             for (uint32_t i0 = tid; i0 < len; i0 += P * kPackThreads) {

@@ -30,7 +30,6 @@ namespace rtcdf {
 
 namespace {
 
-constexpr uint32_t kPartShift = 15;
 constexpr uint32_t kPartWidth = 1u << kPartShift;  // values per bucket
 constexpr int kPartThreads = 1024;
 constexpr uint32_t kPartSlabMax = 32768;           // keys per slab: 32 a thread, in registers
@@ -282,6 +281,11 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(PartArgs a) {
     const uint32_t t = tid < B ? s_keys[tid] : 0u;
     const uint32_t weight = t ? t / 16 + a.tile_cost : 0u;
     uint32_t total = 0, items = 0;
+    if (blockIdx.x == 0) {  // (for wide_out.cu)
+        const uint32_t end = block_incl(t, &total);
+        if (tid < B) a.bucket_start[tid + 1] = end;
+        if (tid == 0) a.bucket_start[0] = 0;
+    }
     block_incl(weight, &total);
     const uint32_t target = max(1u, total / a.target_items);
     const uint32_t incl = block_incl(t ? min(a.slabs, max(1u, t / 16 / target)) : 0u, &items);
@@ -434,9 +438,15 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(PartArgs a) {
         }
         __syncthreads();
         uint32_t *H = a.H + (size_t)b * kPartWidth;
+        uint32_t lower = 0;
         for (uint32_t i = tid; i < w; i += kBucketThreads) {
             const uint32_t c = S[i];
             if (c) atomicAdd(&H[i], c);
+            if (i < kPartWidth / 2) lower += c;
+        }
+        if (a.half) {
+            lower = __reduce_add_sync(0xffffffffu, lower);
+            if (lane == 0 && lower) atomicAdd(&a.half[b], lower);
         }
     }
     asm volatile("griddepcontrol.launch_dependents;");
@@ -471,7 +481,8 @@ bool part_plan(uint64_t n, uint32_t R, uint32_t head, uint64_t nvec, uintptr_t o
 }
 
 cudaError_t launch_part(const PartPlan &p, const int32_t *in, uint64_t n, uint32_t head, uint64_t nvec, uint32_t min_u,
-                        uint32_t R, uint32_t *H, Ctl *ctl, int sms, cudaStream_t s) {
+                        uint32_t R, uint32_t *H, uint32_t *bucket_start, uint32_t *half, Ctl *ctl, int sms,
+                        cudaStream_t s) {
     PartArgs a;
     a.in = in; a.n = n; a.nvec = nvec; a.head = head; a.min_u = min_u; a.R = R;
     a.buckets = p.buckets; a.slabs = p.slabs; a.slab_keys = p.slab_keys; a.slab_units = p.slab_units;
@@ -481,7 +492,7 @@ cudaError_t launch_part(const PartPlan &p, const int32_t *in, uint64_t n, uint32
     a.payload = reinterpret_cast<int4 *>(p.payload);
     a.starts = reinterpret_cast<uint16_t *>(p.starts);
     a.rows = reinterpret_cast<uint32_t *>(p.rows);
-    a.H = H; a.ctl = ctl;
+    a.H = H; a.bucket_start = bucket_start; a.half = half; a.ctl = ctl;
     void *args[] = {&a};
     const void *pf = p.buckets <= 64    ? (const void *)part_kernel<part_log_copies(64)>
                      : p.buckets <= 128 ? (const void *)part_kernel<part_log_copies(128)>

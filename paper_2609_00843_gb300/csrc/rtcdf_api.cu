@@ -233,9 +233,11 @@ bool use_part(uint64_t n, const Plan &pl, uintptr_t scratch, PartPlan *pp) {
 
 // Algorithm 5 (all tiles) into H (R counters).  H accumulates, so several calls
 // over slices of one array add up to the array's histogram.  ctl and scratch (n
-// words, 0 if there are none): of a whole sort.
+// words, 0 if there are none): of a whole sort, as bucket_start and half (or null)
+// of a histogram by partition, which *parted says was made.
 rtcdf_status hist_phase(const int32_t *in, uint64_t n, int64_t minVal, uint32_t R, const Plan &pl, uint32_t *H,
-                        Ctl *ctl, uintptr_t scratch, cudaStream_t s) {
+                        Ctl *ctl, uintptr_t scratch, uint32_t *bucket_start, uint32_t *half, bool *parted,
+                        cudaStream_t s) {
     HistArgs h;
     h.in = in; h.n = n; h.nvec = pl.nvec; h.head = pl.head;
     h.min_u = (uint32_t)(int32_t)minVal; h.R = R; h.T = pl.T; h.m = pl.m; h.g = pl.g;
@@ -245,12 +247,21 @@ rtcdf_status hist_phase(const int32_t *in, uint64_t n, int64_t minVal, uint32_t 
     cudaError_t e;
     if (use_pack(n, pl, scratch, &pack))
         e = launch_pack(pack, h, ctl && pack.dump ? &ctl->pack_copies : nullptr, s);
-    else if (ctl && use_part(n, pl, scratch, &part))
-        e = launch_part(part, in, n, pl.head, pl.nvec, h.min_u, R, H, ctl, pl.sms, s);
+    else if (ctl && (*parted = use_part(n, pl, scratch, &part)))
+        e = launch_part(part, in, n, pl.head, pl.nvec, h.min_u, R, H, bucket_start, half, ctl, pl.sms, s);
     else
         e = launch_hist(h, pl.hist_threads, pl.hist_smem, pl.streaming, s);
     return e == cudaSuccess ? RTCDF_OK : RTCDF_ERR_CUDA;
 }
+
+// After a histogram by partition: scan and output in one launch (wide_out.cu)
+// where the run table's way through memory is a large part of both, at few keys a
+// value, and there are enough tiles.  Whole sorts replayed from a graph, us, one
+// launch / two, uniform, normal and one value: n = 1e8, R = 2^24 423 412 306 / 506 482
+// 333; n = 1e6 81 79 43 / 111 109 73; n = 2e7, R = 2^20 90 96 73 / 102 106 76; n = 1.2e7
+// 67 70 55 / 72 75 55; beyond the lines, n = 5e7, R = 2^21 184 196 144 / 187 195 140;
+// n = 1e8, R = 2^20 302 331 248 / 287 307 236; n = 6e6, R = 7e5 47 51 40 / 50 56 38.
+bool use_wide_out(uint64_t n, uint32_t R) { return R >= 1000000 && n <= 20ull * R; }
 
 // Most positions that scan and output in one launch serve (small.cu).  Whole
 // sorts replayed from a graph, us, one launch / two, uniform keys over R = 128 and
@@ -313,9 +324,20 @@ rtcdf_status run_pipeline(const int32_t *in, int32_t *out, uint64_t n, int64_t m
         for (int i = 0; i < 4; i++) ev[i] = (cudaEvent_t)dbg->stage_events[i];
     if (ev[0] && cudaEventRecord(ev[0], s) != cudaSuccess) return RTCDF_ERR_CUDA;
     // (a sort in place has no scratch)
+    bool parted = false;
+    const bool wide = !dbg && !pl.fill_given && use_wide_out(n, R);
+    uint32_t *half = (uint32_t *)(base + L.scan_state) + 2 * kPartMaxBuckets;
     rtcdf_status st = hist_phase(in, n, minVal, R, pl, (uint32_t *)(base + L.hist), (Ctl *)(base + L.ctl),
-                                 in == out ? 0 : (uintptr_t)out, s);
+                                 in == out ? 0 : (uintptr_t)out, (uint32_t *)(base + L.start_run),
+                                 wide ? half : nullptr, &parted, s);
     if (st) return st;
+    if (parted && wide) {
+        WideOutArgs w;
+        w.H = (uint32_t *)(base + L.hist); w.out = out; w.n = (uint32_t)n; w.R = R;
+        w.min_u = (uint32_t)(int32_t)minVal; w.starts = (uint32_t *)(base + L.start_run);
+        w.half = half; w.read = (uint32_t *)(base + L.scan_state); w.ctl = (Ctl *)(base + L.ctl);
+        return launch_wide_out(w, pl.sms, s) == cudaSuccess ? RTCDF_OK : RTCDF_ERR_CUDA;
+    }
     if (ev[1] && cudaEventRecord(ev[1], s) != cudaSuccess) return RTCDF_ERR_CUDA;
     return finish_phase(out, n, minVal, R, pl, L, base, dbg, ev[2], ev[3], s, 0, n);
 }
@@ -423,7 +445,8 @@ rtcdf_status host_pipeline_hist(const int32_t *in, uint64_t n, int64_t minVal, u
     Plan pl;
     rtcdf_status st = make_plan(n, R, (uintptr_t)in, 0, nullptr, &pl);
     if (st) return st;
-    return hist_phase(in, n, minVal, R, pl, (uint32_t *)((char *)ws + ws_layout(R, ws_bytes).hist), nullptr, 0, s);
+    return hist_phase(in, n, minVal, R, pl, (uint32_t *)((char *)ws + ws_layout(R, ws_bytes).hist), nullptr, 0, nullptr,
+                      nullptr, nullptr, s);
 }
 
 rtcdf_status host_pipeline_finish(int32_t *out, uint64_t n, int64_t minVal, uint32_t R, void *ws,
@@ -535,7 +558,7 @@ rtcdf_status rtcdf_hist_accumulate(const int32_t *in, uint64_t n, int64_t minVal
     st = make_plan(n, R, (uintptr_t)in, 0, nullptr, &pl);
     if (st) return st;
     // Algorithm 5 for every tile, added straight into the caller's counts.
-    return hist_phase(in, n, minVal, R, pl, counts, nullptr, 0, (cudaStream_t)stream);
+    return hist_phase(in, n, minVal, R, pl, counts, nullptr, 0, nullptr, nullptr, nullptr, (cudaStream_t)stream);
 }
 
 rtcdf_status rtcdf_fill_from_counts(const uint32_t *counts, uint64_t total_n, int64_t minVal,

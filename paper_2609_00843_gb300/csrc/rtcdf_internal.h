@@ -156,6 +156,7 @@ bool pack_plan(uint64_t n, uint32_t R, uint64_t nvec, uintptr_t scratch, int sms
 cudaError_t launch_pack(const PackPlan &p, const HistArgs &hist, uint32_t *copies, cudaStream_t s);
 
 // ---------------------------------------------------------------- histogram by partition
+constexpr int kPartShift = 15;  // values per bucket, log2
 constexpr uint32_t kPartMaxBuckets = 512;
 
 struct PartArgs {
@@ -172,6 +173,8 @@ struct PartArgs {
     uint16_t *starts;      // per slab: buckets + 1 starts (units)
     uint32_t *rows;        // per CTA of part_kernel: its keys of each bucket
     uint32_t *H;           // global histogram, R entries (zero on entry)
+    uint32_t *bucket_start;  // written: keys before each bucket, buckets + 1
+    uint32_t *half;        // null, or added to: keys in the lower half of each bucket (zero on entry)
     Ctl *ctl;
 };
 struct PartPlan {
@@ -183,7 +186,21 @@ struct PartPlan {
 // false when they cannot hold it.
 bool part_plan(uint64_t n, uint32_t R, uint32_t head, uint64_t nvec, uintptr_t out_addr, int sms, PartPlan *p);
 cudaError_t launch_part(const PartPlan &p, const int32_t *in, uint64_t n, uint32_t head, uint64_t nvec, uint32_t min_u,
-                        uint32_t R, uint32_t *H, Ctl *ctl, int sms, cudaStream_t s);
+                        uint32_t R, uint32_t *H, uint32_t *bucket_start, uint32_t *half, Ctl *ctl, int sms,
+                        cudaStream_t s);
+
+// Scan and output after it in one launch.
+struct WideOutArgs {
+    uint32_t *H;           // R counts, zeroed
+    int32_t *out;
+    uint32_t n, R, min_u;
+    uint32_t buckets, tile_cost, target_items;  // (set by launch_wide_out)
+    const uint32_t *starts;  // keys before each bucket
+    uint32_t *half;        // keys in the lower half of each bucket, zeroed
+    uint32_t *read;        // per half bucket: items that have read its counts (zero between sorts)
+    Ctl *ctl;
+};
+cudaError_t launch_wide_out(const WideOutArgs &a, int sms, cudaStream_t s);
 
 // ---------------------------------------------------------------- scan
 struct ScanArgs {

@@ -118,3 +118,75 @@ def test_short_runs(R, n, dist, offset):
     gpu_sort(x, mn, mn + R, out[offset:offset + n])
     assert_matches_oracle(x, out[offset:offset + n], mn, mn + R)
     assert bool((out[:offset] == 5).all()) and bool((out[offset + n:] == 5).all())
+
+
+def _wide_shape(name, n, R):
+    g = torch.Generator("cuda")
+    g.manual_seed(R)
+    x = (torch.rand(n, device="cuda", generator=g, dtype=torch.float64) * R).int().clamp_(0, R - 1)
+    if name == "half":             # half of a tile's values: the most that its table leaves the others out for
+        x = x // 2 * 2
+    elif name == "one":
+        x.fill_(R - 1)
+    elif name == "ends":           # the first and last value of every tile, and long runs
+        x = (x // 16384 * 16384 + torch.where(x % 2 == 0, 0, 16383)).clamp_(max=R - 1)
+    elif name == "gap":            # a long run and a few keys: most tiles empty
+        x = torch.where(x % 1000 == 0, x, R // 3)
+    return x.int()
+
+
+# Scan and output in one launch: the narrowest and widest range, tiles of 16384
+# values with a last one of a single value, whole and absent, the most keys a
+# value and one more, few keys; against the oracle and against the launches of
+# the general path (which explicit parameters select).
+@pytest.mark.parametrize("R,n", [(999_999, 3_000_001), (1_000_000, 20_000_000), (1_000_000, 20_000_001), (31 * 32768 + 1, 2_800_002),
+                                 (31 * 32768 + 16384, 2_900_003), (31 * 32768 + 16385, 2_900_001), (1 << 22, 5_000_002),
+                                 (1 << 24, 200_003), (1 << 24, 30_000_001)])
+@pytest.mark.parametrize("shape", ["uniform", "half", "one", "ends", "gap"])
+def test_scan_and_output_of_a_wide_range(R, n, shape):
+    mn, k = -(1 << 31), n % 4
+    x = _wide_shape(shape, n, R) + mn
+    out = torch.full((n + 8,), 5, dtype=torch.int32, device="cuda")
+    gpu_sort(x, mn, mn + R, out[k:k + n])
+    assert_matches_oracle(x, out[k:k + n], mn, mn + R)
+    assert bool((out[:k] == 5).all()) and bool((out[k + n:] == 5).all())
+    s, wsb = stream_handle(), rtcdf.rtcdf_workspace_size(R)
+    ws = torch.zeros(wsb // 4, dtype=torch.int32, device="cuda")
+    general = torch.empty_like(x)
+    for params, dst in ((rtcdf.Params(), general), (None, out[k:k + n]), (rtcdf.Params(), general)):
+        dst.fill_(0)               # one workspace for both, in turn
+        assert rtcdf.rtcdf_sort_ex(x.data_ptr(), dst.data_ptr(), n, mn, mn + R, params, ws.data_ptr(), wsb, None, s) == rtcdf.OK
+    assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
+    assert torch.equal(general, out[k:k + n])
+
+
+# Keys past the last value: in its tile, in the bucket's other half, beyond.
+@pytest.mark.parametrize("R", [31 * 32768 + 7, 31 * 32768 + 16384, 31 * 32768 + 20_000, 31 * 32768])
+@pytest.mark.parametrize("past", [0, 16_383, 16_384, 40_000])
+def test_wide_output_reports_a_key_past_the_range(R, past):
+    n, s = 3_000_000, stream_handle()
+    x = dev_keys(n, 0, R, gen.UNIFORM, 14)
+    x[17] = R + past
+    out = torch.empty_like(x)
+    assert rtcdf.rtcdf_sort(x.data_ptr(), out.data_ptr(), n, 0, R, s) == rtcdf.OK
+    assert rtcdf.rtcdf_status_get(s) == (rtcdf.ERR_KEY_OUT_OF_RANGE, rtcdf.DEV_KEY_OUT_OF_RANGE)
+    want = torch.cat([x[:17], x[18:]]).sort().values
+    assert torch.equal(out[:n - 1], want)
+    x[17] = 0
+    gpu_sort(x, 0, R, out)
+    assert_matches_oracle(x, out, 0, R)
+
+
+def test_wide_output_reports_a_stray_ticket():
+    n, R, s = 300_000, 1 << 24, stream_handle()  # (more tiles than CTAs)
+    x = dev_keys(n, 0, R, gen.UNIFORM, 15)
+    out = torch.empty_like(x)
+    wsb = rtcdf.rtcdf_workspace_size(R)
+    ws = torch.zeros(wsb // 4, dtype=torch.int32, device="cuda")
+    ws[1] = 2                      # control block word 1: the scan's ticket
+    assert rtcdf.rtcdf_sort_ws(x.data_ptr(), out.data_ptr(), n, 0, R, ws.data_ptr(), wsb, s) == rtcdf.OK
+    assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.ERR_TIMEOUT, rtcdf.DEV_TIMEOUT)
+    ws.zero_()
+    assert rtcdf.rtcdf_sort_ws(x.data_ptr(), out.data_ptr(), n, 0, R, ws.data_ptr(), wsb, s) == rtcdf.OK
+    assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
+    assert_matches_oracle(x, out, 0, R)
