@@ -19,8 +19,8 @@
 // place has none and keeps the range-tile kernel.
 //
 // Measured (n = 1e8, uniform / normal / one value, both kernels, us; the range
-// tiles before that): R = 2^19 214 / 225 / 167 (459 / 424 / 400), 2^20 220 / 237 / 172
-// (771 / 777 / 717), 2^22 287 / 273 / 198 (2394 / 2699 / 2718), 2^24 335 / 329 / 246
+// tiles before that): R = 2^19 214 / 225 / 167 (459 / 424 / 400), 2^20 218 / 236 / 170
+// (771 / 777 / 717), 2^22 282 / 269 / 201 (2394 / 2699 / 2718), 2^24 340 / 333 / 249
 // (8144 / 8353 / 9810).
 #include <algorithm>
 
@@ -44,9 +44,11 @@ constexpr uint32_t kPartTileKeys = 32768;
 static_assert(RTCDF_MAX_R >> kPartShift == kPartMaxBuckets, "buckets of the widest range");
 
 // Counters per bucket, log2: lane l of a warp counts in copy l mod copies.
-// With 32 copies (up to 64 buckets) the lanes of a warp never meet in a bank or
-// on a word, whatever the keys; more buckets spread the lanes by themselves.
-__host__ __device__ constexpr int part_log_copies(uint32_t B) { return B <= 64 ? 5 : B <= 128 ? 4 : 3; }
+// With 32 copies (up to 128 buckets) the lanes of a warp never meet in a bank or
+// on a word, whatever the keys.  With more buckets the passes over the counters
+// cost as much as the conflicts they save (n = 1e8, part_kernel, us, 8 / 16 / 32
+// copies: 512 buckets 195 / 194 / 222, 256 187 / 175 / 182, 128 180 / 167 / 162).
+__host__ __device__ constexpr int part_log_copies(uint32_t B) { return B <= 128 ? 5 : 4; }
 
 // Words of part_kernel's shared memory before the staged slab (which starts on
 // 128 bytes, see stage_slot).
@@ -494,9 +496,8 @@ cudaError_t launch_part(const PartPlan &p, const int32_t *in, uint64_t n, uint32
     a.rows = reinterpret_cast<uint32_t *>(p.rows);
     a.H = H; a.bucket_start = bucket_start; a.half = half; a.ctl = ctl;
     void *args[] = {&a};
-    const void *pf = p.buckets <= 64    ? (const void *)part_kernel<part_log_copies(64)>
-                     : p.buckets <= 128 ? (const void *)part_kernel<part_log_copies(128)>
-                                        : (const void *)part_kernel<part_log_copies(512)>;
+    const void *pf = p.buckets <= 128 ? (const void *)part_kernel<part_log_copies(128)>
+                                      : (const void *)part_kernel<part_log_copies(512)>;
     cudaError_t e = cudaFuncSetAttribute(pf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e != cudaSuccess) return e;
     if ((e = cudaLaunchKernel(pf, dim3(p.ctas), dim3(kPartThreads), args, p.smem, s)) != cudaSuccess) return e;
