@@ -84,6 +84,13 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack_kernel(PackArgs a) {
     const uint64_t nvec = h.nvec;
     const uint32_t min_u = h.min_u, R = h.R;
 
+    // After a wait that ran out nothing is written to the output (nor to its
+    // use as scratch) until the status has been read.
+    if (a.dump && (a.ctl->status & kDevTimeout)) {
+        if (blockIdx.x == 0 && tid == 0) a.ctl->pack_copies = 0;
+        return;
+    }
+
     // ---- the sample
     for (uint32_t i = tid; i < (1u << kHashBits); i += kPackThreads) S[i] = 0;
     if (tid < kCoarse) s_coarse[tid] = 0;
@@ -174,7 +181,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack_kernel(PackArgs a) {
     const float want = ceilf(fullest / a.limit);
     const bool tiles = want > (float)a.max_rounds || (int)s_near > (int)(kSampleVecs * kPackThreads / 16);
     const uint32_t rounds = tiles ? 0u : max(1u, (uint32_t)want);
-    if (blockIdx.x == 0 && tid == 0 && a.dump) *a.copies = rounds * gridDim.x;
+    if (blockIdx.x == 0 && tid == 0 && a.dump) a.ctl->pack_copies = rounds * gridDim.x;
     if (tiles) {
         if (blockIdx.x < h.m * h.g) hist_tiles<false, 8, true>(h, blockIdx.x, S, s_tc);
         return;
@@ -349,7 +356,7 @@ __global__ void __launch_bounds__(256) pack_sum_kernel(PackArgs a) {
     const uint32_t q = blockIdx.x * 16 + l, quads = a.words / 4;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
-    const uint32_t copies = *a.copies;
+    const uint32_t copies = a.ctl->pack_copies;
     if (copies == 0) return;
     uint32_t acc[F][4] = {};
     if (q < quads) {
@@ -422,15 +429,15 @@ bool pack_plan(uint64_t n, uint32_t R, uint64_t nvec, uintptr_t scratch, int sms
     return true;
 }
 
-cudaError_t launch_pack(const PackPlan &p, const HistArgs &hist, uint32_t *copies, cudaStream_t s) {
+cudaError_t launch_pack(const PackPlan &p, const HistArgs &hist, Ctl *ctl, cudaStream_t s) {
     PackArgs a;
     a.h = hist;
     a.h.T = p.tile; a.h.m = p.m; a.h.g = p.g;
     a.words = p.words; a.fields = p.fields; a.magic = p.magic; a.limit = p.limit; a.max_rounds = p.max_rounds;
     a.coarse_shift = 0;
     while (((hist.R - 1) >> a.coarse_shift) >= kCoarse) a.coarse_shift++;
-    a.dump = copies ? reinterpret_cast<uint32_t *>(p.dump) : nullptr;
-    a.copies = copies;
+    a.dump = ctl ? reinterpret_cast<uint32_t *>(p.dump) : nullptr;
+    a.ctl = ctl;
     void *args[] = {&a};
     cudaError_t e = cudaFuncSetAttribute(pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e != cudaSuccess) return e;

@@ -246,7 +246,7 @@ rtcdf_status hist_phase(const int32_t *in, uint64_t n, int64_t minVal, uint32_t 
     PartPlan part;
     cudaError_t e;
     if (use_pack(n, pl, scratch, &pack))
-        e = launch_pack(pack, h, ctl && pack.dump ? &ctl->pack_copies : nullptr, s);
+        e = launch_pack(pack, h, ctl, s);
     else if (ctl && (*parted = use_part(n, pl, scratch, &part)))
         e = launch_part(part, in, n, pl.head, pl.nvec, h.min_u, R, H, bucket_start, half, ctl, pl.sms, s);
     else

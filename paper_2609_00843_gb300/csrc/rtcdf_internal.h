@@ -140,8 +140,8 @@ struct PackArgs {
     uint32_t coarse_shift; // the sample's stretches of the range
     float limit;           // expected keys of the fullest field in a round
     uint32_t max_rounds;
-    uint32_t *dump;        // written-out counters, or null: added to H by each CTA
-    uint32_t *copies;
+    uint32_t *dump;        // written-out counters, or null: added to H by pairs of CTAs
+    Ctl *ctl;              // (with dump)
 };
 struct PackPlan {
     uint32_t words, fields, magic, max_rounds, ctas, tile, m, g;
@@ -152,8 +152,8 @@ struct PackPlan {
 // The plan for n keys over R values; scratch: n words, or 0.  False when the
 // range does not fit.
 bool pack_plan(uint64_t n, uint32_t R, uint64_t nvec, uintptr_t scratch, int sms, PackPlan *p);
-// copies: a word of the workspace, or null for no scratch.
-cudaError_t launch_pack(const PackPlan &p, const HistArgs &hist, uint32_t *copies, cudaStream_t s);
+// ctl: the control block of a whole sort, or null (no scratch).
+cudaError_t launch_pack(const PackPlan &p, const HistArgs &hist, Ctl *ctl, cudaStream_t s);
 
 // ---------------------------------------------------------------- histogram by partition
 constexpr int kPartShift = 15;  // values per bucket, log2

@@ -96,3 +96,18 @@ def test_packed_counts_of_every_layout_without_scratch(R, n, dist):
     counts = torch.zeros(R, dtype=torch.int32, device="cuda")
     assert rtcdf.rtcdf_hist_accumulate(x.data_ptr(), n, -5, R - 5, counts.data_ptr(), stream_handle()) == rtcdf.OK
     assert np.array_equal(counts.cpu().numpy(), np.bincount(x.cpu().numpy() + 5, minlength=R))
+
+
+def test_nothing_is_written_while_a_timeout_is_unread():
+    n, R, s = 20_000_000, 1 << 18, stream_handle()
+    x = dev_keys(n, 0, R, gen.UNIFORM, 16)
+    out = torch.full_like(x, -7)
+    wsb = rtcdf.rtcdf_workspace_size(R)
+    ws = torch.zeros(wsb // 4, dtype=torch.int32, device="cuda")
+    ws[0] = rtcdf.DEV_TIMEOUT                    # control block word 0: the status
+    assert rtcdf.rtcdf_sort_ws(x.data_ptr(), out.data_ptr(), n, 0, R, ws.data_ptr(), wsb, s) == rtcdf.OK
+    assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s)[0] == rtcdf.ERR_TIMEOUT
+    assert bool((out == -7).all())
+    assert rtcdf.rtcdf_sort_ws(x.data_ptr(), out.data_ptr(), n, 0, R, ws.data_ptr(), wsb, s) == rtcdf.OK
+    assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
+    assert_matches_oracle(x, out, 0, R)
