@@ -253,6 +253,7 @@ __global__ void __launch_bounds__(1024) devplan_kernel(DevPlanArgs p) {
 struct BatchCache {
     void *ptr = nullptr;
     size_t bytes = 0;
+    DevBounds used{0, 0, 0};  // of the last sort in it (S = 0: none since it was cleared)
 };
 std::mutex g_bmu;
 std::map<std::pair<int, cudaStream_t>, BatchCache> g_bws;
@@ -265,7 +266,8 @@ rtcdf_status check_bounds(int32_t S, uint64_t N, int64_t max_R, DevBounds *b) {
     return RTCDF_OK;
 }
 
-rtcdf_status grow_cache(cudaStream_t s, size_t need, void **ptr, size_t *bytes) {
+// next: the bounds of the sort that will use it, or null.
+rtcdf_status grow_cache(cudaStream_t s, size_t need, const DevBounds *next, void **ptr, size_t *bytes) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return RTCDF_ERR_CUDA;
     std::lock_guard<std::mutex> lk(g_bmu);
@@ -288,7 +290,18 @@ rtcdf_status grow_cache(cudaStream_t s, size_t need, void **ptr, size_t *bytes) 
         void *old = c->ptr;
         c->ptr = p;
         c->bytes = need;
+        c->used = DevBounds{0, 0, 0};
         if (old && cudaFreeAsync(old, s) != cudaSuccess) return RTCDF_ERR_CUDA;
+    }
+    if (next) {
+        // Other bounds lay the workspace out in another way: what must be zero
+        // there holds lists and run tables of the last sort.  (All but the status
+        // word at its start.)
+        const DevBounds &u = c->used;
+        if (u.S && (u.S != next->S || u.max_R != next->max_R || u.max_total_keys != next->max_total_keys) &&
+            cudaMemsetAsync((char *)c->ptr + 4, 0, need - 4, s) != cudaSuccess)
+            return RTCDF_ERR_CUDA;
+        c->used = *next;
     }
     *ptr = c->ptr;
     *bytes = c->bytes;
@@ -483,7 +496,7 @@ rtcdf_status rtcdf_batch_reserve(int32_t num_segments, uint64_t max_total_keys, 
     if (st) return st;
     void *ws = nullptr;
     size_t bytes = 0;
-    return grow_cache((cudaStream_t)stream, std::max<size_t>(need, 256), &ws, &bytes);
+    return grow_cache((cudaStream_t)stream, std::max<size_t>(need, 256), nullptr, &ws, &bytes);
 } catch (...) {
     return RTCDF_ERR_NO_MEMORY;
 }
@@ -498,7 +511,8 @@ rtcdf_status rtcdf_sort_batched(const int32_t *in, int32_t *out, const int64_t *
     if (!in || !out || !seg_offsets || !seg_minVal || !seg_maxVal) return RTCDF_ERR_INVALID_ARG;
     void *ws = nullptr;
     size_t bytes = 0;
-    st = grow_cache((cudaStream_t)stream, std::max<size_t>(need, 256), &ws, &bytes);
+    const DevBounds next{(uint32_t)num_segments, (uint32_t)max_R, max_total_keys};
+    st = grow_cache((cudaStream_t)stream, std::max<size_t>(need, 256), &next, &ws, &bytes);
     if (st) return st;
     return rtcdf_sort_batched_device_ws(in, out, seg_offsets, seg_minVal, seg_maxVal, num_segments,
                                         max_total_keys, max_R, ws, bytes, stream);

@@ -369,3 +369,23 @@ def test_lists_longer_than_the_scan_grid():
     for s in list(np.nonzero(L == 70_000)[0]) + list(range(0, S, 997)):
         lo, hi = int(offs[s]), int(offs[s + 1])
         np.testing.assert_array_equal(b[lo:hi], oracle.counting_sort(a[lo:hi], int(mns[s]), int(mxs[s])))
+
+
+def test_library_workspace_with_other_bounds():
+    # The workspace is laid out by the bounds: each call finds what must be zero
+    # zeroed, whatever the bounds of the call before.
+    s = stream_handle()
+    m = MIXED
+    many = dict(lengths=[2000 + 7 * i for i in range(300)], Rs=[4096 - i for i in range(300)], mins=[-i for i in range(300)],
+                dists=[i % 3 for i in range(300)])
+    for shape, max_R, more in ((m, 1 << 20, 0), (many, 4096, 0), (many, 5000, 70_000), (m, 1 << 20, 0)):
+        x, offs, mn, mx = make_layout(shape["lengths"], shape["Rs"], shape["mins"], shape["dists"],
+                                      range(1, 1 + len(shape["lengths"])), cap=sum(shape["lengths"]) + more)
+        out = torch.full_like(x, 0x7FFFFFFF)
+        d_o, d_mn, d_mx = to_dev(offs), to_dev(mn), to_dev(mx)
+        for _ in range(2):
+            rc = rtcdf.rtcdf_sort_batched(x.data_ptr(), out.data_ptr(), d_o.data_ptr(), d_mn.data_ptr(),
+                                          d_mx.data_ptr(), len(mn), x.numel(), max_R, s)
+            assert rc == rtcdf.OK, rtcdf.rtcdf_status_str(rc)
+        assert rtcdf.rtcdf_status_get(s) == (rtcdf.OK, 0)
+        check_segments(x, out, offs, mn, mx)
