@@ -159,6 +159,12 @@ def code_sha256(src_files) -> str:
     return h.hexdigest()
 
 
+def hist_form(R: int) -> str:
+    """Form of the histogram of a sweep array (n = 1e8): up to 49152 values one
+    shared-memory tile (a sort is three launches), above packed counters (four)."""
+    return "1" if R <= 49152 else "packed"
+
+
 def traffic_for(kernel: str, src_files):
     """DRAM bytes per launch of `kernel` on the sweep arrays, averaged over the
     ncu captures committed in profiles/ncu_traffic.json -- only if they were
@@ -940,15 +946,14 @@ def main():
         ksrc = ["paper_2609_00843_gb300/csrc/fill.cu", "paper_2609_00843_gb300/csrc/rtcdf_internal.h"]
     avg_launch_s = ktime / launches * 1e-3
     achieved = 4 * n / avg_launch_s / 1e9  # algorithmic: 4n bytes read (hist) or written (fill)
-    # The same fraction split by the number of range tiles m of the launch
-    # (one tile streams the input once; m > 1 tiles re-read it from L2).
+    # The same fraction split by the form of the histogram: one shared-memory
+    # tile, or packed counters (pack_kernel and pack_sum_kernel).
     j = 0 if kname == "hist_kernel" else 2
     by_tiles = {}
     for i, c in enumerate(cases):
-        m = -(-c["R"] // rtcdf.rtcdf_plan(n, c["R"]).tile_width)
-        by_tiles.setdefault(m, []).append(stage_ms[i][j] / nsteps)
-    by_tiles = {str(m): {"launches_per_step": len(t),
-                         "frac": round(4 * n / (sum(t) / len(t) * 1e-3) / 1e9 / hbm, 4)}
+        by_tiles.setdefault(hist_form(c["R"]), []).append(stage_ms[i][j] / nsteps)
+    by_tiles = {m: {"arrays_per_step": len(t),
+                    "frac": round(4 * n / (sum(t) / len(t) * 1e-3) / 1e9 / hbm, 4)}
                 for m, t in sorted(by_tiles.items())}
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
                 "frac": round(achieved / hbm, 4),
@@ -976,7 +981,7 @@ def main():
         "whole_sort_roofline": whole,
         "per_config": per_config,
         "clocks": clocks,
-        "gpu_launches": 3 * len(cases) * args.steps,
+        "gpu_launches": sum(4 if hist_form(c["R"]) == "packed" else 3 for c in cases) * args.steps,
         "timed_region_ms": round(total_ms, 3),
     }
 

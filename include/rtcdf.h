@@ -410,8 +410,8 @@ rtcdf_status rtcdf_sort_batched_host(const int32_t *in, int32_t *out, const int6
  * (S+1 entries, nondecreasing, seg_offsets[0] >= 0), seg_minVal and
  * seg_maxVal (S entries), 8-byte aligned.  Each segment s is sorted as in the
  * plan API (Section 2.1's problem per segment, Algorithms 4-7).  The work
- * lists are built on the device by two planner kernels, so the call enqueues
- * five launches and returns: asynchronous, stream-ordered, no host
+ * lists are built on the device by a planner kernel, so the call enqueues
+ * four launches and returns: asynchronous, stream-ordered, no host
  * synchronisation.
  *
  * The caller states bounds the metadata must keep: num_segments (S),

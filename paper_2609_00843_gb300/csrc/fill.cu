@@ -13,7 +13,8 @@
 // the common case -- that is one shared load and one compare before the
 // store; a vector across runs reads the next runs' ends independently.  The
 // few positions of a window that do not fill a whole aligned vector are
-// written one by one.
+// written one by one.  Windows of short runs are filled from the runs' first
+// positions instead (fill_runs.cuh).
 //
 // All positions are below n < 2^32, so the index arithmetic is 32-bit.  The
 // CTA also clears the scan's lookback state so the workspace is ready for the
@@ -22,10 +23,10 @@
 
 namespace rtcdf {
 
-// Runs per shared-memory window: four per thread (eight for short runs), so that a CTA whose
-// positions cross thousands of short runs (the tails of a peaked distribution
-// over a wide range) needs few window rounds -- each round costs a global
-// round trip and two barriers.
+// Runs per shared-memory window: four per thread (eight for short runs), so that a
+// CTA whose positions cross thousands of short runs (the tails of a peaked
+// distribution over a wide range) needs few window rounds -- each round costs a
+// global round trip and two barriers.
 template <int WIN, bool SHORT>
 constexpr int kRunWindow = SHORT && WIN < 1024 ? 8 * WIN : 4 * WIN;
 

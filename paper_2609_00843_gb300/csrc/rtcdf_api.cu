@@ -1,13 +1,18 @@
 // Host side of the C ABI (include/rtcdf.h): argument checks, launch planning,
-// workspace management and the three-kernel pipeline of Algorithm 4.
+// workspace management and the pipeline of Algorithm 4.
 //
-//   1. hist  -- Algorithm 5 for all m tiles in one launch
-//   2. scan  -- local CDFs + tile offsets (Algorithm 6) as one lookback scan
-//   3. fill  -- Algorithm 7 for all tiles in one launch
+//   1. histogram -- Algorithm 5: one shared-memory tile or several (hist.cu), packed
+//                   counters for ranges of a few tiles (pack.cu), by partition for
+//                   wider ones (part.cu)
+//   2. scan      -- local CDFs + tile offsets (Algorithm 6) as one scan (scan.cu)
+//   3. output    -- Algorithm 7 for all tiles in one launch (fill.cu)
+//
+// 2 and 3 are one launch over narrow ranges (small.cu) and over wide ones with few
+// keys a value (wide_out.cu), and a small array takes one launch in all (small.cu).
 //
 // Unlike the paper's host driver there is no device-to-host copy of the tile
 // offsets and no per-tile launch loop: every launch size is known from (n, R)
-// alone, so a sort is three stream-ordered launches with no host
+// alone, so a sort is one to four stream-ordered launches with no host
 // synchronisation and can be captured in a CUDA graph.
 #include <algorithm>
 #include <cstring>

@@ -1,8 +1,8 @@
 // Sorts over narrow ranges with fewer launches.
 //
-// small_kernel: a whole sort in one CTA, for arrays of a few ten thousand keys over a narrow
-// range: histogram (Algorithm 5), local CDF and runs (Algorithm 6) and output
-// (Algorithm 7) in shared memory, with nothing but the status word in the
+// small_kernel: a whole sort in one CTA, for arrays of a few ten thousand keys over
+// a narrow range: histogram (Algorithm 5), local CDF and runs (Algorithm 6) and
+// output (Algorithm 7) in shared memory, with nothing but the status word in the
 // workspace.
 //
 // What bounds such a sort is its chain of dependent steps, and as three launches
