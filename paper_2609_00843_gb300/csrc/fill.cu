@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(WIN) fill_kernel(FillArgs a) {
 
     // Programmatic dependent of the scan: wait for its results.
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
     for (uint32_t i = c * WIN + tid; i < a.scan_chunks; i += a.fill_ctas * WIN) a.scan_state[i] = 0;
     if (c == 0 && tid == 0) a.ctl->scan_ticket = a.ctl->part_ticket = 0;
 

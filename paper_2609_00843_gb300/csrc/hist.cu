@@ -57,13 +57,13 @@ const void *hist_fn(int variant, int unroll) {
 // the 2-to-8-tile form.
 int hist_unroll(size_t smem) { return smem > 114 * 1024 ? 8 : 4; }
 
-cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool streaming,
-                        cudaStream_t s) {
+cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool streaming, bool first, cudaStream_t s) {
     // hist_max_ctas_per_sm() has raised the shared-memory limit for this size.
     dim3 grid(a.m * a.g);
     void *args[] = {const_cast<HistArgs *>(&a)};
-    return cudaLaunchKernel(hist_fn(hist_variant(streaming, a.m), hist_unroll(smem)), grid, dim3(threads),
-                            args, smem, s);
+    const void *fn = hist_fn(hist_variant(streaming, a.m), hist_unroll(smem));
+    if (streaming && first) return launch_first(fn, grid.x, threads, smem, args, s);
+    return cudaLaunchKernel(fn, grid, dim3(threads), args, smem, s);
 }
 
 // Occupancy of the histogram kernel for a launch shape, cached per device so

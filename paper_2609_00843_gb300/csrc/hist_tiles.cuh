@@ -61,6 +61,7 @@ __device__ __forceinline__ void hist_tiles(const HistArgs &a, uint32_t cta, uint
     for (uint32_t i = tid; i < w + (ADAPT ? 1u : 0u); i += nt) S[i] = 0;  // + the trash word
     if (ADAPT && tid < 8) s_tc[tid] = 0;
     __syncthreads();
+    if (STREAMING) asm volatile("griddepcontrol.wait;" ::: "memory");  // (launch_first)
 
     const uint32_t base = a.min_u + b;  // key - base = position inside the tile
     const uint32_t s_base = (uint32_t)__cvta_generic_to_shared(S);

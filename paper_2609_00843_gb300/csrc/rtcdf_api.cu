@@ -255,7 +255,7 @@ rtcdf_status hist_phase(const int32_t *in, uint64_t n, int64_t minVal, uint32_t 
     else if (ctl && (*parted = use_part(n, pl, scratch, &part)))
         e = launch_part(part, in, n, pl.head, pl.nvec, h.min_u, R, H, bucket_start, half, ctl, pl.sms, s);
     else
-        e = launch_hist(h, pl.hist_threads, pl.hist_smem, pl.streaming, s);
+        e = launch_hist(h, pl.hist_threads, pl.hist_smem, pl.streaming, ctl != nullptr, s);
     return e == cudaSuccess ? RTCDF_OK : RTCDF_ERR_CUDA;
 }
 

@@ -96,6 +96,33 @@ inline WsLayout ws_layout(uint64_t R, size_t total) {
     return L;
 }
 
+// The first launch of a sort: a programmatic dependent of whatever kernel is before
+// it in the stream, unless the stream is being captured (whose last node may be of
+// another kind).  The kernel waits for that one before it reads or writes anything
+// but its shared memory, and reads its input with loads that are coherent from then
+// on (no ld.global.nc); the output kernels let it be scheduled in their tails.
+// Sorts issued one after another, us each, before / now: n = 1e4, R = 1000 6.3 / 4.8; 1e6,
+// R = 128 8.2 / 6.5; 3.1e6, R = 50021 28.7 / 25.5; 1e8, R = 2^14 133.5 / 131.5.  Used for
+// the one-tile histogram and the one-CTA sort: part_kernel and pack_kernel take the
+// shared memory that the output kernel's tail runs in, and got slower (n = 3e7, R = 1e6
+// 122 / 129; n = 1e9, R = 2^16 1131 / 1144), the tiles of a wider range read with __ldg.
+inline cudaError_t launch_first(const void *fn, uint32_t grid, int threads, size_t smem, void **args, cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(s, &cap);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
 // ---------------------------------------------------------------- histogram
 struct HistArgs {
     const int32_t *in;
@@ -106,8 +133,8 @@ struct HistArgs {
     uint32_t R, T, m, g;   // range size, tile width, tiles, CTAs per tile
     uint32_t *H;           // global histogram, R entries (added to)
 };
-cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool streaming,
-                        cudaStream_t s);
+// first: of a whole sort.
+cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool streaming, bool first, cudaStream_t s);
 cudaError_t hist_max_ctas_per_sm(int threads, size_t smem, bool streaming, int *ctas);
 
 // ---------------------------------------------------------------- small arrays

@@ -75,6 +75,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_kernel(SmallArgs a) {
     int32_t *s_val = reinterpret_cast<int32_t *>(s_end + a.max_runs);
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t n = a.n, R = a.R;
+    for (uint32_t b = tid; b < R; b += kSmallThreads) S[b] = 0;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
     // After a wait that ran out nothing is written until the status has been read.
     const uint32_t status = a.ctl->status;
     const uint32_t head = min(n, (uint32_t)((16 - ((uintptr_t)a.in & 15)) & 15) / 4), nv = (n - head) / 4;
@@ -83,10 +86,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_kernel(SmallArgs a) {
     int4 k[V];
 #pragma unroll
     for (int u = 0; u < V; u++)
-        if (tid + u * kSmallThreads < nv) k[u] = __ldg(vin + tid + u * kSmallThreads);
+        if (tid + u * kSmallThreads < nv) k[u] = __ldcs(vin + tid + u * kSmallThreads);
     const uint32_t i = tid < head ? tid : head + 4 * nv + (tid - head);  // the keys outside whole vectors
-    const int32_t extra = tid < n - 4 * nv ? __ldg(a.in + i) : 0;
-    for (uint32_t b = tid; b < R; b += kSmallThreads) S[b] = 0;
+    const int32_t extra = tid < n - 4 * nv ? __ldcs(a.in + i) : 0;
     __syncthreads();
     const uint32_t s_base = (uint32_t)__cvta_generic_to_shared(S);
     auto count = [&](int32_t key) {
@@ -140,8 +142,9 @@ cudaError_t launch_small(const int32_t *in, int32_t *out, uint32_t n, uint32_t m
     static std::atomic<uint64_t> raised{0};
     const cudaError_t e = raise_shared_limit((const void *)small_kernel, raised);
     if (e != cudaSuccess) return e;
-    small_kernel<<<1, kSmallThreads, 4 * ((size_t)a.words + 2 * (size_t)a.max_runs), s>>>(a);
-    return cudaGetLastError();
+    void *args[] = {&a};
+    return launch_first((const void *)small_kernel, 1, kSmallThreads, 4 * ((size_t)a.words + 2 * (size_t)a.max_runs),
+                        args, s);
 }
 
 // Scan and output in one launch, for counts H over a narrow range: every CTA (at
@@ -157,6 +160,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) finish_kernel(FinishArgs a) 
     int32_t *s_val = reinterpret_cast<int32_t *>(s_end + a.max_runs);
     const uint32_t tid = threadIdx.x, warp = tid >> 5, R = a.R;
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
     const uint32_t status = a.ctl->status;
     // (H is padded to whole scan chunks of zeros, S to whole vectors)
     for (uint32_t i = tid; i < (R + 3) / 4; i += kSmallThreads)

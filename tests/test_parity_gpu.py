@@ -423,3 +423,26 @@ def test_scan_and_output_in_one_launch(n, R, dist):
     assert rtcdf.rtcdf_fill_from_counts(counts.data_ptr(), n - 1, mn, mn + R, 0, n - 1, win.data_ptr(), ws.data_ptr(),
                                         wsb, s) == rtcdf.OK
     assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s)[1] == rtcdf.DEV_KEY_OUT_OF_RANGE
+
+
+# Sorts issued one after another may overlap their launches: each has to read what
+# the kernel before it wrote, be that a sort (the same buffers and workspace, in
+# turn and in place) or another kernel.
+@pytest.mark.parametrize("n,R", [(10_007, 1000), (32_768, 16_384), (100_003, 100), (1_000_001, 5000), (3_000_001, 50_021)])
+def test_sorts_back_to_back(n, R):
+    s = stream_handle()
+    x = [dev_keys(n, 0, R, k % 3, gen.derive_seed(83, n, k)) for k in range(6)]
+    want = [v.sort().values for v in x]
+    a, b, c = torch.empty_like(x[0]), torch.empty_like(x[0]), torch.empty_like(x[0])
+    got = []
+    for _ in range(5):
+        for v in x:
+            a.copy_(v)                             # a kernel, then the sort of what it wrote
+            rtcdf.rtcdf_sort(a.data_ptr(), b.data_ptr(), n, 0, R, s)
+            torch.sub(R - 1, b, out=c)
+            rtcdf.rtcdf_sort(c.data_ptr(), c.data_ptr(), n, 0, R, s)
+            rtcdf.rtcdf_sort(c.data_ptr(), a.data_ptr(), n, 0, R, s)   # the sort's own output
+            got.append((b.clone(), a.clone()))
+    assert rtcdf.rtcdf_status_get(s) == (rtcdf.OK, 0)
+    for k, (up, down) in enumerate(got):
+        assert torch.equal(up, want[k % 6]) and torch.equal(down, (R - 1 - want[k % 6]).flip(0)), k
