@@ -474,8 +474,13 @@ status_str = rtcdf_status_str
 
 # ---------------------------------------------------------------- torch convenience
 def _stream_handle(stream) -> int:
-    import torch
     if stream is None:
+        # torch.cuda.current_stream() builds a Stream object: 2.9 us of a call whose
+        # sort takes 5 to 7 (n = 1e4 ... 1e6).  The handle alone takes 0.4.
+        import torch
+        raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if raw is not None and dev is not None and torch.cuda.is_initialized():
+            return raw(dev())
         stream = torch.cuda.current_stream()
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
