@@ -138,7 +138,7 @@ cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool stream
 cudaError_t hist_max_ctas_per_sm(int threads, size_t smem, bool streaming, int *ctas);
 
 // ---------------------------------------------------------------- small arrays
-constexpr uint32_t kSmallMaxN = 32768, kSmallMaxR = 16384;
+constexpr uint32_t kSmallMaxN = 24576, kSmallMaxR = 16384;
 struct SmallArgs {
     const int32_t *in;
     int32_t *out;

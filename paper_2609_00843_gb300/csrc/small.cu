@@ -5,13 +5,13 @@
 // output (Algorithm 7) in shared memory, with nothing but the status word in the
 // workspace.
 //
-// What bounds such a sort is its chain of dependent steps, and as three launches
+// What bounds such a sort is its chain of dependent steps, and as two launches
 // also their latency and the host's submission of them.  One CTA's steps take
-// longer with more keys, and pass the three launches' at about 32768 keys
-// (replayed from a graph, us a sort, uniform keys, this kernel / the three
-// launches): n = 100, R = 128 3.7 / 8.1; n = 10007, R = 1000 5.4 / 9.0; n = 16384,
-// R = 16384 8.9 / 12.9; n = 32768, R = 128 7.4 / 7.3, R = 16384 11.6 / 12.9; and
-// issued one by one from Python: n = 10007, R = 1000 8.2 / 11.7.
+// longer with more keys, and pass the two launches' at about 24000 (issued one after
+// another, us, this kernel / histogram, then scan and output, uniform keys): n = 100, R
+// = 100 3.3 / 4.8; n = 8000, R = 1000 4.6 / 6.5; n = 16000, R = 16384 8.1 / 10.7; n = 24000, R =
+// 100 6.3 / 5.9, R = 16384 10.1 / 10.6; n = 32000 6.8 / 5.5 and 11.0 / 10.9; before, as three
+// launches, n = 10007, R = 1000 11.7.
 #include <algorithm>
 #include <atomic>
 

@@ -378,7 +378,7 @@ def test_bounded_wait_runs_out_and_reports_timeout():
 
 # One launch for the whole sort: its largest size and range and one more of each,
 # the smallest, keys and outputs at every alignment, a key out of range, in place.
-@pytest.mark.parametrize("n", [1, 3, 5, 4095, 10_007, 32768, 32769])
+@pytest.mark.parametrize("n", [1, 3, 5, 4095, 10_007, 24576, 24577, 32768, 32769])
 @pytest.mark.parametrize("R", [1, 2, 1024, 1025, 16384, 16385])
 def test_small_arrays(n, R):
     for k in range(4):
