@@ -221,6 +221,8 @@ rtcdf_status check_args(const int32_t *in, int32_t *out, uint64_t n) {
     return RTCDF_OK;
 }
 
+constexpr uint32_t kWideOutMinR = 1000000;  // (use_wide_out)
+
 // Histogram by packed counters (pack.cu) or by range tiles (hist.cu): one pass
 // over the input against one per tile, and about 10 us more (the sample and a
 // second launch; without scratch, the counters added to H by pairs of CTAs: packed
@@ -233,9 +235,14 @@ bool use_pack(uint64_t n, const Plan &pl, uintptr_t scratch, PackPlan *pp) {
 
 // Histogram by partition (part.cu) or by range tiles (hist.cu).  Partition
 // takes about 9 us more (two launches) and reads the input once where the
-// tiles read it m times, so it needs several tiles and enough keys.
+// tiles read it m times, so it needs several tiles and enough keys; fewer where
+// wide_out.cu follows, whose launch takes the place of two that grow with R.  Whole
+// sorts one after another, us, partition / tiles, uniform, normal, one value: R = 2^22, n =
+// 3000 27 27 25 / 32 32 27, n = 3e5 33 32 29 / 45 47 34; R = 2^21, n = 1e6 35 33 31 / 46 49 33, n
+// = 1e5 29 27 27 / 31 32 24; R = 1e6, n = 3e6 43 43 31 / 51 55 39, n = 1e6 35 34 29 / 35 36 26.
 bool use_part(uint64_t n, const Plan &pl, uintptr_t scratch, PartPlan *pp) {
-    if (!scratch || pl.shape_given || pl.m <= 5 || n * (pl.m - 5) < 40000000u) return false;
+    const uint64_t keys = pl.R >= 1u << 22 ? 0 : pl.R >= kWideOutMinR ? 20000000 : 40000000;
+    if (!scratch || pl.shape_given || pl.m <= 5 || n * (pl.m - 5) < keys) return false;
     return part_plan(n, pl.R, pl.head, pl.nvec, scratch, pl.sms, pp);
 }
 
@@ -269,7 +276,7 @@ rtcdf_status hist_phase(const int32_t *in, uint64_t n, int64_t minVal, uint32_t 
 // 333; n = 1e6 81 79 43 / 111 109 73; n = 2e7, R = 2^20 90 96 73 / 102 106 76; n = 1.2e7
 // 67 70 55 / 72 75 55; beyond the lines, n = 5e7, R = 2^21 184 196 144 / 187 195 140;
 // n = 1e8, R = 2^20 302 331 248 / 287 307 236; n = 6e6, R = 7e5 47 51 40 / 50 56 38.
-bool use_wide_out(uint64_t n, uint32_t R) { return R >= 1000000 && n <= 20ull * R; }
+bool use_wide_out(uint64_t n, uint32_t R) { return R >= kWideOutMinR && n <= 20ull * R; }
 
 // Most positions that scan and output in one launch serve (small.cu).  Whole
 // sorts replayed from a graph, us, one launch / two, uniform keys over R = 128 and

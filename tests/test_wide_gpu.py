@@ -190,3 +190,20 @@ def test_wide_output_reports_a_stray_ticket():
     assert rtcdf.rtcdf_sort_ws(x.data_ptr(), out.data_ptr(), n, 0, R, ws.data_ptr(), wsb, s) == rtcdf.OK
     assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
     assert_matches_oracle(x, out, 0, R)
+
+
+# Few keys over a wide range: the fewest that the output buffer holds the partition
+# of and fewer, both sides of the keys from which 2^20 < R < 2^22 is partitioned.
+@pytest.mark.parametrize("R,n", [(1 << 22, 100), (1 << 22, 2600), (1 << 22, 2774), (1 << 22, 3001), ((1 << 22) + 1, 5003),
+                                 (1 << 24, 16_000), (1 << 24, 30_001), (1_000_000, 1_538_461), (1_000_000, 1_538_462),
+                                 (1 << 21, 625_000), (1 << 21, 625_001)])
+@pytest.mark.parametrize("dist", [gen.UNIFORM, gen.NORMAL, gen.ALL_EQUAL])
+def test_few_keys_over_a_wide_range(R, n, dist):
+    mn = (1 << 31) - R
+    for k in range(4):
+        x = torch.empty(n + 3, dtype=torch.int32, device="cuda")[k:k + n]
+        gen.keys_device(x.data_ptr(), n, mn, R, dist, gen.derive_seed(36, R, n, k), stream=stream_handle())
+        out = torch.full((n + 8,), 5, dtype=torch.int32, device="cuda")
+        gpu_sort(x, mn, mn + R, out[3 - k:3 - k + n])
+        assert_matches_oracle(x, out[3 - k:3 - k + n], mn, mn + R)
+        assert bool((out[:3 - k] == 5).all()) and bool((out[3 - k + n:] == 5).all())
