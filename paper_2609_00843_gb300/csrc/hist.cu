@@ -62,7 +62,7 @@ cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool stream
     dim3 grid(a.m * a.g);
     void *args[] = {const_cast<HistArgs *>(&a)};
     const void *fn = hist_fn(hist_variant(streaming, a.m), hist_unroll(smem));
-    if (streaming && first) return launch_first(fn, grid.x, threads, smem, args, s);
+    if (first) return launch_first(fn, grid.x, threads, smem, args, s);
     return cudaLaunchKernel(fn, grid, dim3(threads), args, smem, s);
 }
 

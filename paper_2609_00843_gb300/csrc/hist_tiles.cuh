@@ -10,7 +10,7 @@ namespace rtcdf {
 template <bool STREAMING>
 __device__ __forceinline__ int4 load_vec(const int4 *p) {
     if (STREAMING) return __ldcs(p);  // read once: evict first
-    return __ldg(p);                  // re-read by the other tiles' CTAs: keep in L2
+    return __ldcg(p);                 // re-read by the other tiles' CTAs: keep in L2
 }
 
 // S[y] += 1 when y < w, as a predicated shared-memory reduction (no branch).
@@ -61,7 +61,7 @@ __device__ __forceinline__ void hist_tiles(const HistArgs &a, uint32_t cta, uint
     for (uint32_t i = tid; i < w + (ADAPT ? 1u : 0u); i += nt) S[i] = 0;  // + the trash word
     if (ADAPT && tid < 8) s_tc[tid] = 0;
     __syncthreads();
-    if (STREAMING) asm volatile("griddepcontrol.wait;" ::: "memory");  // (launch_first)
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // (launch_first)
 
     const uint32_t base = a.min_u + b;  // key - base = position inside the tile
     const uint32_t s_base = (uint32_t)__cvta_generic_to_shared(S);
@@ -76,7 +76,7 @@ __device__ __forceinline__ void hist_tiles(const HistArgs &a, uint32_t cta, uint
     bool pf = false;
     if (ADAPT) {
         if ((tid & 31) == 0 && v < nvec) {
-            const int4 k = __ldg(vin + v);
+            const int4 k = __ldcg(vin + v);
             const uint32_t y[4] = {(uint32_t)k.x - a.min_u, (uint32_t)k.y - a.min_u,
                                    (uint32_t)k.z - a.min_u, (uint32_t)k.w - a.min_u};
 #pragma unroll

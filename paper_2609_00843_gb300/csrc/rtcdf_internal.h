@@ -102,10 +102,10 @@ inline WsLayout ws_layout(uint64_t R, size_t total) {
 // but its shared memory, and reads its input with loads that are coherent from then
 // on (no ld.global.nc); the output kernels let it be scheduled in their tails.
 // Sorts issued one after another, us each, before / now: n = 1e4, R = 1000 6.3 / 4.8; 1e6,
-// R = 128 8.2 / 6.5; 3.1e6, R = 50021 28.7 / 25.5; 1e8, R = 2^14 133.5 / 131.5.  Used for
-// the one-tile histogram and the one-CTA sort: part_kernel and pack_kernel take the
-// shared memory that the output kernel's tail runs in, and got slower (n = 3e7, R = 1e6
-// 122 / 129; n = 1e9, R = 2^16 1131 / 1144), the tiles of a wider range read with __ldg.
+// R = 128 8.2 / 6.5, R = 350000 28.3 / 25.0; 3.1e6, R = 50021 28.7 / 25.5; 1e7, R = 200000 44.8 /
+// 41.5; 1e8, R = 2^14 133.5 / 131.5.  Used for all range tiles and the one-CTA sort;
+// part_kernel and pack_kernel take the shared memory that the output kernel's tail runs
+// in and got slower (n = 3e7, R = 1e6 122 / 129; n = 1e8, R = 2^18 158.5 / 166.7).
 inline cudaError_t launch_first(const void *fn, uint32_t grid, int threads, size_t smem, void **args, cudaStream_t s) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const cudaError_t e = cudaStreamIsCapturing(s, &cap);
