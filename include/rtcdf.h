@@ -425,8 +425,8 @@ rtcdf_status rtcdf_sort_batched_host(const int32_t *in, int32_t *out, const int6
  *
  * rtcdf_sort_batched uses a library-owned workspace per (device, stream),
  * grown on demand by stream-ordered allocation (inside CUDA graph capture it
- * must already be large enough: rtcdf_batch_reserve); rtcdf_status_get reads
- * its status.  rtcdf_sort_batched_device_ws takes a caller workspace
+ * must already be large enough: rtcdf_batch_reserve) and cleared when a call's
+ * bounds differ from the last call's; rtcdf_status_get reads its status.  rtcdf_sort_batched_device_ws takes a caller workspace
  * (256-byte aligned, zero-filled before its first use, left ready for the
  * next call of any layout within the same bounds; calls sharing it must be
  * ordered): no allocation, so it can be captured in a CUDA graph and replayed
