@@ -33,6 +33,16 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a) {
     hist_tiles<STREAMING, UNROLL, ADAPT>(a, blockIdx.x, S, s_tc);
 }
 
+// One tile of a long input: one CTA per SM, whose 64 registers a thread hold six
+// vectors in flight while six are counted.  n = 1e9, R = 4096, whole sort, us: 1142 against
+// 1181 with two CTAs of 32 registers (2e8, R = 128 237 / 240); below 2e8 keys the two are
+// within 1 % of each other either way (1e8: R = 128 125.5 / 126.5, 16384 129.8 / 129.2, 49000
+// 134.4 / 133.5), and two leave room for other streams' kernels.
+__global__ void __launch_bounds__(1024, 1) hist_long_kernel(HistArgs a) {
+    extern __shared__ uint32_t S[];
+    hist_tiles<true, 6, false, true>(a, blockIdx.x, S, nullptr);
+}
+
 // Kernel variant: streaming loads for one tile; the adaptive form for 2 to 8
 // tiles; the plain predicated form beyond.
 enum HistVariant { kHistStreaming = 0, kHistAdaptive = 1, kHistPlain = 2 };
@@ -62,6 +72,11 @@ cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool stream
     dim3 grid(a.m * a.g);
     void *args[] = {const_cast<HistArgs *>(&a)};
     const void *fn = hist_fn(hist_variant(streaming, a.m), hist_unroll(smem));
+    if (a.long_form) {
+        fn = (const void *)hist_long_kernel;
+        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
     if (first) return launch_first(fn, grid.x, threads, smem, args, s);
     return cudaLaunchKernel(fn, grid, dim3(threads), args, smem, s);
 }

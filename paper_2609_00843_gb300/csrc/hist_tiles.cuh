@@ -50,7 +50,7 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
 // CTA `cta` of m * g: tile cta mod m, the (cta / m)-th of the tile's g CTAs.  S is
 // the tile's shared memory (the tile, and the trash word if ADAPT), s_tc eight
 // words of it.
-template <bool STREAMING, int UNROLL, bool ADAPT>
+template <bool STREAMING, int UNROLL, bool ADAPT, bool PIPE = ADAPT>
 __device__ __forceinline__ void hist_tiles(const HistArgs &a, uint32_t cta, uint32_t *S, uint32_t *s_tc) {
     const uint32_t t = cta % a.m;
     const uint32_t q = cta / a.m;
@@ -106,7 +106,7 @@ __device__ __forceinline__ void hist_tiles(const HistArgs &a, uint32_t cta, uint
             count_key(s_base, (uint32_t)k.w - base, w);
         }
     };
-    if (!ADAPT) {
+    if (!PIPE) {
         // One tile: UNROLL vectors loaded, then counted (32 registers, so
         // that two CTAs fit an SM: with the pipeline below these CTAs took 64
         // registers and the 12-array step on three streams got slower).
@@ -118,7 +118,8 @@ __device__ __forceinline__ void hist_tiles(const HistArgs &a, uint32_t cta, uint
             for (int u = 0; u < UNROLL; u++) count_vec(k[u]);
         }
     } else {
-        // Several tiles (one CTA per SM, its shared memory being the tile):
+        // Several tiles (one CTA per SM, its shared memory being the tile), or a
+        // long input over one tile (hist_long_kernel):
         // software pipelined, the next P vectors in flight while the last P
         // are counted (R = 2^18 uniform, n = 1e8: 0.272 against 0.281 ms per
         // sort, measured).

@@ -64,6 +64,7 @@ struct Plan {
     int hist_threads;
     size_t hist_smem;
     bool streaming;
+    bool hist_long;     // one tile of a long input (hist_long_kernel)
     bool shape_given;   // the histogram's shape comes from the caller or the tuning table
     bool fill_given;    // the output's shape comes from the caller
     int sms;
@@ -86,6 +87,8 @@ rtcdf_status check_range(int64_t minVal, int64_t maxVal, uint32_t *R) {
 // Few keys per value: the output kernel's form for short runs.  (R = 2^19, n =
 // 1e8, 190 keys per value: 65.5 against 71.7 us; 381 keys: 73.7 against 63.5.)
 bool short_runs(uint64_t n, uint32_t R) { return n < 256ull * R; }
+
+constexpr uint64_t kHistLongMinN = 200000000;  // (see hist_long_kernel)
 
 // Choose the launch shape (Section 3.3): tile width T from shared memory, CTAs
 // per tile from occupancy, output CTAs from n.
@@ -144,6 +147,8 @@ rtcdf_status make_plan_with(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t
     uint64_t g = std::max<uint64_t>(1, (uint64_t)occ * dev.sms / pl->m);
     uint64_t g_n = std::max<uint64_t>(1, (n + 16ull * pl->hist_threads - 1) / (16ull * pl->hist_threads));
     g = std::min(g, g_n);
+    pl->hist_long = pl->streaming && !pl->shape_given && n >= kHistLongMinN;
+    if (pl->hist_long) g = dev.sms;
     if (q.hist_ctas_per_tile > 0) g = (uint64_t)q.hist_ctas_per_tile;
     pl->g = (uint32_t)g;
 
@@ -256,7 +261,7 @@ rtcdf_status hist_phase(const int32_t *in, uint64_t n, int64_t minVal, uint32_t 
     HistArgs h;
     h.in = in; h.n = n; h.nvec = pl.nvec; h.head = pl.head;
     h.min_u = (uint32_t)(int32_t)minVal; h.R = R; h.T = pl.T; h.m = pl.m; h.g = pl.g;
-    h.H = H;
+    h.H = H; h.long_form = pl.hist_long;
     PackPlan pack;
     PartPlan part;
     cudaError_t e;

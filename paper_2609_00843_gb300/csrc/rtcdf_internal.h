@@ -132,6 +132,7 @@ struct HistArgs {
     uint32_t min_u;        // (uint32_t)minVal
     uint32_t R, T, m, g;   // range size, tile width, tiles, CTAs per tile
     uint32_t *H;           // global histogram, R entries (added to)
+    bool long_form = false;  // one tile, one CTA per SM: hist_long_kernel
 };
 // first: of a whole sort.
 cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool streaming, bool first, cudaStream_t s);

@@ -447,3 +447,15 @@ def test_sorts_back_to_back(n, R):
     assert rtcdf.rtcdf_status_get(s) == (rtcdf.OK, 0)
     for k, (up, down) in enumerate(got):
         assert torch.equal(up, want[k % 6]) and torch.equal(down, (R - 1 - want[k % 6]).flip(0)), k
+
+
+# The histogram of a long input over one tile: from its fewest keys on.
+@pytest.mark.parametrize("n,R", [(199_999_999, 300), (200_000_003, 300), (200_000_001, 49_152)])
+def test_long_inputs_over_one_tile(n, R):
+    x = torch.empty(n + 1, dtype=torch.int32, device="cuda")[1:]
+    gen.keys_device(x.data_ptr(), n, -7, R, gen.NORMAL, gen.derive_seed(84, R), stream=stream_handle())
+    counts = torch.bincount(x.sub(-7).clamp_(0, R), minlength=R + 1)
+    assert int(counts[R]) == 0
+    out = gpu_sort(x, -7, R - 7)
+    want = torch.repeat_interleave(torch.arange(-7, R - 7, device="cuda", dtype=torch.int32), counts[:R])
+    assert torch.equal(out, want)
