@@ -303,7 +303,11 @@ rtcdf_status finish_phase(int32_t *out, uint64_t n, int64_t minVal, uint32_t R, 
     uint32_t *run_end = (uint32_t *)(base + L.run_end);
     int32_t *run_val = (int32_t *)(base + L.run_val);
     uint32_t *start_run = (uint32_t *)(base + L.start_run);
-    const uint32_t head_out = (uint32_t)(((16 - ((uintptr_t)out & 15)) & 15) / 4);
+    // Positions before the first whole vector: all of them in a window without one,
+    // since pos_base + head must not pass 2^32 (with no vector to store, the frame's
+    // alignment does not matter).
+    const uint32_t head_out =
+        (uint32_t)std::min<uint64_t>(((16 - ((uintptr_t)out & 15)) & 15) / 4, pos_end - pos_base);
     if (!dbg && !pl.fill_given && R <= kSmallMaxR && pos_end - pos_base <= kFinishMaxN) {
         FinishArgs f;
         f.H = (uint32_t *)(base + L.hist); f.out = out; f.n = (uint32_t)n;

@@ -1,0 +1,42 @@
+"""Outputs at the limits of the arithmetic: the last positions of the largest
+arrays, where 32-bit positions end."""
+import pytest
+import torch
+
+from gpu_util import stream_handle
+from paper_2609_00843_gb300 import rtcdf
+
+pytestmark = pytest.mark.gpu
+
+N_MAX = (1 << 32) - 1
+
+
+def u32(x):
+    """The int32 with the bits of the 32-bit unsigned x."""
+    return x - (1 << 32) if x >= 1 << 31 else x
+
+
+def end_window(counts, R, length, offset, ws, wsb):
+    """Positions [N_MAX - length, N_MAX) of the array with these counts, written `offset`
+    elements into a buffer whose other elements stay -5."""
+    s = stream_handle()
+    out = torch.full((length + 8,), -5, dtype=torch.int32, device="cuda")
+    win = out[offset:offset + length]
+    assert rtcdf.rtcdf_fill_from_counts(counts.data_ptr(), N_MAX, 0, R, N_MAX - length, N_MAX, win.data_ptr(),
+                                        ws.data_ptr(), wsb, s) == rtcdf.OK
+    assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
+    assert bool((out[:offset] == -5).all()) and bool((out[offset + length:] == -5).all())
+    return win
+
+
+# Windows that end before their output's first whole vector would begin.
+@pytest.mark.parametrize("R", [20_000, 1 << 20])
+def test_windows_without_a_whole_vector_at_the_end_of_the_largest_array(R):
+    counts = torch.ones(R, dtype=torch.int32, device="cuda")
+    counts[0] = u32(N_MAX - (R - 1))
+    wsb = rtcdf.rtcdf_workspace_size(R)
+    ws = torch.zeros(wsb // 4, dtype=torch.int32, device="cuda")
+    for offset in range(4):
+        for length in range(1, 8):
+            win = end_window(counts, R, length, offset, ws, wsb)
+            assert win.tolist() == list(range(R - length, R)), (offset, length)
