@@ -817,7 +817,7 @@ __device__ __forceinline__ void fill_item(const BatchArgs &a, const BatchItem &i
         }
         __syncthreads();
         const uint32_t hi = min(P1, s_end[nw - 1]);
-        const uint32_t w_lo = pos >= head ? (pos - head + 3) >> 2 : 0u;
+        const uint32_t w_lo = pos >= head ? vec_ceil(pos - head) : 0u;
         const uint32_t w_hi = hi >= head ? (hi - head) >> 2 : 0u;
         const uint32_t nvec = w_hi > w_lo ? w_hi - w_lo : 0u;
         const uint32_t per_warp = ((nvec + kFillWarps - 1) / kFillWarps + 31) & ~31u;

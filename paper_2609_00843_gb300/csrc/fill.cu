@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(WIN) fill_kernel(FillArgs a) {
         __syncthreads();
         const uint32_t hi = min(P1, s_end[nw - 1]);
         // Whole vectors w cover [hb + 4w, hb + 4w + 4) inside [pos, hi).
-        const uint32_t w_lo = pos >= hb ? (pos - hb + 3) >> 2 : 0u;
+        const uint32_t w_lo = pos >= hb ? vec_ceil(pos - hb) : 0u;
         const uint32_t w_hi = hi >= hb ? (hi - hb) >> 2 : 0u;
 
         if (s_end[0] >= hi) {

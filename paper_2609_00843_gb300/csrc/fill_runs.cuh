@@ -6,6 +6,9 @@
 
 namespace rtcdf {
 
+// Vectors of four positions that begin before position p, p = 2^32 - 1 included.
+__device__ __forceinline__ uint32_t vec_ceil(uint32_t p) { return (p >> 2) + ((p & 3) != 0); }
+
 // Smallest j in [lo, hi] with s_end[j] > p, given s_end[hi] > p.
 __device__ __forceinline__ int first_run_after(const uint32_t *s_end, int lo, int hi, uint32_t p) {
     while (lo < hi) {

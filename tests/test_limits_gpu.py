@@ -40,3 +40,27 @@ def test_windows_without_a_whole_vector_at_the_end_of_the_largest_array(R):
         for length in range(1, 8):
             win = end_window(counts, R, length, offset, ws, wsb)
             assert win.tolist() == list(range(R - length, R)), (offset, length)
+
+
+# A last window of runs that begins within three positions of 2^32: as many runs as
+# fill whole windows of the output kernel (of 1024, 2048, 4096, 8192), and one.
+@pytest.mark.parametrize("offset", [0, 3])
+def test_last_run_of_the_largest_array(offset):
+    out = torch.empty(N_MAX + 4, dtype=torch.int32, device="cuda")
+    win, s = out[offset:offset + N_MAX], stream_handle()
+    for runs in (1024, 2048, 4096, 8192):
+        for last in (1, 2):                      # keys of the last run
+            R = runs + 1
+            counts = torch.ones(R, dtype=torch.int32, device="cuda")
+            counts[R - 1] = last
+            counts[0] = u32(N_MAX - (R - 2) - last)
+            wsb = rtcdf.rtcdf_workspace_size(R)
+            ws = torch.zeros(wsb // 4, dtype=torch.int32, device="cuda")
+            out.fill_(-5)
+            assert rtcdf.rtcdf_fill_from_counts(counts.data_ptr(), N_MAX, 0, R, 0, N_MAX, win.data_ptr(), ws.data_ptr(),
+                                                wsb, s) == rtcdf.OK
+            assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
+            tail = list(range(1, R - 1)) + [R - 1] * last
+            assert win[N_MAX - len(tail):].tolist() == tail, (runs, last)
+            assert int(torch.count_nonzero(win[:N_MAX - len(tail)])) == 0, (runs, last)
+            assert bool((out[:offset] == -5).all()) and bool((out[offset + N_MAX:] == -5).all())
