@@ -64,3 +64,18 @@ def test_last_run_of_the_largest_array(offset):
             assert win[N_MAX - len(tail):].tolist() == tail, (runs, last)
             assert int(torch.count_nonzero(win[:N_MAX - len(tail)])) == 0, (runs, last)
             assert bool((out[:offset] == -5).all()) and bool((out[offset + N_MAX:] == -5).all())
+
+
+# Runs of one key up to the very last position: scan and output in one launch (R up
+# to 16384), and the general kernels' form for short runs.
+@pytest.mark.parametrize("R", [301, 16384, 1 << 24])
+def test_short_runs_at_the_end_of_the_largest_array(R):
+    counts = torch.ones(R, dtype=torch.int32, device="cuda")
+    counts[0] = u32(N_MAX - (R - 1))             # value 0 to position 2^32 - R, then a position each
+    wsb = rtcdf.rtcdf_workspace_size(R)
+    ws = torch.zeros(wsb // 4, dtype=torch.int32, device="cuda")
+    for offset in (0, 1, 3):
+        for length in (1, 300, 512, 1000, 5003, 70_001):
+            win = end_window(counts, R, length, offset, ws, wsb)
+            want = torch.arange(R - length, R, device="cuda").clamp_(min=0).int()
+            assert torch.equal(win, want), (offset, length)
