@@ -171,7 +171,9 @@ __global__ void __launch_bounds__(WIN) fill_kernel(FillArgs a) {
             if (p >= pos && p < hi && (w_lo >= w_hi || p < q_lo || p >= q_hi))
                 a.out[p - pb] = s_val[first_run_after(s_end, 0, nw - 1, p)];
         }
-        pos = hi;
+        // (counts that a caller gives and that pass 2^32 make run ends that decrease:
+        // never back, where the positions are not this CTA's)
+        pos = max(pos, hi);
         k_cur += nw;
     }
 }

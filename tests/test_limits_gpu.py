@@ -1,5 +1,5 @@
 """Outputs at the limits of the arithmetic: the last positions of the largest
-arrays, where 32-bit positions end."""
+arrays, where 32-bit positions end, and counts whose sums pass 2^32."""
 import pytest
 import torch
 
@@ -79,3 +79,38 @@ def test_short_runs_at_the_end_of_the_largest_array(R):
             win = end_window(counts, R, length, offset, ws, wsb)
             want = torch.arange(R - length, R, device="cuda").clamp_(min=0).int()
             assert torch.equal(win, want), (offset, length)
+
+
+# Counts that do not add up and whose running sum passes 2^32 on the way, so that the
+# run ends decrease: reported, nothing stored outside the window, and the workspace
+# serves the next call.  Scan and output in one launch, then the general kernels over
+# short runs and over long ones (each with more runs than a window of the kernel).
+# The sum falls at value `at` to that of value `to`; one window ends early in the scan's
+# chunk of 4096 values with the fall.
+@pytest.mark.parametrize("R,each", [(1501, 40), (16384, 40), (20_000, 40), (20_000, 700), (50_000, 3)])
+@pytest.mark.parametrize("at,to", [(500, 250), (8192, 1638), (16_484, 1000)])
+def test_counts_that_pass_the_largest_sum(R, each, at, to):
+    at, to = min(at, R - 500), min(to, R - 600)
+    s = stream_handle()
+    counts = torch.full((R,), each, dtype=torch.int32, device="cuda")
+    counts[at] = u32((1 << 32) - each * (at - to))
+    top = each * at                                      # the sum before the fall
+    ends = (R - 1 - at + to) * each                      # the last sum
+    total = max(top, ends) + 1
+    wsb = rtcdf.rtcdf_workspace_size(R)
+    ws = torch.zeros(wsb // 4, dtype=torch.int32, device="cuda")
+    chunk = at // 4096 * 4096 * each
+    windows = [(0, total), (total // 3, total), (total // 2 + 1, total - 5), (top * 3 // 4, top), (total - 3, total)]
+    for lo, hi in windows + [(chunk - 1500, chunk + 500)] * (chunk > 0):
+        length = hi - lo
+        out = torch.full((length + 72,), -5, dtype=torch.int32, device="cuda")
+        assert rtcdf.rtcdf_fill_from_counts(counts.data_ptr(), total, 0, R, lo, hi, out[33:].data_ptr(),
+                                            ws.data_ptr(), wsb, s) == rtcdf.OK
+        assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.ERR_KEY_OUT_OF_RANGE, rtcdf.DEV_KEY_OUT_OF_RANGE)
+        assert bool((out[:33] == -5).all()) and bool((out[33 + length:] == -5).all())
+    counts[at] = each
+    out = torch.empty(each * R, dtype=torch.int32, device="cuda")
+    assert rtcdf.rtcdf_fill_from_counts(counts.data_ptr(), each * R, 0, R, 0, each * R, out.data_ptr(), ws.data_ptr(),
+                                        wsb, s) == rtcdf.OK
+    assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
+    assert torch.equal(out, torch.arange(R, device="cuda", dtype=torch.int32).repeat_interleave(each))
