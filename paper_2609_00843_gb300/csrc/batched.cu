@@ -797,7 +797,7 @@ __device__ __forceinline__ void fill_item(const BatchArgs &a, const BatchItem &i
     const uint32_t len = (uint32_t)(it.b - it.a), per = ((len + parts - 1) / parts + 127) & ~127u;
     if (part * per >= len) return;
     uint32_t pos = (uint32_t)it.a + part * per;
-    const uint32_t P1 = min((uint32_t)it.b, pos + per);
+    const uint32_t P1 = pos + min(per, len - part * per);  // (pos + per may pass 2^32)
     uint32_t k_cur = min(start_run[it.aux], D - 1);
     // Last run this item can need: the one holding the next item's first position.
     const uint32_t k_last = (it.aux + 1 < g.fill_items) ? min(start_run[it.aux + 1], D - 1) : D - 1;

@@ -114,3 +114,30 @@ def test_counts_that_pass_the_largest_sum(R, each, at, to):
                                         wsb, s) == rtcdf.OK
     assert rtcdf.rtcdf_ws_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
     assert torch.equal(out, torch.arange(R, device="cuda", dtype=torch.int32).repeat_interleave(each))
+
+
+# The largest segment, its last values in runs of one key: the shares of its last
+# output item, the last block of short runs, and (2048 values: a window of the
+# kernel) a last run that begins a window at the last position.
+@pytest.mark.parametrize("values", [2048, 5000])
+@pytest.mark.parametrize("planned", ["device"])
+def test_largest_segment(values, planned):
+    s, R = stream_handle(), 70_000
+    x = torch.zeros(N_MAX, dtype=torch.int32, device="cuda")
+    x[torch.arange(1, values + 1, device="cuda") * 800_000] = torch.arange(R - values, R, device="cuda", dtype=torch.int32)
+    out = torch.full((N_MAX + 4,), -5, dtype=torch.int32, device="cuda")
+    if planned == "host":
+        plan = rtcdf.BatchPlan([0, N_MAX], [0], [R])
+        wsb = plan.workspace_size()
+        ws = torch.zeros(wsb // 4, dtype=torch.int32, device="cuda")
+        assert plan.run(x.data_ptr(), out.data_ptr(), ws.data_ptr(), wsb, s) == rtcdf.OK
+    else:
+        offs, mn, mx = (torch.tensor(v, dtype=torch.int64, device="cuda") for v in ([0, N_MAX], [0], [R]))
+        wsb = rtcdf.rtcdf_batch_device_workspace_size(1, N_MAX, R)
+        ws = torch.zeros(wsb // 4, dtype=torch.int32, device="cuda")
+        assert rtcdf.rtcdf_sort_batched_device_ws(x.data_ptr(), out.data_ptr(), offs.data_ptr(), mn.data_ptr(),
+                                                  mx.data_ptr(), 1, N_MAX, R, ws.data_ptr(), wsb, s) == rtcdf.OK
+    assert rtcdf.rtcdf_batch_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
+    assert torch.equal(out[N_MAX - values:N_MAX], torch.arange(R - values, R, device="cuda", dtype=torch.int32))
+    assert int(torch.count_nonzero(out[:N_MAX - values])) == 0
+    assert bool((out[N_MAX:] == -5).all())
