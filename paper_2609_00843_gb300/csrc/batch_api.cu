@@ -111,7 +111,7 @@ int build_host_plan(const SegSpec *spec, uint32_t S, HostPlan *P, const BatchTun
         g.single_hist = chunks == 1 ? 1u : 0u;
         g.scan_chunks = (g.R + kBatchScanChunk - 1) / kBatchScanChunk;
         g.fill_chunk = tun.fill_chunk;
-        g.fill_items = (uint32_t)((g.n + tun.fill_chunk - 1) / tun.fill_chunk);
+        g.fill_items = (uint32_t)(((uint64_t)g.n + tun.fill_chunk - 1) / tun.fill_chunk);
         g.hist_off = w;      w += words_align((size_t)g.scan_chunks * kBatchScanChunk);
         g.run_end_off = w;   w += words_align(g.R);
         g.run_val_off = w;   w += words_align(g.R);

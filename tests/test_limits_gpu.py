@@ -120,7 +120,7 @@ def test_counts_that_pass_the_largest_sum(R, each, at, to):
 # output item, the last block of short runs, and (2048 values: a window of the
 # kernel) a last run that begins a window at the last position.
 @pytest.mark.parametrize("values", [2048, 5000])
-@pytest.mark.parametrize("planned", ["device"])
+@pytest.mark.parametrize("planned", ["host", "device"])
 def test_largest_segment(values, planned):
     s, R = stream_handle(), 70_000
     x = torch.zeros(N_MAX, dtype=torch.int32, device="cuda")
