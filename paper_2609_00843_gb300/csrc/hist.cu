@@ -68,15 +68,11 @@ const void *hist_fn(int variant, int unroll) {
 int hist_unroll(size_t smem) { return smem > 114 * 1024 ? 8 : 4; }
 
 cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool streaming, bool first, cudaStream_t s) {
-    // hist_max_ctas_per_sm() has raised the shared-memory limit for this size.
+    // hist_max_ctas_per_sm() has raised the shared-memory limits for this size.
     dim3 grid(a.m * a.g);
     void *args[] = {const_cast<HistArgs *>(&a)};
     const void *fn = hist_fn(hist_variant(streaming, a.m), hist_unroll(smem));
-    if (a.long_form) {
-        fn = (const void *)hist_long_kernel;
-        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (a.long_form) fn = (const void *)hist_long_kernel;
     if (first) return launch_first(fn, grid.x, threads, smem, args, s);
     return cudaLaunchKernel(fn, grid, dim3(threads), args, smem, s);
 }
@@ -107,6 +103,10 @@ cudaError_t hist_max_ctas_per_sm(int threads, size_t smem, bool streaming, int *
                 e = cudaFuncSetAttribute(hist_fn(v, u), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 if (e != cudaSuccess) return e;
             }
+        }
+        if (streaming) {
+            e = cudaFuncSetAttribute(hist_long_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
         }
         lim = smem;
     }

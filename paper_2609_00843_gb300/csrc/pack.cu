@@ -53,6 +53,8 @@ constexpr uint32_t kHashBits = 14;                  // sample hash table, in the
 constexpr uint32_t kCoarse = 256;                   // stretches of the range
 constexpr int kPackCluster = 2;                     // CTAs that add up their fields before H (without scratch)
 constexpr uint32_t kHotMin = 64;                    // sampled keys that make a key hot
+constexpr uint32_t kPackMaxWords = 45056 + 1024, kPackMaxTile = 45056;  // of pack_plan
+constexpr size_t kPackSmem = 4 * (size_t)kPackMaxWords + 16;
 constexpr uint32_t kSingleNoise = 12;               // hash counts that uniform and normal keys reach
 
 __device__ __forceinline__ uint32_t sample_hash(uint32_t y) { return (y * 0x9E3779B1u) >> (32 - kHashBits); }
@@ -396,7 +398,7 @@ bool pack_plan(uint64_t n, uint32_t R, uint64_t nvec, uintptr_t scratch, int sms
     // e = magic * W - 2^32 that holds when y * e < 2^32.
     uint32_t W = std::max<uint32_t>((R + fields - 1) / fields, 1u << kHashBits);
     for (W = (W + 3) / 4 * 4;; W += 4) {
-        if (W > 45056 + 1024) return false;
+        if (W > kPackMaxWords) return false;
         p->magic = (uint32_t)(((1ull << 32) + W - 1) / W);
         if (((uint64_t)p->magic * W - (1ull << 32)) * fields * W < (1ull << 32)) break;
     }
@@ -406,8 +408,8 @@ bool pack_plan(uint64_t n, uint32_t R, uint64_t nvec, uintptr_t scratch, int sms
     p->limit = fields == 2 ? 30000.f : fields == 4 ? 140.f : fields == 5 ? 24.f : fields == 6 ? 10.f : 2.5f;
     p->ctas = (uint32_t)std::min<uint64_t>(sms, nvec / (4 * kPackThreads)) / kPackCluster * kPackCluster;
     if (p->ctas == 0) return false;
-    // Range tiles: as few as 45056 values allow, and the trash word.
-    p->m = (R + 45055) / 45056;
+    // Range tiles: as few as kPackMaxTile values allow, and the trash word.
+    p->m = (R + kPackMaxTile - 1) / kPackMaxTile;
     p->tile = (R + p->m - 1) / p->m;
     p->smem = (size_t)std::max(W, p->tile) * 4 + 16;
     p->g = std::max(1u, p->ctas / p->m);
@@ -439,7 +441,8 @@ cudaError_t launch_pack(const PackPlan &p, const HistArgs &hist, Ctl *ctl, cudaS
     a.dump = ctl ? reinterpret_cast<uint32_t *>(p.dump) : nullptr;
     a.ctl = ctl;
     void *args[] = {&a};
-    cudaError_t e = cudaFuncSetAttribute(pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    static std::atomic<uint64_t> raised{0};
+    cudaError_t e = raise_shared_limit((const void *)pack_kernel, kPackSmem, raised);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];

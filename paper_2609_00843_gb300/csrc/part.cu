@@ -56,6 +56,14 @@ __host__ __device__ inline uint32_t part_head_words(uint32_t B) {
     return (((B + 1) << part_log_copies(B)) + 2 * (B + 1) + 31) / 32 * 32;
 }
 
+// 16-byte units of a staged slab: its keys (and up to six outside whole vectors),
+// each bucket padded to 8.
+__host__ __device__ inline uint32_t part_slab_units(uint32_t B, uint32_t slab_keys) { return (slab_keys + 8 + 8 * B) / 8; }
+// Bytes of part_kernel's shared memory.
+inline size_t part_smem(uint32_t B, uint32_t slab_keys) {
+    return 4 * (size_t)part_head_words(B) + align_up(16 * (size_t)part_slab_units(B, slab_keys), 128);
+}
+
 __device__ __forceinline__ uint32_t atom_inc(uint32_t s_addr) {
     uint32_t r;
     asm volatile("atom.shared.add.u32 %0, [%1], 1;" : "=r"(r) : "r"(s_addr));
@@ -468,10 +476,9 @@ bool part_plan(uint64_t n, uint32_t R, uint32_t head, uint64_t nvec, uintptr_t o
     p->slab_keys = (uint32_t)std::min<uint64_t>(kPartSlabMax, (keys + step - 1) / step * step);
     const uint64_t slabs = std::max<uint64_t>(1, (nvec + p->slab_keys / 4 - 1) / (p->slab_keys / 4));
     p->slabs = (uint32_t)slabs;
-    // A slab's keys (and up to six outside whole vectors), each bucket padded to 8.
-    p->slab_units = (p->slab_keys + 8 + 8 * B) / 8;
+    p->slab_units = part_slab_units(B, p->slab_keys);
     p->ctas = (uint32_t)std::min<uint64_t>(slabs, sms);
-    p->smem = 4 * (size_t)part_head_words(B) + align_up(16 * (size_t)p->slab_units, 128);
+    p->smem = part_smem(B, p->slab_keys);
     const uintptr_t base = (out_addr + 15) & ~(uintptr_t)15;
     const uint64_t payload = slabs * p->slab_units * 16;
     const uint64_t starts = (slabs * (B + 1) * 2 + 15) / 16 * 16;
@@ -496,9 +503,11 @@ cudaError_t launch_part(const PartPlan &p, const int32_t *in, uint64_t n, uint32
     a.rows = reinterpret_cast<uint32_t *>(p.rows);
     a.H = H; a.bucket_start = bucket_start; a.half = half; a.ctl = ctl;
     void *args[] = {&a};
-    const void *pf = p.buckets <= 128 ? (const void *)part_kernel<part_log_copies(128)>
-                                      : (const void *)part_kernel<part_log_copies(512)>;
-    cudaError_t e = cudaFuncSetAttribute(pf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    static std::atomic<uint64_t> raised[2] = {};
+    const bool few = p.buckets <= 128;
+    const void *pf = few ? (const void *)part_kernel<part_log_copies(128)>
+                         : (const void *)part_kernel<part_log_copies(kPartMaxBuckets)>;
+    cudaError_t e = raise_shared_limit(pf, part_smem(few ? 128 : kPartMaxBuckets, kPartSlabMax), raised[few]);
     if (e != cudaSuccess) return e;
     if ((e = cudaLaunchKernel(pf, dim3(p.ctas), dim3(kPartThreads), args, p.smem, s)) != cudaSuccess) return e;
     const void *fn = (const void *)bucket_kernel;

@@ -2,6 +2,7 @@
 // Not installed; the public interface is include/rtcdf.h.
 #pragma once
 
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -94,6 +95,20 @@ inline WsLayout ws_layout(uint64_t R, size_t total) {
     L.start_run = L.run_end - align_up((size_t)kMaxFillCtas * 4, 256);
     L.total = total;
     return L;
+}
+
+// Raises a kernel's shared-memory limit to `bytes`, the most that any of its launches
+// takes, once per device (bits of `raised`).  Never to one launch's own size: the limit
+// belongs to the kernel, and another thread's smaller launch would lower it between
+// this thread's raise and launch.
+inline cudaError_t raise_shared_limit(const void *kernel, size_t bytes, std::atomic<uint64_t> &raised) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 64 && (raised.load(std::memory_order_relaxed) >> dev & 1)) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && dev < 64) raised.fetch_or(1ull << dev, std::memory_order_relaxed);
+    return e;
 }
 
 // The first launch of a sort: a programmatic dependent of whatever kernel is before

@@ -13,7 +13,6 @@
 // 100 6.3 / 5.9, R = 16384 10.1 / 10.6; n = 32000 6.8 / 5.5 and 11.0 / 10.9; before, as three
 // launches, n = 10007, R = 1000 11.7.
 #include <algorithm>
-#include <atomic>
 
 #include "fill_runs.cuh"
 
@@ -121,17 +120,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_kernel(SmallArgs a) {
     }
 }
 
-// Raises a kernel's shared-memory limit for kSmallMaxR, once per device (a sort
-// must not pay for it each time).
-static cudaError_t raise_shared_limit(const void *kernel, std::atomic<uint64_t> &raised) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 64 && (raised.load(std::memory_order_relaxed) >> dev & 1)) return cudaSuccess;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 3 * (int)kSmallMaxR);
-    if (e == cudaSuccess && dev < 64) raised.fetch_or(1ull << dev, std::memory_order_relaxed);
-    return e;
-}
+constexpr size_t kSmallSmem = 4 * 3 * (size_t)kSmallMaxR;  // of both kernels, at most
 
 cudaError_t launch_small(const int32_t *in, int32_t *out, uint32_t n, uint32_t min_u, uint32_t R, Ctl *ctl,
                          cudaStream_t s) {
@@ -140,7 +129,7 @@ cudaError_t launch_small(const int32_t *in, int32_t *out, uint32_t n, uint32_t m
     a.words = R > kSmallWarps * kBlock ? (R + 3) / 4 * 4 : kSmallWarps * kBlock;
     a.max_runs = R < n ? R : n;
     static std::atomic<uint64_t> raised{0};
-    const cudaError_t e = raise_shared_limit((const void *)small_kernel, raised);
+    const cudaError_t e = raise_shared_limit((const void *)small_kernel, kSmallSmem, raised);
     if (e != cudaSuccess) return e;
     void *args[] = {&a};
     return launch_first((const void *)small_kernel, 1, kSmallThreads, 4 * ((size_t)a.words + 2 * (size_t)a.max_runs),
@@ -200,7 +189,7 @@ cudaError_t launch_finish(const FinishArgs &args, int sms, cudaStream_t s) {
     a.words = a.R > kSmallWarps * kBlock ? (a.R + 3) / 4 * 4 : kSmallWarps * kBlock;
     a.max_runs = a.R;
     static std::atomic<uint64_t> raised{0};
-    cudaError_t e = raise_shared_limit((const void *)finish_kernel, raised);
+    cudaError_t e = raise_shared_limit((const void *)finish_kernel, kSmallSmem, raised);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((uint32_t)std::min<uint64_t>(sms, ((uint64_t)a.pos_end - a.pos_base + 2047) / 2048));
