@@ -660,6 +660,13 @@ __global__ void __launch_bounds__(kScanCtaThreads, 6) seg_scan_kernel(BatchArgs 
     // the host plan's lengths, or the device lists' bounds).
     const uint32_t n_scan = DEV ? a.dev_counts[1] : a.n_scan;
     const uint32_t n_small2 = DEV ? a.dev_counts[2] : a.n_small2;
+    // The grid must not be done before the first launch is: what comes after it in the
+    // stream may be a programmatic dependent of this grid alone (launch_first), and
+    // neither an in-CTA segment nor a CTA without an item waits for the first launch.
+    // Where a CTA returns without having waited, the last one does.
+    auto last_cta_waits = [&]() {
+        if (blockIdx.x == gridDim.x - 1) asm volatile("griddepcontrol.wait;" ::: "memory");
+    };
     auto small_item = [&](uint32_t i) {
         const unsigned long long ts = (a.prof && tid == 0) ? global_ns() : 0ull;
         const BatchItem it = a.items[DEV ? devplan_pos(dev_lb(a), kListSmall2, i) : a.n_first + a.n_scan + i];
@@ -683,10 +690,14 @@ __global__ void __launch_bounds__(kScanCtaThreads, 6) seg_scan_kernel(BatchArgs 
         // too) every chunk ran about twice as slow, measured.
         const uint32_t grid = gridDim.x;
         if (grid >= n_small2 + n_scan) {
-            if (blockIdx.x >= n_small2 + n_scan) return;
+            if (blockIdx.x >= n_small2 + n_scan) {
+                last_cta_waits();
+                return;
+            }
             if (blockIdx.x < n_small2) {
                 asm volatile("griddepcontrol.launch_dependents;");
                 small_item(blockIdx.x);
+                last_cta_waits();
                 return;
             }
             if (tid == 0) s_ticket = atomicAdd(&a.ctl->scan_ticket, 1u);
@@ -723,6 +734,7 @@ __global__ void __launch_bounds__(kScanCtaThreads, 6) seg_scan_kernel(BatchArgs 
         // An in-CTA segment: independent of the first launch, so no wait.
         asm volatile("griddepcontrol.launch_dependents;");
         small_item(blockIdx.x);
+        last_cta_waits();
         return;
     }
     // The ticket and the chunk's descriptors come from plan data, not from
@@ -736,6 +748,7 @@ __global__ void __launch_bounds__(kScanCtaThreads, 6) seg_scan_kernel(BatchArgs 
         // ticket stood for is never published, so the output launch must not
         // trust the run tables.
         if (tid == 0) atomicOr(&a.ctl->status, kDevTimeout);
+        last_cta_waits();
         return;
     }
     const BatchItem it = a.items[a.n_first + s_ticket];

@@ -1,0 +1,49 @@
+"""Calls in a row on one stream, whose kernels may overlap: each finds what the call
+before it wrote."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import dev_keys, stream_handle
+from paper_2609_00843_gb300 import gen, rtcdf
+
+pytestmark = pytest.mark.gpu
+
+
+# A segmented sort of in-CTA segments only: those over wide ranges keep the first
+# launch busy long after the second one has sorted the few others.  The sort after it
+# reads what the first launch writes.
+@pytest.mark.parametrize("planned", ["host", "device"])
+def test_sort_after_a_segmented_sort_without_scan_items(planned):
+    s, S, n, R = stream_handle(), 1520, 60_000, 55_000
+    lengths = np.full(S, n, np.int64)
+    lengths[::100] = 50
+    ranges = np.where(lengths == n, R, 100)
+    offs = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+    x = dev_keys(int(offs[-1]), 0, 100, gen.UNIFORM, 51)
+    for i in range(S):
+        if lengths[i] == n:
+            gen.keys_device(x.data_ptr() + 4 * int(offs[i]), n, 0, R, gen.UNIFORM, gen.derive_seed(52, i), stream=s)
+    out = torch.empty_like(x)
+    mn, mx = np.zeros(S, np.int64), ranges
+    if planned == "host":
+        plan = rtcdf.BatchPlan(offs, mn, mx)
+        wsb = plan.workspace_size()
+    else:
+        meta = [torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in (offs, mn, mx)]
+        wsb = rtcdf.rtcdf_batch_device_workspace_size(S, int(offs[-1]), R)
+    ws = torch.zeros(wsb // 4, dtype=torch.int32, device="cuda")
+    m, at = 24_000, 17_000
+    back = torch.empty(m, dtype=torch.int32, device="cuda")
+    for i in (1, S // 2 + 1, S - 2) * 6:
+        out.fill_(7)
+        lo = int(offs[i])
+        if planned == "host":
+            assert plan.run(x.data_ptr(), out.data_ptr(), ws.data_ptr(), wsb, s) == rtcdf.OK
+        else:
+            assert rtcdf.rtcdf_sort_batched_device_ws(x.data_ptr(), out.data_ptr(), *[t.data_ptr() for t in meta], S,
+                                                      int(offs[-1]), R, ws.data_ptr(), wsb, s) == rtcdf.OK
+        assert rtcdf.rtcdf_sort(out.data_ptr() + 4 * (lo + at), back.data_ptr(), m, 0, R, s) == rtcdf.OK
+        assert torch.equal(back, x[lo:lo + n].sort().values[at:at + m])
+    assert rtcdf.rtcdf_status_get(s) == (rtcdf.OK, 0)
+    assert rtcdf.rtcdf_batch_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
