@@ -425,12 +425,16 @@ rtcdf_status rtcdf_sort_batched_host(const int32_t *in, int32_t *out, const int6
  *
  * rtcdf_sort_batched uses a library-owned workspace per (device, stream),
  * grown on demand by stream-ordered allocation (inside CUDA graph capture it
- * must already be large enough: rtcdf_batch_reserve) and cleared when a call's
- * bounds differ from the last call's; rtcdf_status_get reads its status.  rtcdf_sort_batched_device_ws takes a caller workspace
- * (256-byte aligned, zero-filled before its first use, left ready for the
- * next call of any layout within the same bounds; calls sharing it must be
- * ordered): no allocation, so it can be captured in a CUDA graph and replayed
- * with new keys AND new segment metadata.  Its status: rtcdf_batch_status_get.
+ * must already be large enough: rtcdf_batch_reserve); it is cleared when a
+ * sort's bounds differ from those of the sort before it in the workspace.  Once
+ * a graph holds a sort in it, one more launch per sort finds that out on the
+ * device, where replays and calls come in an order the host does not know.
+ * rtcdf_status_get reads its status.  rtcdf_sort_batched_device_ws takes a
+ * caller workspace (256-byte aligned, zero-filled before its first use, left
+ * ready for the next call of any layout within the same bounds; calls sharing
+ * it must be ordered): no allocation, so it can be captured in a CUDA graph
+ * and replayed with new keys AND new segment metadata.  Its status:
+ * rtcdf_batch_status_get.
  * Host-side errors (returned at once, nothing enqueued): RTCDF_ERR_INVALID_ARG
  * for S < 0, max_total_keys >= 2^40, null or misaligned pointers, in/out
  * partial overlap; RTCDF_ERR_RANGE for max_R outside 1..2^20;

@@ -67,8 +67,13 @@ struct BatchCtl {
     uint32_t first_ticket;  // device-built lists: items of the first launch taken so far
                             // (reset by the planner before the first launch)
     uint32_t plan_ticket;   // device planner: CTAs in start order (reset by the output launch)
-    uint32_t pad[60];
+    // Device planner: the bounds (DevBounds) of the last run, whose layout the workspace
+    // is in; S = 0 in a workspace that is zero.
+    uint32_t plan_S, plan_max_R;
+    uint64_t plan_keys;
+    uint32_t pad[56];
 };
+static_assert(sizeof(BatchCtl) == 256, "control block is 64 words");
 
 struct BatchArgs {
     const int32_t *in;

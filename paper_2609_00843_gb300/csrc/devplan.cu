@@ -115,6 +115,9 @@ __global__ void __launch_bounds__(1024) devplan_kernel(DevPlanArgs p) {
     if (blk == 0 && sub == 0 && tid == 0) {  // the previous run has finished (stream order)
         ctl->first_ticket = 0;
         ctl->scan_ticket = 0;
+        ctl->plan_S = p.b.S;
+        ctl->plan_max_R = p.b.max_R;
+        ctl->plan_keys = p.b.max_total_keys;
     }
     const uint32_t S = p.b.S, s = blk * 1024 + tid;
     DevSegCount c{};
@@ -249,11 +252,29 @@ __global__ void __launch_bounds__(1024) devplan_kernel(DevPlanArgs p) {
     }
 }
 
+// Other bounds lay a workspace out in another way: what must be zero there holds lists
+// and run tables of the last run.  Clears it (all but the control block, whose tickets
+// every run leaves zero) when the last run's bounds, which the planner has left in the
+// control block, are not `next`.  The device decides: a graph's replays and the
+// calls between them come in an order that the host does not see.
+constexpr int kClearThreads = 512;
+__global__ void __launch_bounds__(kClearThreads) devplan_clear_kernel(uint32_t *ws, size_t words, DevBounds next) {
+    const BatchCtl *ctl = reinterpret_cast<const BatchCtl *>(ws);
+    if (ctl->plan_S == 0 || (ctl->plan_S == next.S && ctl->plan_max_R == next.max_R &&
+                             ctl->plan_keys == next.max_total_keys))
+        return;
+    constexpr size_t first = sizeof(BatchCtl) / 16;
+    for (size_t i = first + (size_t)blockIdx.x * kClearThreads + threadIdx.x; i < words / 4;
+         i += (size_t)gridDim.x * kClearThreads)
+        reinterpret_cast<uint4 *>(ws)[i] = make_uint4(0, 0, 0, 0);
+}
+
 // Library-owned workspaces of rtcdf_sort_batched, per (device, stream).
 struct BatchCache {
     void *ptr = nullptr;
     size_t bytes = 0;
     DevBounds used{0, 0, 0};  // of the last sort in it (S = 0: none since it was cleared)
+    bool captured = false;    // a graph holds a sort in it
 };
 std::mutex g_bmu;
 std::map<std::pair<int, cudaStream_t>, BatchCache> g_bws;
@@ -291,16 +312,23 @@ rtcdf_status grow_cache(cudaStream_t s, size_t need, const DevBounds *next, void
         c->ptr = p;
         c->bytes = need;
         c->used = DevBounds{0, 0, 0};
+        c->captured = false;
         if (old && cudaFreeAsync(old, s) != cudaSuccess) return RTCDF_ERR_CUDA;
     }
     if (next) {
-        // Other bounds lay the workspace out in another way: what must be zero
-        // there holds lists and run tables of the last sort.  (All but the status
-        // word at its start.)
+        // The check is a launch of its own, left out while it has nothing to find: no
+        // graph holds a sort in this workspace, and the last one had the same bounds.
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return RTCDF_ERR_CUDA;
+        if (cap != cudaStreamCaptureStatusNone) c->captured = true;
         const DevBounds &u = c->used;
-        if (u.S && (u.S != next->S || u.max_R != next->max_R || u.max_total_keys != next->max_total_keys) &&
-            cudaMemsetAsync((char *)c->ptr + 4, 0, need - 4, s) != cudaSuccess)
-            return RTCDF_ERR_CUDA;
+        if (c->captured ||
+            (u.S && (u.S != next->S || u.max_R != next->max_R || u.max_total_keys != next->max_total_keys))) {
+            int sms = 0;
+            if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return RTCDF_ERR_CUDA;
+            devplan_clear_kernel<<<4 * sms, kClearThreads, 0, s>>>((uint32_t *)c->ptr, need / 4, *next);
+            if (cudaGetLastError() != cudaSuccess) return RTCDF_ERR_CUDA;
+        }
         c->used = *next;
     }
     *ptr = c->ptr;

@@ -6,6 +6,7 @@ import torch
 
 from gpu_util import dev_keys, stream_handle
 from paper_2609_00843_gb300 import gen, rtcdf
+from test_batched_gpu import check_segments, make_segments
 
 pytestmark = pytest.mark.gpu
 
@@ -47,3 +48,57 @@ def test_sort_after_a_segmented_sort_without_scan_items(planned):
         assert torch.equal(back, x[lo:lo + n].sort().values[at:at + m])
     assert rtcdf.rtcdf_status_get(s) == (rtcdf.OK, 0)
     assert rtcdf.rtcdf_batch_status_get(ws.data_ptr(), s) == (rtcdf.OK, 0)
+
+
+class Segments:
+    """One layout, sorted in the library's workspace of a stream."""
+
+    def __init__(self, lengths, Rs, max_R, stream):
+        S = len(lengths)
+        self.x, self.offs, self.mn, self.mx = make_segments(lengths, Rs, [-7] * S, [i % 3 for i in range(S)], range(S))
+        self.out = torch.empty_like(self.x)
+        self.meta = [torch.from_numpy(v).cuda() for v in (self.offs, self.mn, self.mx)]
+        self.max_R, self.s = max_R, stream
+
+    def reserve(self):
+        assert rtcdf.rtcdf_batch_reserve(len(self.mn), self.x.numel(), self.max_R, self.s) == rtcdf.OK
+
+    def sort(self):
+        return rtcdf.rtcdf_sort_batched(self.x.data_ptr(), self.out.data_ptr(), *[t.data_ptr() for t in self.meta],
+                                        len(self.mn), self.x.numel(), self.max_R, self.s)
+
+    def check(self, sort):
+        self.out.fill_(0x7FFFFFFF)
+        torch.cuda.synchronize()
+        assert sort() in (None, rtcdf.OK)
+        assert rtcdf.rtcdf_status_get(self.s) == (rtcdf.OK, 0)
+        check_segments(self.x, self.out, self.offs, self.mn, self.mx)
+
+
+# The library's workspace is in the layout of the bounds of the sort before, which is a
+# call or a graph's replay: the host sees the calls only.  (R: Y is replayed; C: Y is
+# captured; the others are calls.)
+@pytest.mark.parametrize("order", ["XCYRXRR", "CXRXR", "CYXYRX", "XYCXRZRZYR"])
+def test_segmented_sorts_and_replays_with_other_bounds(order):
+    stream = torch.cuda.Stream()
+    s = stream.cuda_stream
+    runs = {"X": Segments([200_001, 70_000, 5, 131_073], [1 << 20, 1 << 16, 3, 70_000], 1 << 20, s),
+            "Y": Segments([2000 + 7 * i for i in range(300)] + [70_000], [4096 - i for i in range(300)] + [4096], 4096, s),
+            "Z": Segments([66_000, 90_000, 1000], [5000, 4097, 100], 5000, s)}
+    for r in runs.values():
+        r.reserve()
+    graph = torch.cuda.CUDAGraph()
+
+    def replay():
+        with torch.cuda.stream(stream):
+            graph.replay()
+
+    torch.cuda.synchronize()
+    for step in order:
+        if step == "C":
+            with torch.cuda.graph(graph, stream=stream):
+                assert runs["Y"].sort() == rtcdf.OK
+        elif step == "R":
+            runs["Y"].check(replay)
+        else:
+            runs[step].check(runs[step].sort)
