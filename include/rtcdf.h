@@ -143,8 +143,14 @@ typedef struct {
     int32_t reserved[2];
 } rtcdf_params;
 
-/* The parameters rtcdf_sort would use for (n, R) on the current device
- * (tuning table first, then the built-in rules). */
+/* The parameters of the general kernels (one launch each for histogram, scan and
+ * output) for (n, R) on the current device: tuning table first, then the built-in
+ * rules.  Where neither the caller nor an entry of a table that rtcdf_tune_set has set
+ * gives parameters, rtcdf_sort may take other kernels instead (one launch for small
+ * arrays, packed counters or a partition for the histogram, scan and output in one
+ * launch); explicit parameters, these among them, select the general ones, except that
+ * a histogram without a tile width, CTAs or threads may still be packed or
+ * partitioned. */
 rtcdf_status rtcdf_plan(uint64_t n, int64_t R, rtcdf_params *params);
 
 /*
@@ -153,7 +159,7 @@ rtcdf_status rtcdf_plan(uint64_t n, int64_t R, rtcdf_params *params);
  * keyed by the range class ceil(log2 R) and the input-size class of n; a
  * range/size pair with no entry, or an entry whose parameters do not fit the
  * current device, falls back to the built-in rules (zero fields of an entry
- * also keep the built-in choice).  The table starts as the one compiled into
+ * also keep the built-in choice, an entry of zeros all of it).  The table starts as the one compiled into
  * the library (measured on GB300 with rtcdf_autotune); rtcdf_tune_set replaces
  * it, rtcdf_tune_reset restores the compiled-in one.  The input distribution
  * is not a key: the sort cannot know it before its histogram, so the tuner
@@ -189,7 +195,9 @@ rtcdf_status rtcdf_tune_get(rtcdf_tune_entry *entries, int32_t capacity, int32_t
  *
  * cases[i].in / .out are device arrays of .n keys in [.minVal, .maxVal);
  * `workspace` (256-byte aligned, zero-filled before first use, then kept as
- * rtcdf_sort_ws keeps it) holds at least rtcdf_workspace_size(max R) bytes.  Host outputs:
+ * rtcdf_sort_ws keeps it) holds at least rtcdf_workspace_size(max R) bytes.
+ * A candidate of zeros is timed as what rtcdf_sort does for a class without an entry:
+ * the built-in rules, with their choice of kernels (rtcdf_plan).  Host outputs:
  * times_ms[c * num_candidates + k] (median ms; -1 if candidate k cannot run
  * case c on this device), geomean[k] (HUGE_VAL for a candidate that cannot
  * run every case), *best.  Synchronises `stream`; not capturable.  Returns

@@ -66,7 +66,7 @@ struct Plan {
     bool streaming;
     bool hist_long;     // one tile of a long input (hist_long_kernel)
     bool shape_given;   // the histogram's shape comes from the caller or the tuning table
-    bool fill_given;    // the output's shape comes from the caller
+    bool given;         // parameters of the caller or of an entry in the caller's tuning table
     int sms;
     uint32_t head;
     uint64_t nvec;
@@ -156,7 +156,7 @@ rtcdf_status make_plan_with(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t
     // Not clamped to n: positions below head_out are written one by one, and
     // the vector frame must stay 16-byte aligned.
     const uint32_t head_out = (uint32_t)(((16 - (out_addr & 15)) & 15) / 4);
-    pl->fill_given = p != nullptr;
+    pl->given = p != nullptr;
     const bool short_fill = short_runs(n, R) && !q.fill_threads && !q.fill_ctas && !q.fill_chunk;
     pl->fill_threads = q.fill_threads ? q.fill_threads : short_fill ? 256 : 512;
     if (pl->fill_threads != 256 && pl->fill_threads != 512 && pl->fill_threads != 1024)
@@ -204,11 +204,9 @@ rtcdf_status make_plan(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t out_
     const bool found = tune_lookup(n, R, &t, &builtin);
     // (the compiled-in table's output shapes are those of the kernel's form for long runs)
     if (found && builtin && short_runs(n, R)) t.fill_ctas = t.fill_threads = t.fill_chunk = 0;
-    if (!(found && make_plan_with(n, R, in_addr, out_addr, &t, pl) == RTCDF_OK)) {
-        const rtcdf_status st = make_plan_with(n, R, in_addr, out_addr, nullptr, pl);
-        if (st) return st;
-    }
-    pl->fill_given = !tune_is_builtin();
+    if (!(found && make_plan_with(n, R, in_addr, out_addr, &t, pl) == RTCDF_OK))
+        return make_plan_with(n, R, in_addr, out_addr, nullptr, pl);
+    pl->given = !builtin;
     return RTCDF_OK;
 }
 
@@ -224,6 +222,17 @@ rtcdf_status check_args(const int32_t *in, int32_t *out, uint64_t n) {
     if (((uintptr_t)in & 3) || ((uintptr_t)out & 3)) return RTCDF_ERR_INVALID_ARG;
     if ((const void *)in != (const void *)out && overlaps(in, out, n)) return RTCDF_ERR_INVALID_ARG;
     return RTCDF_OK;
+}
+
+// The arguments of rtcdf_sort_ex (nothing beyond the range for an empty array).
+rtcdf_status check_sort_ex(const int32_t *in, int32_t *out, uint64_t n, int64_t minVal, int64_t maxVal,
+                           const void *workspace, size_t ws_bytes, uint32_t *R) {
+    rtcdf_status st = check_range(minVal, maxVal, R);
+    if (st || n == 0) return st;
+    st = check_args(in, out, n);
+    if (st) return st;
+    if (!workspace || ((uintptr_t)workspace & 255)) return RTCDF_ERR_INVALID_ARG;
+    return ws_bytes < ws_required(*R) ? RTCDF_ERR_NO_MEMORY : RTCDF_OK;
 }
 
 constexpr uint32_t kWideOutMinR = 1000000;  // (use_wide_out)
@@ -308,7 +317,7 @@ rtcdf_status finish_phase(int32_t *out, uint64_t n, int64_t minVal, uint32_t R, 
     // alignment does not matter).
     const uint32_t head_out =
         (uint32_t)std::min<uint64_t>(((16 - ((uintptr_t)out & 15)) & 15) / 4, pos_end - pos_base);
-    if (!dbg && !pl.fill_given && R <= kSmallMaxR && pos_end - pos_base <= kFinishMaxN) {
+    if (!dbg && !pl.given && R <= kSmallMaxR && pos_end - pos_base <= kFinishMaxN) {
         FinishArgs f;
         f.H = (uint32_t *)(base + L.hist); f.out = out; f.n = (uint32_t)n;
         f.pos_base = (uint32_t)pos_base; f.pos_end = (uint32_t)pos_end;
@@ -349,7 +358,7 @@ rtcdf_status run_pipeline(const int32_t *in, int32_t *out, uint64_t n, int64_t m
     if (ev[0] && cudaEventRecord(ev[0], s) != cudaSuccess) return RTCDF_ERR_CUDA;
     // (a sort in place has no scratch)
     bool parted = false;
-    const bool wide = !dbg && !pl.fill_given && use_wide_out(n, R);
+    const bool wide = !dbg && !pl.given && use_wide_out(n, R);
     uint32_t *half = (uint32_t *)(base + L.scan_state) + 2 * kPartMaxBuckets;
     rtcdf_status st = hist_phase(in, n, minVal, R, pl, (uint32_t *)(base + L.hist), (Ctl *)(base + L.ctl),
                                  in == out ? 0 : (uintptr_t)out, (uint32_t *)(base + L.start_run),
@@ -367,19 +376,24 @@ rtcdf_status run_pipeline(const int32_t *in, int32_t *out, uint64_t n, int64_t m
 }
 
 // One sort with checked arguments in a workspace of at least ws_required(R) bytes.
+// rules: by the built-in rules whatever the tuning table holds (params is null).
 rtcdf_status sort_checked(const int32_t *in, int32_t *out, uint64_t n, int64_t minVal, uint32_t R,
                           const rtcdf_params *params, void *ws, size_t ws_bytes, const rtcdf_debug *dbg,
-                          cudaStream_t s) {
+                          cudaStream_t s, bool rules = false) {
     // Small arrays in one launch (small.cu), unless the caller asks for launch
-    // parameters, intermediates or stage events.
-    if (n <= kSmallMaxN && R <= kSmallMaxR && !params && !dbg && tune_is_builtin())
-        return launch_small(in, out, (uint32_t)n, (uint32_t)(int32_t)minVal, R, (Ctl *)ws, s) == cudaSuccess
-                   ? RTCDF_OK
-                   : RTCDF_ERR_CUDA;
+    // parameters, intermediates or stage events.  (The compiled-in table has no say in
+    // them: no plan is made to find that out.)
+    const bool small = n <= kSmallMaxN && R <= kSmallMaxR && !params && !dbg;
     Plan pl;
-    const rtcdf_status st = make_plan(n, R, (uintptr_t)in, (uintptr_t)out, params, &pl);
-    if (st) return st;
-    return run_pipeline(in, out, n, minVal, R, pl, ws, ws_bytes, dbg, s);
+    if (!(small && (rules || tune_is_builtin()))) {
+        const rtcdf_status st = rules ? make_plan_with(n, R, (uintptr_t)in, (uintptr_t)out, nullptr, &pl)
+                                      : make_plan(n, R, (uintptr_t)in, (uintptr_t)out, params, &pl);
+        if (st) return st;
+        if (!small || pl.given) return run_pipeline(in, out, n, minVal, R, pl, ws, ws_bytes, dbg, s);
+    }
+    return launch_small(in, out, (uint32_t)n, (uint32_t)(int32_t)minVal, R, (Ctl *)ws, s) == cudaSuccess
+               ? RTCDF_OK
+               : RTCDF_ERR_CUDA;
 }
 
 // ---------------------------------------------------------------- workspace cache
@@ -461,6 +475,15 @@ rtcdf_status sort_with_workspace(const int32_t *in, int32_t *out, uint64_t n, in
     return sort_checked(in, out, n, minVal, R, nullptr, ws, ws_bytes, nullptr, s);
 }
 
+// A sort with checked arguments by the built-in rules, for rtcdf_autotune.
+rtcdf_status sort_by_rules(const int32_t *in, int32_t *out, uint64_t n, int64_t minVal, int64_t maxVal, void *ws,
+                           size_t ws_bytes, cudaStream_t s) {
+    uint32_t R = 0;
+    const rtcdf_status st = check_sort_ex(in, out, n, minVal, maxVal, ws, ws_bytes, &R);
+    if (st || n == 0) return st;
+    return sort_checked(in, out, n, minVal, R, nullptr, ws, ws_bytes, nullptr, s, true);
+}
+
 // The two halves of a sort, for rtcdf_sort_host: histogram of a slice (may be
 // called once per uploaded chunk), then scan + output for the whole array.
 rtcdf_status host_pipeline_hist(const int32_t *in, uint64_t n, int64_t minVal, uint32_t R, void *ws,
@@ -528,13 +551,8 @@ rtcdf_status rtcdf_sort_ex(const int32_t *in, int32_t *out, uint64_t n, int64_t 
                            int64_t maxVal, const rtcdf_params *params, void *workspace,
                            size_t ws_bytes, const rtcdf_debug *debug, rtcdf_stream_t stream) {
     uint32_t R = 0;
-    rtcdf_status st = check_range(minVal, maxVal, &R);
-    if (st) return st;
-    if (n == 0) return RTCDF_OK;
-    st = check_args(in, out, n);
-    if (st) return st;
-    if (!workspace || ((uintptr_t)workspace & 255)) return RTCDF_ERR_INVALID_ARG;
-    if (ws_bytes < ws_required(R)) return RTCDF_ERR_NO_MEMORY;
+    const rtcdf_status st = check_sort_ex(in, out, n, minVal, maxVal, workspace, ws_bytes, &R);
+    if (st || n == 0) return st;
     return sort_checked(in, out, n, minVal, R, params, workspace, ws_bytes, debug, (cudaStream_t)stream);
 }
 

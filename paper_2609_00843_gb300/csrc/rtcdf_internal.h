@@ -12,10 +12,14 @@
 namespace rtcdf {
 
 // Launch parameters of the tuning table for (n, R), if it has an entry
-// (tune.cu); whether the table is the compiled-in one.
+// (tune.cu) that sets any of them; whether the table is the compiled-in one.
 bool tune_lookup(uint64_t n, uint32_t R, rtcdf_params *out, bool *builtin);
 // Whether the tuning table is the compiled-in one.
 bool tune_is_builtin();
+
+// rtcdf_sort_ex by the built-in rules, whatever the tuning table holds (rtcdf_api.cu).
+rtcdf_status sort_by_rules(const int32_t *in, int32_t *out, uint64_t n, int64_t minVal, int64_t maxVal, void *ws,
+                           size_t ws_bytes, cudaStream_t s);
 
 // Device status bits (mirror RTCDF_DEV_* in rtcdf.h).
 constexpr uint32_t kDevKeyOutOfRange = 0x1;

@@ -39,6 +39,11 @@ int32_t log2_ceil(uint32_t R) {
     return l;
 }
 
+// Every choice left to the built-in rules.
+bool no_params(const rtcdf_params &p) {
+    return !p.tile_width && !p.hist_ctas_per_tile && !p.hist_threads && !p.fill_ctas && !p.fill_threads && !p.fill_chunk;
+}
+
 }  // namespace
 
 namespace rtcdf {
@@ -61,7 +66,7 @@ bool tune_lookup(uint64_t n, uint32_t R, rtcdf_params *out, bool *builtin) {
         if (it->log2_R == lr && it->n_class == nc) {
             *out = it->params;
             *builtin = g_builtin;
-            return true;
+            return !no_params(*out);
         }
     }
     return false;
@@ -135,15 +140,21 @@ rtcdf_status rtcdf_autotune(const rtcdf_tune_case *cases, int32_t num_cases,
         for (int32_t k = 0; k < num_candidates; k++) {
             float &cell = times_ms[(size_t)c * num_candidates + k];
             cell = -1.0f;
-            // One untimed sort; a candidate that cannot run here is skipped.
-            rtcdf_status st = rtcdf_sort_ex(tc.in, tc.out, tc.n, tc.minVal, tc.maxVal, &candidates[k],
-                                            workspace, ws_bytes, nullptr, stream);
+            // One untimed sort; a candidate that cannot run here is skipped.  A candidate of
+            // zeros is what a class without an entry gets: the rules' own choice of kernels,
+            // which explicit parameters pass by.
+            auto sort = [&]() {
+                return no_params(candidates[k])
+                           ? rtcdf::sort_by_rules(tc.in, tc.out, tc.n, tc.minVal, tc.maxVal, workspace, ws_bytes, s)
+                           : rtcdf_sort_ex(tc.in, tc.out, tc.n, tc.minVal, tc.maxVal, &candidates[k], workspace,
+                                           ws_bytes, nullptr, stream);
+            };
+            rtcdf_status st = sort();
             if (st == RTCDF_ERR_INVALID_ARG) continue;
             if (st) { result = st; break; }
             if (cudaEventRecord(ev[0], s) != cudaSuccess) { result = RTCDF_ERR_CUDA; break; }
             for (int32_t r = 0; r < reps && result == RTCDF_OK; r++) {
-                st = rtcdf_sort_ex(tc.in, tc.out, tc.n, tc.minVal, tc.maxVal, &candidates[k], workspace,
-                                   ws_bytes, nullptr, stream);
+                st = sort();
                 if (st) result = st;
                 else if (cudaEventRecord(ev[(size_t)r + 1], s) != cudaSuccess) result = RTCDF_ERR_CUDA;
             }
