@@ -260,23 +260,10 @@ __host__ __device__ inline uint32_t devplan_hist_class(uint64_t keys, uint64_t h
     return keys >= hist_chunk / 2 ? 0u : keys >= hist_chunk / 4 ? 1u : 2u;
 }
 
-// Whether an in-CTA sort of the scan launch (256 threads: about 5 us + 1.05 ns
-// per key + 1.9 ns per value) would outlast the rest of that launch, which the
-// output launch waits for: the segment is split into work items instead.  The
-// device planner knows only the number of segments when it classifies one; the
-// launch takes about 42 ns for each (six CTAs per SM, measured on the benchmark's
-// shapes), and 20 us at least.
-__host__ __device__ inline bool devplan_outlasts(uint32_t n, uint32_t R, uint32_t S) {
-    const uint64_t launch_ns = 42ull * S > 20000 ? 42ull * S : 20000;
-    return 5000 + 21ull * n / 20 + 19ull * R / 10 > launch_ns;
-}
-
-// Segment s from its metadata: its descriptor (workspace offsets left to the
-// caller) and its items per list, as build_host_plan classifies it; false
-// when it breaks the bounds or the limits of a segmented sort.
+// A segment from its metadata, its classification (m and what follows) left out;
+// false when it breaks the bounds or the limits of a segmented sort.
 __host__ __device__ inline bool devplan_segment(int64_t o0, int64_t o1, int64_t mn, int64_t mx, const DevBounds &b,
-                                                const BatchTuning &t, BatchSeg *g, DevSegCount *c) {
-    for (uint32_t i = 0; i < kNumLists; i++) c->v[i] = 0;
+                                                BatchSeg *g) {
     *g = BatchSeg{};
     if (o0 < 0 || o1 < o0 || (uint64_t)o1 > b.max_total_keys) return false;
     const uint64_t n = (uint64_t)(o1 - o0);
@@ -286,12 +273,42 @@ __host__ __device__ inline bool devplan_segment(int64_t o0, int64_t o1, int64_t 
     g->n = (uint32_t)n;
     g->R = (uint32_t)(mx - mn);
     g->minVal = (int32_t)mn;
-    if (n == 0) return true;
-    if (g->n <= t.small_max_n && g->R <= kBatchSmallMaxR &&
-        !(t.small_by_time && g->R <= t.small_scan_max_R && devplan_outlasts(g->n, g->R, b.S))) {
+    return true;
+}
+
+// An in-CTA sort of the scan launch (256 threads: about 5 us + 1.05 ns per key +
+// 1.9 ns per value) that outlasts the rest of that launch, which the output launch
+// waits for, can be split into work items instead.  Its estimated time if it
+// outlasts the launch, else 0.  The launch takes about 42 ns for each of the S
+// segments (six CTAs per SM, measured on the benchmark's shapes), and 20 us at least.
+// Few keys over a wide range (n <= R / 8) are done in about 10 us, whatever the
+// estimate says: a value without keys costs 0.3 ns.
+__host__ __device__ inline uint32_t devplan_outlasts(const BatchSeg &g, uint32_t S, const BatchTuning &t) {
+    if (!t.small_by_time || g.n == 0 || g.n > t.small_max_n || g.R > t.small_scan_max_R || g.n <= g.R / 8) return 0;
+    const uint64_t ns = 5000 + 21ull * g.n / 20 + 19ull * g.R / 10;
+    return ns > 20000 && ns > 42ull * S ? (uint32_t)ns : 0u;
+}
+
+// Whether they are split: `count` of a block's segments outlast the launch, the
+// longest of them by its estimate.  Their work items take about 45 ns each, and 25 us
+// more for the three launches' chain.  Measured (us, split / not; log-uniform keys and
+// values): 500 segments of 1e3 ... 6e4 keys over 128 ... 16000 values 58 / 92, 1024 85 / 115,
+// of 1e4 ... 1e5 keys 91 / 180 and 136 / 198; 256 equal segments of 6e4 keys over 16000 80 /
+// 190; but 400 of 8000 keys over 4000 70 / 39, 1024 of 20000 over 16000 189 / 135.
+__host__ __device__ inline bool devplan_split(uint32_t count, uint32_t longest_ns, uint32_t S) {
+    return longest_ns > 25000 + 45ull * count * ((S + 1023) / 1024);
+}
+
+// The rest of a segment's descriptor (workspace offsets left to the caller) and its
+// items per list, as build_host_plan classifies it.  split: it is not to be sorted in
+// one CTA.
+__host__ __device__ inline void devplan_classify(const BatchTuning &t, bool split, BatchSeg *g, DevSegCount *c) {
+    for (uint32_t i = 0; i < kNumLists; i++) c->v[i] = 0;
+    if (g->n == 0) return;
+    if (g->n <= t.small_max_n && g->R <= kBatchSmallMaxR && !split) {
         if (g->R <= t.small_scan_max_R) c->v[kListSmall2] = 1;
         else c->v[kListSmall1] = 1;
-        return true;
+        return;
     }
     g->m = (g->R + kBatchTileMax - 1) / kBatchTileMax;
     g->T = (g->R + g->m - 1) / g->m;
@@ -312,7 +329,6 @@ __host__ __device__ inline bool devplan_segment(int64_t o0, int64_t o1, int64_t 
     c->v[g->scan_chunks >= kLongChain ? kListScan0 : kListScan1] = g->scan_chunks;
     c->v[kListFill0 + devplan_fill_class(t.fill_chunk, *g)] = fwhole;
     if (frest) c->v[kListFill0 + devplan_fill_class(frest, *g)] += 1;
-    return true;
 }
 
 // The k-th item of list `list` that belongs to segment s (k counted within the

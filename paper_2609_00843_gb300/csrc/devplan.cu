@@ -7,7 +7,7 @@
 // Each segment is still sorted by Algorithms 4-7 (Section 3); the plan is the
 // same three work lists as the host planner's (batch_api.cu), built by one
 // kernel: eight CTAs each classify the same 1024 segments (the rules of
-// devplan_segment, batched.h), scan their item counts per list, get the counts
+// devplan_classify, batched.h), scan their item counts per list, get the counts
 // of the segments before from the CTAs before them (a decoupled lookback over
 // CTAs taken in start order, every wait bounded), and write an eighth of the
 // segments' descriptors and items each.  The lists sit at fixed offsets (the bounds of the
@@ -92,17 +92,26 @@ __global__ void __launch_bounds__(1024) devplan_kernel(DevPlanArgs p) {
     __shared__ uint32_t s_warp[kNumLists][32];
     __shared__ uint32_t s_tot[kLookCounts], s_base[kLookCounts];
     __shared__ uint32_t s_n[1024], s_R[1024];   // keys and range of the block's segments
-    __shared__ uint32_t s_ticket;
+    __shared__ uint32_t s_ticket, s_count, s_longest;
     __shared__ int s_bad;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     BatchCtl *ctl = reinterpret_cast<BatchCtl *>(p.ws + p.L.ctl);
     BatchSeg *segs = reinterpret_cast<BatchSeg *>(p.ws + p.L.segs);
     BatchItem *items = reinterpret_cast<BatchItem *>(p.ws + p.L.items);
     DevLook *look = reinterpret_cast<DevLook *>(p.ws + p.L.look);
+    // Offsets, minVal and maxVal of the thread's segment; those of the only block
+    // are on their way while the ticket is drawn.
+    const uint32_t S = p.b.S;
+    int64_t meta[4] = {0, 0, 0, 0};
+    auto load_meta = [&](uint32_t s) {
+        if (s < S) meta[0] = p.offs[s], meta[1] = p.offs[s + 1], meta[2] = p.mn[s], meta[3] = p.mx[s];
+    };
+    if (p.L.look_blocks == 1) load_meta(tid);
     // CTAs in start order, so a CTA only waits for CTAs already running.
     if (tid == 0) {
         s_ticket = atomicAdd(&ctl->plan_ticket, 1u);
         s_bad = 0;
+        s_count = s_longest = 0;
     }
     __syncthreads();
     const uint32_t blk = s_ticket / kPlanSplit, sub = s_ticket % kPlanSplit;
@@ -119,10 +128,19 @@ __global__ void __launch_bounds__(1024) devplan_kernel(DevPlanArgs p) {
         ctl->plan_max_R = p.b.max_R;
         ctl->plan_keys = p.b.max_total_keys;
     }
-    const uint32_t S = p.b.S, s = blk * 1024 + tid;
+    const uint32_t s = blk * 1024 + tid;
+    if (p.L.look_blocks > 1) load_meta(s);
     DevSegCount c{};
     BatchSeg g{};
-    if (s < S && !devplan_segment(p.offs[s], p.offs[s + 1], p.mn[s], p.mx[s], p.b, p.t, &g, &c)) s_bad = 1;
+    if (s < S && !devplan_segment(meta[0], meta[1], meta[2], meta[3], p.b, &g)) s_bad = 1;
+    const uint32_t ns = devplan_outlasts(g, S, p.t);  // (0 for the empty ones past the last)
+    const unsigned outlast = __ballot_sync(0xffffffffu, ns > 0);
+    if (outlast) {
+        const uint32_t longest = __reduce_max_sync(0xffffffffu, ns);
+        if (lane == 0) atomicAdd(&s_count, (uint32_t)__popc(outlast)), atomicMax(&s_longest, longest);
+    }
+    __syncthreads();
+    devplan_classify(p.t, ns > 0 && devplan_split(s_count, s_longest, S), &g, &c);
     const uint32_t *v = c.v;
     uint32_t inc[kNumLists];
 #pragma unroll
@@ -378,10 +396,22 @@ int devplan_host(const int64_t *offs, const int64_t *mn, const int64_t *mx, cons
     memset(hdr, 0, sizeof(*hdr));
     items->clear();
     DevPfx run{};
+    uint32_t count = 0, longest = 0;  // of the block of 1024 segments
     for (uint32_t s = 0; s < S; s++) {
+        if (s % 1024 == 0) {
+            count = longest = 0;
+            for (uint32_t i = s; i < std::min(S, s + 1024); i++) {
+                BatchSeg g;
+                if (!devplan_segment(offs[i], offs[i + 1], mn[i], mx[i], b, &g)) return RTCDF_ERR_INVALID_ARG;
+                const uint32_t ns = devplan_outlasts(g, S, t);
+                count += ns > 0;
+                longest = std::max(longest, ns);
+            }
+        }
         DevSegCount c;
         BatchSeg g;
-        if (!devplan_segment(offs[s], offs[s + 1], mn[s], mx[s], b, t, &g, &c)) return RTCDF_ERR_INVALID_ARG;
+        devplan_segment(offs[s], offs[s + 1], mn[s], mx[s], b, &g);
+        devplan_classify(t, devplan_outlasts(g, S, t) > 0 && devplan_split(count, longest, S), &g, &c);
         (*pfx)[s] = run;
         if (g.m > 0) {
             const size_t slot = L.slots + (size_t)s * L.slot_words;
