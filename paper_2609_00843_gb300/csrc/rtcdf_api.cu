@@ -93,7 +93,7 @@ constexpr uint64_t kHistLongMinN = 200000000;  // (see hist_long_kernel)
 // Choose the launch shape (Section 3.3): tile width T from shared memory, CTAs
 // per tile from occupancy, output CTAs from n.
 rtcdf_status make_plan_with(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t out_addr,
-                            const rtcdf_params *p, Plan *pl) {
+                            const rtcdf_params *p, bool alone, Plan *pl) {
     DeviceInfo dev;
     rtcdf_status st = device_info(&dev);
     if (st) return st;
@@ -118,7 +118,12 @@ rtcdf_status make_plan_with(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t
         T = m == 1 ? R : std::min(t_max, ((R + m - 1) / m + 1023) & ~1023u);
         // Small arrays just past one tile: four, whose clearing and merging is less
         // than the keys' extra passes (n = 1e5, R = 60000 16.5 us against 18.5).
-        if (m == 2 && R <= 65536 && rtcdf_tune_n_class(n) == 0) T = 16384;
+        const bool small = rtcdf_tune_n_class(n) == RTCDF_TUNE_N_SMALL;
+        if (m == 2 && R <= 65536 && small) T = 16384;
+        // A histogram alone: so too where a tile would hold the range, since its clearing
+        // overlaps no earlier launch (n = 1e4 ... 1e6, R = 30000 6.2 us against 8.2, 50000 8.2
+        // against 10.3).
+        if (m == 1 && R > 16384 && small && alone) T = R > 32768 ? 16384 : 11264;
     }
     if (T > t_max) return RTCDF_ERR_INVALID_ARG;
     if (T > R) T = R;
@@ -196,16 +201,17 @@ rtcdf_status make_plan_with(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t
 // Explicit parameters are used as given; without them the tuning table is
 // tried first and the built-in rules cover what it lacks (or what does not fit
 // this device).
+// alone: for a histogram that no sort follows at once.
 rtcdf_status make_plan(uint64_t n, uint32_t R, uintptr_t in_addr, uintptr_t out_addr,
-                       const rtcdf_params *p, Plan *pl) {
-    if (p) return make_plan_with(n, R, in_addr, out_addr, p, pl);
+                       const rtcdf_params *p, Plan *pl, bool alone = false) {
+    if (p) return make_plan_with(n, R, in_addr, out_addr, p, alone, pl);
     rtcdf_params t;
     bool builtin = false;
     const bool found = tune_lookup(n, R, &t, &builtin);
     // (the compiled-in table's output shapes are those of the kernel's form for long runs)
     if (found && builtin && short_runs(n, R)) t.fill_ctas = t.fill_threads = t.fill_chunk = 0;
-    if (!(found && make_plan_with(n, R, in_addr, out_addr, &t, pl) == RTCDF_OK))
-        return make_plan_with(n, R, in_addr, out_addr, nullptr, pl);
+    if (!(found && make_plan_with(n, R, in_addr, out_addr, &t, alone, pl) == RTCDF_OK))
+        return make_plan_with(n, R, in_addr, out_addr, nullptr, alone, pl);
     pl->given = !builtin;
     return RTCDF_OK;
 }
@@ -386,7 +392,7 @@ rtcdf_status sort_checked(const int32_t *in, int32_t *out, uint64_t n, int64_t m
     const bool small = n <= kSmallMaxN && R <= kSmallMaxR && !params && !dbg;
     Plan pl;
     if (!(small && (rules || tune_is_builtin()))) {
-        const rtcdf_status st = rules ? make_plan_with(n, R, (uintptr_t)in, (uintptr_t)out, nullptr, &pl)
+        const rtcdf_status st = rules ? make_plan_with(n, R, (uintptr_t)in, (uintptr_t)out, nullptr, false, &pl)
                                       : make_plan(n, R, (uintptr_t)in, (uintptr_t)out, params, &pl);
         if (st) return st;
         if (!small || pl.given) return run_pipeline(in, out, n, minVal, R, pl, ws, ws_bytes, dbg, s);
@@ -490,7 +496,7 @@ rtcdf_status host_pipeline_hist(const int32_t *in, uint64_t n, int64_t minVal, u
                                 size_t ws_bytes, cudaStream_t s) {
     if (n == 0) return RTCDF_OK;
     Plan pl;
-    rtcdf_status st = make_plan(n, R, (uintptr_t)in, 0, nullptr, &pl);
+    rtcdf_status st = make_plan(n, R, (uintptr_t)in, 0, nullptr, &pl, true);
     if (st) return st;
     return hist_phase(in, n, minVal, R, pl, (uint32_t *)((char *)ws + ws_layout(R, ws_bytes).hist), nullptr, 0, nullptr,
                       nullptr, nullptr, s);
@@ -597,7 +603,7 @@ rtcdf_status rtcdf_hist_accumulate(const int32_t *in, uint64_t n, int64_t minVal
         if (x < y + (uint64_t)R * 4 && y < x + n * 4) return RTCDF_ERR_INVALID_ARG;
     }
     Plan pl;
-    st = make_plan(n, R, (uintptr_t)in, 0, nullptr, &pl);
+    st = make_plan(n, R, (uintptr_t)in, 0, nullptr, &pl, true);
     if (st) return st;
     // Algorithm 5 for every tile, added straight into the caller's counts.
     return hist_phase(in, n, minVal, R, pl, counts, nullptr, 0, nullptr, nullptr, nullptr, (cudaStream_t)stream);

@@ -68,3 +68,15 @@ def test_autotune_times_the_rules_with_their_kernels():
     ws.zero_()
     t, gm, best = rtcdf.rtcdf_autotune(cases, [rtcdf.Params(), rtcdf.Params(hist_threads=512)], 3, ws.data_ptr(), wsb, s)
     assert all(v > 0 for v in t[0])
+
+
+# A histogram alone: several tiles for small arrays over a range that one would hold.
+@pytest.mark.parametrize("R", [16_384, 16_385, 32_768, 32_769, 57_344, 57_345])
+@pytest.mark.parametrize("n", [1, 70_003, (1 << 20) - 1, 1 << 20])
+def test_histogram_alone(R, n):
+    x = torch.empty(n + 1, dtype=torch.int32, device="cuda")[1:]
+    gen.keys_device(x.data_ptr(), n, -4, R, gen.NORMAL, gen.derive_seed(64, R, n), stream=stream_handle())
+    counts = torch.zeros(R, dtype=torch.int32, device="cuda")
+    for k in (1, 2):
+        assert rtcdf.rtcdf_hist_accumulate(x.data_ptr(), n, -4, R - 4, counts.data_ptr(), stream_handle()) == rtcdf.OK
+        assert torch.equal(counts.long(), k * torch.bincount(x + 4, minlength=R))
