@@ -26,11 +26,11 @@
 
 namespace rtcdf {
 
-template <bool STREAMING, int UNROLL, bool ADAPT>
+template <bool STREAMING, int UNROLL, bool ADAPT, bool FIXED = false>
 __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a) {
     extern __shared__ uint32_t S[];
     __shared__ uint32_t s_tc[8];
-    hist_tiles<STREAMING, UNROLL, ADAPT>(a, blockIdx.x, S, s_tc);
+    hist_tiles<STREAMING, UNROLL, ADAPT, ADAPT, FIXED>(a, blockIdx.x, S, s_tc);
 }
 
 // One tile of a long input: one CTA per SM, whose 64 registers a thread hold six
@@ -40,14 +40,16 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a) {
 // 134.4 / 133.5), and two leave room for other streams' kernels.
 __global__ void __launch_bounds__(1024, 1) hist_long_kernel(HistArgs a) {
     extern __shared__ uint32_t S[];
-    hist_tiles<true, 6, false, true>(a, blockIdx.x, S, nullptr);
+    hist_tiles<true, 6, false, true, true>(a, blockIdx.x, S, nullptr);
 }
 
 // Kernel variant: streaming loads for one tile; the adaptive form for 2 to 8
-// tiles; the plain predicated form beyond.
-enum HistVariant { kHistStreaming = 0, kHistAdaptive = 1, kHistPlain = 2 };
-int hist_variant(bool streaming, uint32_t m) {
-    return streaming ? kHistStreaming : (m <= 8 ? kHistAdaptive : kHistPlain);
+// tiles; the plain predicated form beyond.  The first two also for launches that are
+// not a sort's first (FIXED), which may have nothing to count.
+enum HistVariant { kHistStreaming, kHistAdaptive, kHistPlain, kHistStreamingFixed, kHistAdaptiveFixed };
+int hist_variant(bool streaming, uint32_t m, bool fixed) {
+    if (streaming) return fixed ? kHistStreamingFixed : kHistStreaming;
+    return m > 8 ? kHistPlain : fixed ? kHistAdaptiveFixed : kHistAdaptive;
 }
 
 const void *hist_fn(int variant, int unroll) {
@@ -57,6 +59,12 @@ const void *hist_fn(int variant, int unroll) {
             return deep ? (const void *)hist_kernel<true, 8, false> : (const void *)hist_kernel<true, 4, false>;
         case kHistAdaptive:
             return deep ? (const void *)hist_kernel<false, 8, true> : (const void *)hist_kernel<false, 4, true>;
+        case kHistStreamingFixed:
+            return deep ? (const void *)hist_kernel<true, 8, false, true>
+                        : (const void *)hist_kernel<true, 4, false, true>;
+        case kHistAdaptiveFixed:
+            return deep ? (const void *)hist_kernel<false, 8, true, true>
+                        : (const void *)hist_kernel<false, 4, true, true>;
         default:
             return deep ? (const void *)hist_kernel<false, 8, false> : (const void *)hist_kernel<false, 4, false>;
     }
@@ -67,13 +75,22 @@ const void *hist_fn(int variant, int unroll) {
 // the 2-to-8-tile form.
 int hist_unroll(size_t smem) { return smem > 114 * 1024 ? 8 : 4; }
 
-cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool streaming, bool first, cudaStream_t s) {
+constexpr uint64_t kHistFixedMinKeys = 500000000;  // (see launch_hist)
+
+cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool streaming, HistLaunch how, cudaStream_t s) {
     // hist_max_ctas_per_sm() has raised the shared-memory limits for this size.
     dim3 grid(a.m * a.g);
     void *args[] = {const_cast<HistArgs *>(&a)};
-    const void *fn = hist_fn(hist_variant(streaming, a.m), hist_unroll(smem));
+    // Loads of a fixed input (ld.global.nc) are faster over long inputs of few values
+    // (n = 3e8, R = 200000, 100 different keys: 467 us against 562).  The first launch of
+    // a sort may overlap the kernel that writes its input, and gains by it up to about
+    // 1e8 keys (n = 2e7, R = 2^18, whole sort 83 / 87); over longer inputs it does not.
+    if (how == kHistFirst && !streaming && a.m <= 8 && a.n * a.m >= kHistFixedMinKeys) how = kHistAlone;
+    const bool fixed = streaming ? a.only_if != nullptr : how != kHistFirst;
+    const void *fn = hist_fn(hist_variant(streaming, a.m, fixed), hist_unroll(smem));
     if (a.long_form) fn = (const void *)hist_long_kernel;
-    if (first) return launch_first(fn, grid.x, threads, smem, args, s);
+    if (how == kHistFirst) return launch_first(fn, grid.x, threads, smem, args, s);
+    if (how == kHistDependent) return launch_dependent(fn, grid.x, threads, smem, args, true, s);
     return cudaLaunchKernel(fn, grid, dim3(threads), args, smem, s);
 }
 
@@ -97,8 +114,8 @@ cudaError_t hist_max_ctas_per_sm(int threads, size_t smem, bool streaming, int *
     const void *f = hist_fn(streaming ? kHistStreaming : kHistAdaptive, hist_unroll(smem));
     size_t &lim = smem_limit[std::make_pair(dev, streaming)];
     if (smem > lim) {
-        for (int v : {kHistStreaming, kHistAdaptive, kHistPlain}) {
-            if ((v == kHistStreaming) != streaming) continue;
+        for (int v : {kHistStreaming, kHistAdaptive, kHistPlain, kHistStreamingFixed, kHistAdaptiveFixed}) {
+            if ((v == kHistStreaming || v == kHistStreamingFixed) != streaming) continue;
             for (int u : {4, 8}) {
                 e = cudaFuncSetAttribute(hist_fn(v, u), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 if (e != cudaSuccess) return e;

@@ -7,10 +7,13 @@
 
 namespace rtcdf {
 
-template <bool STREAMING>
+// FIXED: not the first launch of a sort, so that the input does not change while the
+// kernel is resident.
+template <bool STREAMING, bool FIXED = false>
 __device__ __forceinline__ int4 load_vec(const int4 *p) {
     if (STREAMING) return __ldcs(p);  // read once: evict first
-    return __ldcg(p);                 // re-read by the other tiles' CTAs: keep in L2
+    if (FIXED) return __ldg(p);       // re-read by the other tiles' CTAs: keep in L2
+    return __ldcg(p);
 }
 
 // S[y] += 1 when y < w, as a predicated shared-memory reduction (no branch).
@@ -50,7 +53,7 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
 // CTA `cta` of m * g: tile cta mod m, the (cta / m)-th of the tile's g CTAs.  S is
 // the tile's shared memory (the tile, and the trash word if ADAPT), s_tc eight
 // words of it.
-template <bool STREAMING, int UNROLL, bool ADAPT, bool PIPE = ADAPT>
+template <bool STREAMING, int UNROLL, bool ADAPT, bool PIPE = ADAPT, bool FIXED = false>
 __device__ __forceinline__ void hist_tiles(const HistArgs &a, uint32_t cta, uint32_t *S, uint32_t *s_tc) {
     const uint32_t t = cta % a.m;
     const uint32_t q = cta / a.m;
@@ -62,6 +65,7 @@ __device__ __forceinline__ void hist_tiles(const HistArgs &a, uint32_t cta, uint
     if (ADAPT && tid < 8) s_tc[tid] = 0;
     __syncthreads();
     asm volatile("griddepcontrol.wait;" ::: "memory");  // (launch_first)
+    if (FIXED && a.only_if && __ldcg(a.only_if) == 0) return;
 
     const uint32_t base = a.min_u + b;  // key - base = position inside the tile
     const uint32_t s_base = (uint32_t)__cvta_generic_to_shared(S);
@@ -113,7 +117,7 @@ __device__ __forceinline__ void hist_tiles(const HistArgs &a, uint32_t cta, uint
         for (; v + (UNROLL - 1) * stride < nvec; v += UNROLL * stride) {
             int4 k[UNROLL];
 #pragma unroll
-            for (int u = 0; u < UNROLL; u++) k[u] = load_vec<STREAMING>(vin + v + u * stride);
+            for (int u = 0; u < UNROLL; u++) k[u] = load_vec<STREAMING, FIXED>(vin + v + u * stride);
 #pragma unroll
             for (int u = 0; u < UNROLL; u++) count_vec(k[u]);
         }
@@ -127,7 +131,7 @@ __device__ __forceinline__ void hist_tiles(const HistArgs &a, uint32_t cta, uint
         if (v + (P - 1) * stride < nvec) {
             int4 kn[P];
 #pragma unroll
-            for (int u = 0; u < P; u++) kn[u] = load_vec<STREAMING>(vin + v + u * stride);
+            for (int u = 0; u < P; u++) kn[u] = load_vec<STREAMING, FIXED>(vin + v + u * stride);
             v += P * stride;
             vb += P * stride;
             for (; v + (P - 1) * stride < nvec; v += P * stride, vb += P * stride) {
@@ -144,7 +148,7 @@ __device__ __forceinline__ void hist_tiles(const HistArgs &a, uint32_t cta, uint
 #pragma unroll
                 for (int u = 0; u < P; u++) kc[u] = kn[u];
 #pragma unroll
-                for (int u = 0; u < P; u++) kn[u] = load_vec<STREAMING>(vin + v + u * stride);
+                for (int u = 0; u < P; u++) kn[u] = load_vec<STREAMING, FIXED>(vin + v + u * stride);
 #pragma unroll
                 for (int u = 0; u < P; u++) count_vec(kc[u]);
             }
@@ -153,7 +157,7 @@ __device__ __forceinline__ void hist_tiles(const HistArgs &a, uint32_t cta, uint
         }
     }
     for (; v < nvec; v += stride) {
-        int4 k0 = load_vec<STREAMING>(vin + v);
+        int4 k0 = load_vec<STREAMING, FIXED>(vin + v);
         count_key(s_base, (uint32_t)k0.x - base, w);
         count_key(s_base, (uint32_t)k0.y - base, w);
         count_key(s_base, (uint32_t)k0.z - base, w);

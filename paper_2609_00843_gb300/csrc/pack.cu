@@ -19,7 +19,8 @@
 //   - an input that would need too many rounds (several frequent keys, or a
 //     range of which only a small part is used), or whose neighbours are alike
 //     (sorted or clustered keys: they fill a field within one block of the
-//     input, and the lanes of a warp meet on a word) is counted by range tiles.
+//     input, and the lanes of a warp meet on a word) is counted by range tiles,
+//     here or by a launch of hist.cu of its own (kPackTilesLaunchMin).
 //
 // The fields leave the CTA as they are, 32 MB for R = 2^18, into the sort's
 // output buffer (which nothing reads before the output kernel fills it), and
@@ -89,7 +90,10 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack_kernel(PackArgs a) {
     // After a wait that ran out nothing is written to the output (nor to its
     // use as scratch) until the status has been read.
     if (a.dump && (a.ctl->status & kDevTimeout)) {
-        if (blockIdx.x == 0 && tid == 0) a.ctl->pack_copies = 0;
+        if (blockIdx.x == 0 && tid == 0) {
+            a.ctl->pack_copies = 0;
+            if (a.tiles_later) *a.tiles_later = 0;
+        }
         return;
     }
 
@@ -183,9 +187,12 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack_kernel(PackArgs a) {
     const float want = ceilf(fullest / a.limit);
     const bool tiles = want > (float)a.max_rounds || (int)s_near > (int)(kSampleVecs * kPackThreads / 16);
     const uint32_t rounds = tiles ? 0u : max(1u, (uint32_t)want);
-    if (blockIdx.x == 0 && tid == 0 && a.dump) a.ctl->pack_copies = rounds * gridDim.x;
+    if (blockIdx.x == 0 && tid == 0) {
+        if (a.dump) a.ctl->pack_copies = rounds * gridDim.x;
+        if (a.tiles_later) *a.tiles_later = tiles;
+    }
     if (tiles) {
-        if (blockIdx.x < h.m * h.g) hist_tiles<false, 8, true>(h, blockIdx.x, S, s_tc);
+        if (!a.tiles_later && blockIdx.x < h.m * h.g) hist_tiles<false, 8, true>(h, blockIdx.x, S, s_tc);
         return;
     }
 
@@ -431,7 +438,7 @@ bool pack_plan(uint64_t n, uint32_t R, uint64_t nvec, uintptr_t scratch, int sms
     return true;
 }
 
-cudaError_t launch_pack(const PackPlan &p, const HistArgs &hist, Ctl *ctl, cudaStream_t s) {
+cudaError_t launch_pack(const PackPlan &p, const HistArgs &hist, Ctl *ctl, bool tiles_later, cudaStream_t s) {
     PackArgs a;
     a.h = hist;
     a.h.T = p.tile; a.h.m = p.m; a.h.g = p.g;
@@ -440,6 +447,7 @@ cudaError_t launch_pack(const PackPlan &p, const HistArgs &hist, Ctl *ctl, cudaS
     while (((hist.R - 1) >> a.coarse_shift) >= kCoarse) a.coarse_shift++;
     a.dump = ctl ? reinterpret_cast<uint32_t *>(p.dump) : nullptr;
     a.ctl = ctl;
+    a.tiles_later = tiles_later ? &ctl->pack_tiles : nullptr;
     void *args[] = {&a};
     static std::atomic<uint64_t> raised{0};
     cudaError_t e = raise_shared_limit((const void *)pack_kernel, kPackSmem, raised);

@@ -12,7 +12,7 @@
 //
 // Unlike the paper's host driver there is no device-to-host copy of the tile
 // offsets and no per-tile launch loop: every launch size is known from (n, R)
-// alone, so a sort is one to four stream-ordered launches with no host
+// alone, so a sort is one to five stream-ordered launches with no host
 // synchronisation and can be captured in a CUDA graph.
 #include <algorithm>
 #include <cstring>
@@ -266,6 +266,17 @@ bool use_part(uint64_t n, const Plan &pl, uintptr_t scratch, PartPlan *pp) {
     return part_plan(n, pl.R, pl.head, pl.nvec, scratch, pl.sms, pp);
 }
 
+// Inputs that packed counters cannot hold (frequent keys, sorted ones) are counted by range
+// tiles: over long inputs by a launch of their own, with the widest tiles, which finds
+// nothing to do otherwise.  In pack_kernel's launch a tile is no wider than the packed
+// counters, so that more passes are needed: whole sorts, us, there / own launch / range
+// tiles from the start, n = 3e8, R = 200000 log-uniform keys 895 / 834 / 820, 100 different
+// keys 762 / 648 / 641, sorted 647 / 633 / 630; but n = 1e8, R = 2^18 359 / 344 / 336, 286 / 274
+// / 264 and 259 / 267 / 260, R = 350000 multiples of 1024 499 / 583 / 625.  The launch costs
+// the others 0.7 us at n = 1e8 (uniform, 160.2 / 160.9), 3 us at 2e7 (69.9 / 73.0) and at n =
+// 1e9, R = 2^16 (1139 / 1142), whose tiles are two either way.
+constexpr uint64_t kPackTilesLaunchMin = 1000000000;
+
 // Algorithm 5 (all tiles) into H (R counters).  H accumulates, so several calls
 // over slices of one array add up to the array's histogram.  ctl and scratch (n
 // words, 0 if there are none): of a whole sort, as bucket_start and half (or null)
@@ -280,12 +291,17 @@ rtcdf_status hist_phase(const int32_t *in, uint64_t n, int64_t minVal, uint32_t 
     PackPlan pack;
     PartPlan part;
     cudaError_t e;
-    if (use_pack(n, pl, scratch, &pack))
-        e = launch_pack(pack, h, ctl, s);
-    else if (ctl && (*parted = use_part(n, pl, scratch, &part)))
+    if (use_pack(n, pl, scratch, &pack)) {
+        const bool tiles_later = ctl && pack.m > pl.m && n * pl.m >= kPackTilesLaunchMin;
+        e = launch_pack(pack, h, ctl, tiles_later, s);
+        if (tiles_later && e == cudaSuccess) {
+            h.only_if = &ctl->pack_tiles;
+            e = launch_hist(h, pl.hist_threads, pl.hist_smem, pl.streaming, kHistDependent, s);
+        }
+    } else if (ctl && (*parted = use_part(n, pl, scratch, &part)))
         e = launch_part(part, in, n, pl.head, pl.nvec, h.min_u, R, H, bucket_start, half, ctl, pl.sms, s);
     else
-        e = launch_hist(h, pl.hist_threads, pl.hist_smem, pl.streaming, ctl != nullptr, s);
+        e = launch_hist(h, pl.hist_threads, pl.hist_smem, pl.streaming, ctl ? kHistFirst : kHistAlone, s);
     return e == cudaSuccess ? RTCDF_OK : RTCDF_ERR_CUDA;
 }
 

@@ -51,7 +51,8 @@ struct Ctl {
     uint32_t part_ticket;  // items of bucket_kernel taken so far (zero between sorts)
     uint32_t pack_copies;  // written-out counters of pack_kernel (written before it is read)
     uint32_t finished;     // CTAs of finish_kernel that have read H (zero between sorts)
-    uint32_t pad[58];
+    uint32_t pack_tiles;   // whether pack_kernel has left the keys to range tiles (written before it is read)
+    uint32_t pad[57];
 };
 static_assert(sizeof(Ctl) == 256, "control block is 256 bytes");
 
@@ -115,6 +116,21 @@ inline cudaError_t raise_shared_limit(const void *kernel, size_t bytes, std::ato
     return e;
 }
 
+inline cudaError_t launch_dependent(const void *fn, uint32_t grid, int threads, size_t smem, void **args,
+                                    bool dependent, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
 // The first launch of a sort: a programmatic dependent of whatever kernel is before
 // it in the stream, unless the stream is being captured (whose last node may be of
 // another kind).  The kernel waits for that one before it reads or writes anything
@@ -129,17 +145,7 @@ inline cudaError_t launch_first(const void *fn, uint32_t grid, int threads, size
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const cudaError_t e = cudaStreamIsCapturing(s, &cap);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
-    return cudaLaunchKernelExC(&cfg, fn, args);
+    return launch_dependent(fn, grid, threads, smem, args, cap == cudaStreamCaptureStatusNone, s);
 }
 
 // ---------------------------------------------------------------- histogram
@@ -152,9 +158,13 @@ struct HistArgs {
     uint32_t R, T, m, g;   // range size, tile width, tiles, CTAs per tile
     uint32_t *H;           // global histogram, R entries (added to)
     bool long_form = false;  // one tile, one CTA per SM: hist_long_kernel
+    const uint32_t *only_if = nullptr;  // nothing is counted when this word is 0
 };
-// first: of a whole sort.
-cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool streaming, bool first, cudaStream_t s);
+// How the histogram is launched: after all earlier work in the stream, as the first
+// launch of a whole sort (launch_first), or as a programmatic dependent of the sort's
+// launch before it.
+enum HistLaunch { kHistAlone, kHistFirst, kHistDependent };
+cudaError_t launch_hist(const HistArgs &a, int threads, size_t smem, bool streaming, HistLaunch how, cudaStream_t s);
 cudaError_t hist_max_ctas_per_sm(int threads, size_t smem, bool streaming, int *ctas);
 
 // ---------------------------------------------------------------- small arrays
@@ -189,6 +199,7 @@ struct PackArgs {
     uint32_t max_rounds;
     uint32_t *dump;        // written-out counters, or null: added to H by pairs of CTAs
     Ctl *ctl;              // (with dump)
+    uint32_t *tiles_later; // written: whether the keys are left to range tiles; null: counted by them here
 };
 struct PackPlan {
     uint32_t words, fields, magic, max_rounds, ctas, tile, m, g;
@@ -199,8 +210,10 @@ struct PackPlan {
 // The plan for n keys over R values; scratch: n words, or 0.  False when the
 // range does not fit.
 bool pack_plan(uint64_t n, uint32_t R, uint64_t nvec, uintptr_t scratch, int sms, PackPlan *p);
-// ctl: the control block of a whole sort, or null (no scratch).
-cudaError_t launch_pack(const PackPlan &p, const HistArgs &hist, Ctl *ctl, cudaStream_t s);
+// ctl: the control block of a whole sort, or null (no scratch).  tiles_later: keys that
+// packed counters cannot hold are left to a launch of the range tiles that follows
+// (Ctl::pack_tiles).
+cudaError_t launch_pack(const PackPlan &p, const HistArgs &hist, Ctl *ctl, bool tiles_later, cudaStream_t s);
 
 // ---------------------------------------------------------------- histogram by partition
 constexpr int kPartShift = 15;  // values per bucket, log2
