@@ -58,17 +58,17 @@ __device__ __forceinline__ void fill_short_runs(uint32_t *m, const uint32_t *s_e
     int4 *m4 = reinterpret_cast<int4 *>(m);
     int j = first_run_after(s_end, 0, nw - 1, frame + 4 * wb);  // the run of the block's first position
     for (uint32_t w = wb; w < we; w += BLK / 4) {
-        // The block's positions are q0 + i, i < len: its end is never formed, since
-        // q0 + BLK passes 2^32 in an array of nearly as many keys.
-        const uint32_t q0 = frame + 4 * w, len = min((uint32_t)BLK, 4 * (we - w));
+        // The block's last position: q0 + BLK passes 2^32 in an array of nearly as many keys.
+        const uint32_t q0 = frame + 4 * w, q_last = q0 + (min((uint32_t)BLK, 4 * (we - w)) - 1);
 #pragma unroll
         for (int k = 0; k < BLK / 128; k++) m4[lane + 32 * k] = make_int4(none, none, none, none);
         int32_t carry = key(j);
         __syncwarp();
         for (int r = j + 1 + lane;; r += 32) {
             const uint32_t start = r < nw ? s_end[r - 1] : 0xffffffffu;
-            const bool begins = start - q0 < len;  // (2^32 - 1 is no position of the block)
-            if (begins && (!CDF || s_end[r] > start)) m[start - q0] = (uint32_t)key(r);
+            const bool begins = start <= q_last;  // (2^32 - 1 is no position)
+            // (start < q0 only where a caller's counts pass 2^32: any place in the block)
+            if (begins && (!CDF || s_end[r] > start)) m[min(start - q0, (uint32_t)BLK - 1)] = (uint32_t)key(r);
             const unsigned b = __ballot_sync(0xffffffffu, begins);
             j += __popc(b);
             if (b != 0xffffffffu) break;
