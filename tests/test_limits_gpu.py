@@ -1,10 +1,10 @@
 """Outputs at the limits of the arithmetic: the last positions of the largest
-arrays, where 32-bit positions end, and counts whose sums pass 2^32."""
+arrays, where 32-bit positions end, counts whose sums pass 2^32, and the longest lists."""
 import pytest
 import torch
 
 from gpu_util import stream_handle
-from paper_2609_00843_gb300 import rtcdf
+from paper_2609_00843_gb300 import gen, rtcdf
 
 pytestmark = pytest.mark.gpu
 
@@ -141,3 +141,16 @@ def test_largest_segment(values, planned):
     assert torch.equal(out[N_MAX - values:N_MAX], torch.arange(R - values, R, device="cuda", dtype=torch.int32))
     assert int(torch.count_nonzero(out[:N_MAX - values])) == 0
     assert bool((out[N_MAX:] == -5).all())
+
+
+# The partition of so many keys that an item of the bucket kernel lists its slabs twice
+# (more than 4096 of 32768 keys; 128 buckets, four items each).
+def test_partition_of_more_slabs_than_a_list_holds():
+    n, R, mn, s = 600_000_003, 1 << 22, -(1 << 20), stream_handle()
+    x = torch.empty(n + 1, dtype=torch.int32, device="cuda")[1:]
+    gen.keys_device(x.data_ptr(), n, mn, R, gen.UNIFORM, gen.derive_seed(92, R), stream=s)
+    out = torch.empty_like(x)
+    assert rtcdf.rtcdf_sort(x.data_ptr(), out.data_ptr(), n, mn, mn + R, s) == rtcdf.OK
+    assert rtcdf.rtcdf_status_get(s) == (rtcdf.OK, 0)
+    counts = torch.bincount(x.sub_(mn), minlength=R)
+    assert torch.equal(out, torch.repeat_interleave(torch.arange(mn, mn + R, device="cuda", dtype=torch.int32), counts))
