@@ -940,10 +940,10 @@ def main():
     launches = len(cases) * nsteps
     if hist_total >= fill_total:
         kname, ktime = "hist_kernel", hist_total
-        ksrc = ["paper_2609_00843_gb300/csrc/hist.cu", "paper_2609_00843_gb300/csrc/rtcdf_internal.h"]
+        ksrc = ["hist.cu", "hist_tiles.cuh", "pack.cu", "rtcdf_internal.h"]
     else:
         kname, ktime = "fill_kernel", fill_total
-        ksrc = ["paper_2609_00843_gb300/csrc/fill.cu", "paper_2609_00843_gb300/csrc/rtcdf_internal.h"]
+        ksrc = ["fill.cu", "fill_runs.cuh", "rtcdf_internal.h"]
     avg_launch_s = ktime / launches * 1e-3
     achieved = 4 * n / avg_launch_s / 1e9  # algorithmic: 4n bytes read (hist) or written (fill)
     # The same fraction split by the form of the histogram: one shared-memory
@@ -957,7 +957,7 @@ def main():
                 for m, t in sorted(by_tiles.items())}
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
                 "frac": round(achieved / hbm, 4),
-                "traffic": traffic_for(kname, ksrc),
+                "traffic": traffic_for(kname, ["paper_2609_00843_gb300/csrc/" + f for f in ksrc]),
                 "kernel": kname, "peak_kind": f"{peak_kind} hbm_gbs (copy)",
                 "algorithmic_bytes_per_launch": 4 * n,
                 "by_range_tiles": by_tiles}
