@@ -936,10 +936,13 @@ __global__ void __launch_bounds__(kFillCtaThreads, 6) seg_fill_kernel(BatchArgs 
 
 // CTAs per output item: two at least (they have 256 threads), and enough for
 // about four waves of six CTAs per SM when the items are few.
-uint32_t fill_parts(uint64_t items) {
-    uint32_t parts = items <= 0x3fffffffu ? 2 : 1;  // (a grid has fewer than 2^31 CTAs)
-    while (parts < 16 && items * parts < 3648) parts *= 2;
-    return parts;
+static cudaError_t fill_parts(uint64_t items, uint32_t *parts) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    *parts = items <= 0x3fffffffu ? 2 : 1;  // (a grid has fewer than 2^31 CTAs)
+    while (*parts < 16 && items * *parts < 4 * 6 * (uint64_t)sms) *parts *= 2;
+    return e;
 }
 
 namespace {
@@ -964,9 +967,10 @@ cudaError_t launch_dep(const void *fn, uint32_t grid, int threads, const BatchAr
 
 cudaError_t launch_batched(const BatchArgs &args, cudaStream_t s) {
     BatchArgs a = args;
-    a.fill_parts = fill_parts(a.n_fill);
-    cudaError_t e = cudaFuncSetAttribute(seg_first_kernel<kFirstHost>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSegSmemBytes);
+    cudaError_t e = fill_parts(a.n_fill, &a.fill_parts);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(seg_first_kernel<kFirstHost>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kSegSmemBytes);
     if (e != cudaSuccess) return e;
     // A launch is a programmatic dependent only of the plan's own launch
     // before it (whose work it waits for, or which its CTAs do not read):
@@ -991,10 +995,11 @@ cudaError_t launch_batched(const BatchArgs &args, cudaStream_t s) {
 cudaError_t launch_batched_dev(const BatchArgs &args, uint32_t first_ctas, uint32_t scan_ctas, uint32_t fill_items,
                                cudaStream_t s) {
     BatchArgs a = args;
-    a.fill_parts = fill_parts(fill_items);
+    cudaError_t e = fill_parts(fill_items, &a.fill_parts);
+    if (e != cudaSuccess) return e;
     const void *first = a.num_segs < 700 ? (const void *)seg_first_kernel<kFirstTickets>
                                          : (const void *)seg_first_kernel<kFirstAhead>;
-    cudaError_t e = cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSmemBytes);
+    e = cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSmemBytes);
     if (e != cudaSuccess) return e;
     // The first launch waits for the planner; every launch runs (the lists
     // may be empty), so that the tickets are consumed and reset in order.

@@ -202,7 +202,7 @@ struct DevLayout {
     size_t slot_state, slot_run_end, slot_run_val;  // offsets inside a slot
     DevListBounds lb;
     uint64_t item_bound;
-    uint32_t look_blocks;  // planner CTAs (1024 segments each)
+    uint32_t look_blocks;  // blocks of 1024 segments (of several planner CTAs each)
 };
 
 // Position in the items array of list `list`'s element k (its base is the

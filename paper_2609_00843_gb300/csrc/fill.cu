@@ -17,7 +17,7 @@
 // positions instead (fill_runs.cuh).
 //
 // All positions are below n < 2^32, so the index arithmetic is 32-bit.  The
-// CTA also clears the scan's lookback state so the workspace is ready for the
+// CTA also clears the scan's published sums so the workspace is ready for the
 // next sort.
 #include "fill_runs.cuh"
 

@@ -64,7 +64,9 @@ __device__ __forceinline__ void hist_tiles(const HistArgs &a, uint32_t cta, uint
     for (uint32_t i = tid; i < w + (ADAPT ? 1u : 0u); i += nt) S[i] = 0;  // + the trash word
     if (ADAPT && tid < 8) s_tc[tid] = 0;
     __syncthreads();
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // (launch_first)
+    // The kernels before are done (launch_first).  Before anything else: the scan
+    // launched after this kernel relies on every CTA here having waited (scan.cu).
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (FIXED && a.only_if && __ldcg(a.only_if) == 0) return;
 
     const uint32_t base = a.min_u + b;  // key - base = position inside the tile

@@ -481,7 +481,7 @@ rtcdf_status read_status(void *ws, cudaStream_t s, int32_t *out) {
 namespace rtcdf {
 
 // Sort in a workspace whose previous contents are unknown: the regions that
-// must start at zero (control block, lookback state, histogram) are cleared
+// must start at zero (control block, the scan's sums, histogram) are cleared
 // on `s` first.  Used by rtcdf_sort_static.
 rtcdf_status sort_with_workspace(const int32_t *in, int32_t *out, uint64_t n, int64_t minVal,
                                  int64_t maxVal, void *ws, size_t ws_bytes, cudaStream_t s) {

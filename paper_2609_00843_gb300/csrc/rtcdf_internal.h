@@ -30,8 +30,9 @@ constexpr uint32_t kDevBadSegment = 0x4;
 // device, or null (devplan.cu).
 void *batch_stream_workspace(cudaStream_t s);
 
-// Local-CDF scan: one CTA of kScanThreads threads scans kScanChunk histogram
-// bins (kScanItems per thread); chunks are chained by a decoupled lookback.
+// Local-CDF scan: a CTA of kScanThreads threads scans kScanChunk histogram bins at a
+// time (kScanItems per thread), one chunk or a range of them; the CTAs exchange their
+// ranges' sums.
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanChunk = kScanThreads * kScanItems;
@@ -46,7 +47,7 @@ constexpr uint32_t kMaxSpin = 1u << 21;
 // Control block at the start of every workspace.
 struct Ctl {
     uint32_t status;       // RTCDF_DEV_* bits, sticky until read
-    uint32_t scan_ticket;  // dynamic chunk index of the lookback scan
+    uint32_t scan_ticket;  // chunk ranges of the scan handed out so far (zero between sorts)
     uint32_t num_runs;     // number of values with c_v > 0 (written by the scan)
     uint32_t part_ticket;  // items of bucket_kernel taken so far (zero between sorts)
     uint32_t pack_copies;  // written-out counters of pack_kernel (written before it is read)
@@ -56,12 +57,12 @@ struct Ctl {
 };
 static_assert(sizeof(Ctl) == 256, "control block is 256 bytes");
 
-// Most lookback chunks any sort can use (RTCDF_MAX_R / kScanChunk).
+// Most scan chunks any sort can have (RTCDF_MAX_R / kScanChunk).
 constexpr uint32_t kMaxScanChunks = (1u << 24) / kScanChunk;
 
 // Byte offsets of the workspace regions for a sort with range size R in a
 // workspace of `total` bytes.  Regions that must be zero when a sort starts
-// (control block, lookback state, histogram H) sit at fixed offsets from the
+// (control block, the scan's published sums, histogram H) sit at fixed offsets from the
 // bottom, so they stay zero whatever R the previous sort had; regions that
 // each sort writes before reading (run table, start-run table) are anchored
 // at the top and may overlap what a previous sort left behind.
@@ -173,7 +174,7 @@ struct SmallArgs {
     const int32_t *in;
     int32_t *out;
     uint32_t n, R, min_u;
-    uint32_t words, max_runs;  // shared memory: counters (and the output's blocks), runs
+    uint32_t max_runs;     // that shared memory has room for
     Ctl *ctl;
 };
 // The whole sort of n <= kSmallMaxN keys over R <= kSmallMaxR values in one CTA.
@@ -185,7 +186,7 @@ struct FinishArgs {
     uint32_t *H;           // R counts, zeroed
     int32_t *out;          // out[0] holds position pos_base
     uint32_t n, pos_base, pos_end, R, min_u;
-    uint32_t words, max_runs;  // (set by launch_finish)
+    uint32_t max_runs;     // (set by launch_finish)
     Ctl *ctl;
 };
 cudaError_t launch_finish(const FinishArgs &a, int sms, cudaStream_t s);
@@ -265,7 +266,7 @@ cudaError_t launch_wide_out(const WideOutArgs &a, int sms, cudaStream_t s);
 // ---------------------------------------------------------------- scan
 struct ScanArgs {
     uint32_t *H;           // histogram, zeroed as it is consumed
-    uint64_t *state;       // lookback state per chunk (zero on entry)
+    uint64_t *state;       // per scan CTA: the sum of its range, published (zero on entry)
     Ctl *ctl;
     uint32_t *run_end;     // inclusive CDF at each non-empty value (exclusive end of its run)
     int32_t *run_val;      // the key of each non-empty value

@@ -82,11 +82,12 @@ __global__ void __launch_bounds__(kScanThreads, 2) scan_kernel(ScanArgs a) {
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     // Launched as a programmatic dependent of the histogram.  The ticket does
-    // not depend on it (the counter was reset by the previous sort's output
-    // kernel, which finished before this sort's histogram began), so it is
-    // taken first; then wait until the histogram grid has finished and its
-    // writes are visible, and let the output kernel be scheduled (it waits for
-    // this grid in the same way).
+    // not depend on it, so it is taken first: the counter was reset by the previous
+    // sort's output kernel, which is done before any CTA here starts, because every
+    // CTA of the launch before waits for its own predecessors before it lets this one
+    // be scheduled or returns (as hist_tiles does).  Then wait until the histogram
+    // grid has finished and its writes are visible, and let the output kernel be
+    // scheduled (it waits for this grid in the same way).
     const bool single = (a.ctas == 1);  // no exchange at all
     if (!single) {
         if (tid == 0) s_slot = atomicAdd(&a.ctl->scan_ticket, 1u);

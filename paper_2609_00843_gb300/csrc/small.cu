@@ -22,6 +22,10 @@ namespace {
 
 constexpr int kSmallThreads = 1024;
 constexpr uint32_t kSmallWarps = kSmallThreads / 32;
+// The counters' words, which become a block per warp for the output.
+constexpr uint32_t kSmallWords = kSmallWarps * kBlock;
+static_assert(kSmallWords >= kSmallMaxR, "the blocks' words hold every counter");
+constexpr size_t kSmallSmem = 4 * (kSmallWords + 2 * (size_t)kSmallMaxR);  // of both kernels, at most
 
 // The run table of the R counts in S: run k's end (exclusive, the keys up to its
 // value) and key.  Returns the number of keys; *num_runs values are not empty.
@@ -70,7 +74,7 @@ __device__ __forceinline__ uint32_t runs_of_counts(const uint32_t *S, uint32_t R
 __global__ void __launch_bounds__(kSmallThreads, 1) small_kernel(SmallArgs a) {
     extern __shared__ __align__(16) uint32_t S[];  // counters, then the output's blocks | run ends | run keys
     __shared__ uint32_t s_keys[kSmallWarps], s_runs[kSmallWarps];
-    uint32_t *s_end = S + a.words;
+    uint32_t *s_end = S + kSmallWords;
     int32_t *s_val = reinterpret_cast<int32_t *>(s_end + a.max_runs);
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t n = a.n, R = a.R;
@@ -120,19 +124,17 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_kernel(SmallArgs a) {
     }
 }
 
-constexpr size_t kSmallSmem = 4 * 3 * (size_t)kSmallMaxR;  // of both kernels, at most
 
 cudaError_t launch_small(const int32_t *in, int32_t *out, uint32_t n, uint32_t min_u, uint32_t R, Ctl *ctl,
                          cudaStream_t s) {
     SmallArgs a;
     a.in = in; a.out = out; a.n = n; a.R = R; a.min_u = min_u; a.ctl = ctl;
-    a.words = R > kSmallWarps * kBlock ? (R + 3) / 4 * 4 : kSmallWarps * kBlock;
     a.max_runs = R < n ? R : n;
     static std::atomic<uint64_t> raised{0};
     const cudaError_t e = raise_shared_limit((const void *)small_kernel, kSmallSmem, raised);
     if (e != cudaSuccess) return e;
     void *args[] = {&a};
-    return launch_first((const void *)small_kernel, 1, kSmallThreads, 4 * ((size_t)a.words + 2 * (size_t)a.max_runs),
+    return launch_first((const void *)small_kernel, 1, kSmallThreads, 4 * (kSmallWords + 2 * (size_t)a.max_runs),
                         args, s);
 }
 
@@ -145,7 +147,7 @@ cudaError_t launch_small(const int32_t *in, int32_t *out, uint32_t n, uint32_t m
 __global__ void __launch_bounds__(kSmallThreads, 1) finish_kernel(FinishArgs a) {
     extern __shared__ __align__(16) uint32_t S[];  // counts, then the output's blocks | run ends | run keys
     __shared__ uint32_t s_keys[kSmallWarps], s_runs[kSmallWarps], s_last;
-    uint32_t *s_end = S + a.words;
+    uint32_t *s_end = S + kSmallWords;
     int32_t *s_val = reinterpret_cast<int32_t *>(s_end + a.max_runs);
     const uint32_t tid = threadIdx.x, warp = tid >> 5, R = a.R;
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -186,7 +188,6 @@ __global__ void __launch_bounds__(kSmallThreads, 1) finish_kernel(FinishArgs a) 
 
 cudaError_t launch_finish(const FinishArgs &args, int sms, cudaStream_t s) {
     FinishArgs a = args;
-    a.words = a.R > kSmallWarps * kBlock ? (a.R + 3) / 4 * 4 : kSmallWarps * kBlock;
     a.max_runs = a.R;
     static std::atomic<uint64_t> raised{0};
     cudaError_t e = raise_shared_limit((const void *)finish_kernel, kSmallSmem, raised);
@@ -194,7 +195,7 @@ cudaError_t launch_finish(const FinishArgs &args, int sms, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((uint32_t)std::min<uint64_t>(sms, ((uint64_t)a.pos_end - a.pos_base + 2047) / 2048));
     cfg.blockDim = dim3(kSmallThreads);
-    cfg.dynamicSmemBytes = 4 * ((size_t)a.words + 2 * (size_t)a.max_runs);
+    cfg.dynamicSmemBytes = 4 * (kSmallWords + 2 * (size_t)a.max_runs);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
