@@ -34,10 +34,11 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a) {
 }
 
 // One tile of a long input: one CTA per SM, whose 64 registers a thread hold six
-// vectors in flight while six are counted.  n = 1e9, R = 4096, whole sort, us: 1142 against
-// 1181 with two CTAs of 32 registers (2e8, R = 128 237 / 240); below 2e8 keys the two are
-// within 1 % of each other either way (1e8: R = 128 125.5 / 126.5, 16384 129.8 / 129.2, 49000
-// 134.4 / 133.5), and two leave room for other streams' kernels.
+// vectors in flight while six are counted.  Whole sorts one after another, us, against two
+// CTAs of 32 registers: n = 1e9, R = 128 1116 / 1142, 4096 1132 / 1158, 16384 1136 / 1176, 49000
+// 1124 / 1125; n = 2e8 246.0 / 246.9, 252.0 / 253.1, 252.3 / 255.8, 251.8 / 252.9; below 2e8 keys
+// the two are within 1 % of each other either way (1e8: R = 128 125.5 / 126.5, 16384 129.8 /
+// 129.2, 49000 134.4 / 133.5), and two leave room for other streams' kernels.
 __global__ void __launch_bounds__(1024, 1) hist_long_kernel(HistArgs a) {
     extern __shared__ uint32_t S[];
     hist_tiles<true, 6, false, true, true>(a, blockIdx.x, S, nullptr);
