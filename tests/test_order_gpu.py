@@ -1,5 +1,7 @@
 """Calls in a row on one stream, whose kernels may overlap: each finds what the call
 before it wrote."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -102,3 +104,34 @@ def test_segmented_sorts_and_replays_with_other_bounds(order):
             runs["Y"].check(replay)
         else:
             runs[step].check(runs[step].sort)
+
+
+# A sort whose first launch may overlap the kernel before it in its stream, and whose
+# input another stream writes after that kernel: behind an event, and on the legacy
+# default stream behind a stream that it waits for by itself.
+@pytest.mark.parametrize("n,R", [(20_000, 1000), (1_000_000, 5000), (3_000_001, 50_021), (400_000, 300_000)])
+@pytest.mark.parametrize("legacy", [False, True])
+def test_sort_of_what_another_stream_writes(n, R, legacy):
+    cuda = ctypes.CDLL("libcuda.so.1")
+    handle = ctypes.c_void_p()
+    assert cuda.cuStreamCreate(ctypes.byref(handle), 0) == 0          # (waits for the legacy stream, and it for this one)
+    other = torch.cuda.ExternalStream(handle.value)
+    mine = torch.cuda.default_stream() if legacy else torch.cuda.Stream()
+    x = [dev_keys(n, 0, R, gen.UNIFORM, gen.derive_seed(53, n, k)) for k in range(2)]
+    want = [v.sort().values for v in x]
+    a, out = torch.empty_like(x[0]), torch.empty_like(x[0])
+    torch.cuda.synchronize()
+    for k in (0, 1, 0, 1):
+        rtcdf.rtcdf_sort(a.data_ptr(), a.data_ptr(), n, 0, R, mine.cuda_stream)   # the kernel before
+        with torch.cuda.stream(other):
+            if not legacy:
+                other.wait_stream(mine)
+            torch.cuda._sleep(400_000)
+            a.copy_(x[k])
+        if not legacy:
+            mine.wait_stream(other)
+        assert rtcdf.rtcdf_sort(a.data_ptr(), out.data_ptr(), n, 0, R, mine.cuda_stream) == rtcdf.OK
+        torch.cuda.synchronize()
+        assert torch.equal(out, want[k])
+    rtcdf.rtcdf_status_get(mine.cuda_stream)         # (the first sort's input was never written)
+    assert cuda.cuStreamDestroy_v2(handle) == 0
